@@ -29,20 +29,24 @@
 //   gbar^s = (dD^s/dG^s) [s in the window] / n + P'(G^s)^T lambda^{s+1}
 //   lambda^s = C'(f^s)^T gbar^s  (identity at inlet and outlet nodes)
 //   dJ/dtheta = sum_s gbar^s . dC/dtheta + lambda^{s+1} . dP/dtheta
-// P^T is a gather: the entry G_i(x) is read by the regular pull of
-// x + c_i, by the bounce-back of x's own cut links and by the Bouzidi rule
-// of the fluid node x + c_i whose link along c_i is cut with q < 1/2; the
-// inlet and outlet rows add the adjoint of rho(1, y, z) and u(nx-2, y, z)
-// to the nodes they read (bc_adj_row).  C^T is the analytic vector-Jacobian
+// Cut links.  A pull of interior fluid node x along a cut link c_j would read
+// population i = opp(j) of the solid node (or wall ghost) x + c_j: a slot no
+// node owns.  Before each step one thread per cut link (k_chan_flinks) puts
+// the bounced-back population there, so the step itself is a plain pull of
+// 19 slots.  The reverse step gathers lambda_i at x + c_i, the transpose of
+// that pull; before it, one thread per cut link (k_chan_rlinks) applies the
+// transpose of the bounce-back to lambda^{s+1} in place (see k_chan_lists),
+// so the gather is as plain.  The geometry is fixed, so both lists are made
+// once.
+// C^T is the analytic vector-Jacobian
 // product of collide_node (chan_collide_vjp).  The forward run keeps f^s
 // every K steps; the reverse sweep recomputes each K-step segment from its
-// checkpoint, keeping its f^s, and runs the segment backwards, one launch
-// per step.  The boundary planes ride in extra blocks of the same launches:
-// the inlet / outlet equilibria of a forward step, and the inlet / outlet
-// adjoint that the next reverse step needs (it depends only on the step's
-// inputs, lambda^{s+1} and f^s).  Parameter gradients are summed per block
-// in FP64 into the block's own slots and added up once at the end of the
-// sweep.
+// checkpoint, keeping its f^s, and runs the segment backwards.  The planes
+// next to the inlet and outlet ride in edge blocks of the same launches,
+// which also do the inlet / outlet equilibria of a forward step and fold
+// their adjoint into lambda^s of a reverse step.  Parameter gradients are
+// summed per warp into the warp's own slots and added up once at the end of
+// the sweep.
 #include <cmath>
 #include <vector>
 
@@ -53,29 +57,20 @@ namespace {
 
 enum : uint8_t { CH_FLUID = 0, CH_SOLID = 1, CH_INLET = 2, CH_OUTLET = 3, CH_PLATE = 4 };
 
+// Populations G and adjoints lambda have one ghost plane below z = 0 and one
+// above z = nz - 1 (the slots of the wall links) and slot stride Ng; the
+// recorded states f^s are [Q][N].
 struct ChanGeo {
     int nx, ny, nz, N;
-    const uint8_t *type;    // [N]
-    const uint32_t *cutm;   // [N]: bit j set if the link x -> x + c_j is cut (q is read only then)
-    const float *q;         // [Q][N]: fraction of the cut link x -> x + c_j, -1 if not cut
+    int plane;              // nx ny
+    size_t Ng;              // nx ny (nz + 2)
+    const uint8_t *type;    // [N] node class
     const uint32_t *plate;  // [N]: bit j set if x -> x + c_j ends in the plate
-    // neighbour masks (static geometry): bit i set if x + c_i is in the box
-    // and is an interior fluid node (mfl), is an interior fluid node whose
-    // link along c_i is cut with q < 1/2 (mbq: the Bouzidi rule there reads
-    // x), or is any fluid class, inlet / outlet included (many)
-    const uint32_t *mfl, *mbq, *many;
 };
 
 __device__ __forceinline__ int wrapy(int y, int ny) { return y < 0 ? y + ny : (y >= ny ? y - ny : y); }
 
 __device__ __forceinline__ bool is_fluid_type(uint8_t t) { return t != CH_SOLID && t != CH_PLATE; }
-
-// Node index of (x, y, z) + c, or -1 outside the box in x or z.
-__device__ __forceinline__ int nbr(const ChanGeo &G, int x, int y, int z, int cxv, int cyv, int czv) {
-    const int xx = x + cxv, zz = z + czv;
-    if (xx < 0 || xx >= G.nx || zz < 0 || zz >= G.nz) return -1;
-    return xx + G.nx * (wrapy(y + cyv, G.ny) + G.ny * zz);
-}
 
 // ---- geometry ---------------------------------------------------------------
 
@@ -122,15 +117,17 @@ __global__ void k_chan_types(const int nx, const int ny, const int nz, const Pla
 }
 
 // Cut links of every fluid node (the branch q < 1/2 is decided in FP64 and
-// kept when q is rounded to FP32).
+// kept when q is rounded to FP32).  A link with q < 1/2 whose second point
+// x - c_j is not fluid takes the halfway rule f = G_j(x), which is the
+// q >= 1/2 rule at q = 1/2 exactly, so it is stored as q = 1/2.
 __global__ void k_chan_links(const int nx, const int ny, const int nz, const int np, const double *__restrict__ X,
                              const double *__restrict__ R, const uint8_t *__restrict__ type, float *__restrict__ qout,
-                             uint32_t *__restrict__ plate, uint32_t *__restrict__ cutm) {
+                             uint32_t *__restrict__ plate) {
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     const int N = nx * ny * nz;
     if (n >= N) return;
     const int x = n % nx, y = (n / nx) % ny, z = n / (nx * ny);
-    uint32_t pm = 0, cm = 0;
+    uint32_t pm = 0;
     qout[n] = -1.f;  // j = 0
     for (int j = 1; j < Q; ++j) {
         float qf = -1.f;
@@ -163,55 +160,105 @@ __global__ void k_chan_links(const int nx, const int ny, const int nz, const int
                     if (best < 0.0) best = 0.0;
                     qf = (float)best;
                     if (best < 0.5 && !(qf < 0.5f)) qf = 0.49999997f;  // keep the FP64 branch
+                    const int bx = x - rcx(j), bz = z - rcz(j);
+                    const bool second = bx >= 0 && bx < nx && bz >= 0 && bz < nz &&
+                                        is_fluid_type(type[bx + nx * (wrapy(y - rcy(j), ny) + ny * bz)]);
+                    if (!second && qf < 0.5f) qf = 0.5f;
                 }
             }
         }
         qout[(size_t)j * N + n] = qf;
-        if (qf >= 0.f) cm |= 1u << j;
     }
     plate[n] = pm;
-    cutm[n] = cm;
 }
 
-// Neighbour masks of every node (see ChanGeo).
-__global__ void k_chan_masks(const ChanGeo G, uint32_t *__restrict__ mfl, uint32_t *__restrict__ mbq,
-                             uint32_t *__restrict__ many) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= G.N) return;
-    const int x = n % G.nx, y = (n / G.nx) % G.ny, z = n / (G.nx * G.ny);
-    uint32_t a = 0u, b = 0u, c = 0u;
-    for (int i = 0; i < Q; ++i) {
-        const int tn = nbr(G, x, y, z, rcx(i), rcy(i), rcz(i));
-        if (tn < 0) continue;
-        const uint8_t t = G.type[tn];
-        if (t == CH_FLUID) {
-            a |= 1u << i;
-            if (((G.cutm[tn] >> i) & 1u) && G.q[(size_t)i * G.N + tn] < 0.5f) b |= 1u << i;
+// The cut links of the interior fluid nodes as lists, grouped by direction
+// (count[j] links along c_j; FILL places them from cursor[j] on; the order
+// within a direction does not matter, no two records of a list write the
+// same slot).  Slots are element indices i Ng + storage index.
+//
+// Forward record of link (x, j), i = opp(j): f_i(x) from G_j(x) and either
+// G_j(x2), x2 = x - c_j (q < 1/2), or G_i(x): (i0, i1, the slot of i at
+// x + c_j, q).
+//
+// Reverse record: with e = lambda_i(x) the transpose adds
+//   a e to gbar_j(x),    a = 2q (q < 1/2) or 1/(2q): through the slot of j at
+//                        x + c_j, which only x gathers;
+//   (1-2q) e to gbar_j(x2)           (q < 1/2): through the slot of j at x;
+//   (2q-1)/(2q) e to gbar_i(x)       (q > 1/2): through the slot of i at x2.
+// A slot is gathered by one node, and e is never one of the slots written
+// (x + c_j is not fluid), so the records are independent but for two cases,
+// which the record of the q > 1/2 link leaves to a special record (value
+// c0 lambda[s0] + c1 lambda[s1], added to the slot or assigned):
+//   x2 is not an interior fluid node: the slot of i at x2 carries nothing,
+//     or the a e of the link (x, i);
+//   the link (x2, i) is cut with q < 1/2 and adds to the same slot.
+struct ChanSpecial {
+    uint32_t dst, s0, s1;
+    float c0, c1;
+    int add;
+};
+constexpr uint32_t kNoSlot = 0xffffffffu;
+
+template <bool FILL>
+__global__ void k_chan_lists(const ChanGeo G, const float *__restrict__ q, uint32_t *__restrict__ cursor,
+                             uint4 *__restrict__ fl, uint4 *__restrict__ rl, ChanSpecial *__restrict__ sp) {
+    const int n = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    const bool in = n < G.N && G.type[n < G.N ? n : 0] == CH_FLUID;
+    const int x = n % G.nx, y = (n / G.nx) % G.ny, z = n / G.plane;
+    auto qof = [&](int j, int m) { return q[(size_t)j * G.N + m]; };
+    auto slot = [&](int i, int xx, int yy, int zz) {
+        return (uint32_t)((size_t)i * G.Ng + xx + (size_t)G.nx * (wrapy(yy, G.ny) + (size_t)G.ny * (zz + 1)));
+    };
+    for (int j = 1; j < Q; ++j) {
+        const float qj = in ? qof(j, n) : -1.f;
+        const unsigned bal = __ballot_sync(0xffffffffu, qj >= 0.f);
+        if (bal) {
+            uint32_t base = 0;
+            if (lane == 0) base = atomicAdd(cursor + j, (uint32_t)__popc(bal));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (qj >= 0.f) {
+                const int i = ropp(j), x2 = x - rcx(j), y2 = y - rcy(j), z2 = z - rcz(j);
+                const bool box2 = z2 >= 0 && z2 < G.nz;  // x2 in [0, nx): x is interior
+                const int n2 = box2 ? x2 + G.nx * (wrapy(y2, G.ny) + G.ny * z2) : -1;
+                const bool fluid2 = box2 && G.type[n2] == CH_FLUID;
+                const float qi = qof(i, n);               // the link (x, i)
+                const float q2 = fluid2 ? qof(i, n2) : -1.f;  // the link (x2, i)
+                const bool low = qj < 0.5f, high = qj > 0.5f;
+                // the slot (i, x2) of a high link is special (see above)
+                const bool special = high && (!fluid2 || (q2 >= 0.f && q2 < 0.5f));
+                if (special) {
+                    const uint32_t k = atomicAdd(cursor, 1u);
+                    if (FILL) {
+                        ChanSpecial r;
+                        r.dst = slot(i, x2, y2, z2);
+                        r.s1 = slot(i, x, y, z);
+                        r.c1 = __fdiv_rn(2.f * qj - 1.f, 2.f * qj);
+                        r.add = fluid2;
+                        r.s0 = fluid2 ? slot(j, x2, y2, z2) : slot(j, x, y, z);
+                        r.c0 = fluid2 ? 1.f - 2.f * q2
+                                      : (qi < 0.f ? 0.f : (qi < 0.5f ? 2.f * qi : __fdiv_rn(1.f, 2.f * qi)));
+                        sp[k] = r;
+                    }
+                }
+                if (FILL) {
+                    const uint32_t k = base + __popc(bal & ((1u << lane) - 1u));
+                    const uint32_t here = slot(j, x, y, z);
+                    const uint32_t second = low ? slot(j, x2, y2, z2) : (high ? slot(i, x, y, z) : here);
+                    fl[k] = make_uint4(here, second, slot(i, x + rcx(j), y + rcy(j), z + rcz(j)), __float_as_uint(qj));
+                    // x + c_j is not fluid: the link (x, i), if cut with q > 1/2, has a special record for this slot
+                    const uint32_t da = qi > 0.5f ? kNoSlot : slot(j, x + rcx(j), y + rcy(j), z + rcz(j));
+                    // the link (x2, i), if cut with q > 1/2, has a special record for the slot (j, x) of a low link
+                    const uint32_t du = low ? (q2 > 0.5f ? kNoSlot : here)
+                                            : (high && !special ? slot(i, x2, y2, z2) : kNoSlot);
+                    rl[k] = make_uint4(slot(i, x, y, z), da, du, __float_as_uint(qj));
+                }
+            }
         }
-        if (is_fluid_type(t)) c |= 1u << i;
     }
-    mfl[n] = a;
-    mbq[n] = b;
-    many[n] = c;
 }
 
 // ---- forward -----------------------------------------------------------------
-
-// Incoming population i at interior fluid node (x, y, z), index n, from G
-// (cut: whether any link of the node is cut).
-__device__ __forceinline__ float pull(const ChanGeo &G, const float *__restrict__ Gin, int x, int y, int z, int n,
-                                      int i, bool cut) {
-    const int j = ropp(i);
-    const float q = cut ? G.q[j * G.N + n] : -1.f;
-    if (q < 0.f) return Gin[i * G.N + nbr(G, x, y, z, -rcx(i), -rcy(i), -rcz(i))];
-    const float gj = Gin[j * G.N + n];
-    if (q < 0.5f) {
-        const int n2 = nbr(G, x, y, z, -rcx(j), -rcy(j), -rcz(j));
-        if (n2 >= 0 && is_fluid_type(G.type[n2])) return 2.f * q * gj + (1.f - 2.f * q) * Gin[j * G.N + n2];
-        return gj;
-    }
-    return gj / (2.f * q) + (2.f * q - 1.f) / (2.f * q) * Gin[i * G.N + n];
-}
 
 // Deviation of f^eq_i(rho, u) (Eq. 9) from w_i.
 __device__ __forceinline__ float feq_dev(int i, float rho, float ux, float uy, float uz) {
@@ -230,6 +277,28 @@ __device__ __forceinline__ void moments(const float *d, float &rho, float &jx, f
         jy += rcy(i) * d[i];
         jz += rcz(i) * d[i];
     }
+}
+
+// Unevaluated FP32 sum h + l of a running total: about 46 bits where the
+// FP64 pipe (1/64 of the FP32 rate) would cost the reverse step more than
+// its arithmetic.  ff_add: two-sum (Knuth) of the high parts, the errors
+// and low parts added, renormalised.
+struct FF {
+    float h, l;
+};
+__device__ __forceinline__ FF ff_add(const FF a, const FF b) {
+    const float s = __fadd_rn(a.h, b.h), bb = __fsub_rn(s, a.h);
+    const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, bb)), __fsub_rn(b.h, bb));
+    const float l = __fadd_rn(__fadd_rn(a.l, b.l), e);
+    const float h = __fadd_rn(s, l);
+    return {h, __fsub_rn(l, __fsub_rn(h, s))};
+}
+__device__ __forceinline__ FF ff_warp_sum(float v) {
+    FF a = {v, 0.f};
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        a = ff_add(a, FF{__shfl_xor_sync(0xffffffffu, a.h, o), __shfl_xor_sync(0xffffffffu, a.l, o)});
+    return a;
 }
 
 // Warp sums of three values added to the warp's own slots dst[0..2] (the
@@ -261,190 +330,185 @@ __device__ __forceinline__ void warp_add(double v, double *dst) {
 // nodes of one x row; grid (ceil(nx / kChanTx), ny, nz), so that (x, y, z)
 // come from the block and thread indices without integer division.
 constexpr int kChanTx = 128;
-// Resident blocks per SM of k_chan_adj: 10 (48 registers, a few hundred
-// bytes of spills to L1) waits out more of its latency than 8 at 64
-// registers without spills (reverse sweep 87.7 against 89.1 ms per gradient
-// of 500 steps; 12 blocks at 40 registers 88.2).
+// Resident blocks per SM of k_chan_step and k_chan_adj.  With the cut links
+// in kernels of their own both are straight code that waits on its 19 (38)
+// loads, and fewer blocks without spills win: 128x64x64 nodes, 200 spheres,
+// 500 steps, ms per gradient with step / adj at 12 / 10 blocks 71.3, 8 / 10
+// 63.1, 6 / 10 61.1, 12 / 6 62.0, 6 / 6 51.4, 7 / 7 52.0, 5 / 5 50.2 (the
+// links tested per direction inside the node kernels: 110.8; walked per
+// node: 79 at best).  Recorded states are written and read once, dozens of
+// steps apart: streaming stores and loads keep them from evicting G and
+// lambda (2 x 40 MB) from L2 (51.9 -> 51.4 ms).
 #ifndef LBM_CHAN_ADJ_MINB
-#define LBM_CHAN_ADJ_MINB 10
+#define LBM_CHAN_ADJ_MINB 5
 #endif
-// Resident blocks per SM of k_chan_step (the forward and the reverse
-// sweep's recompute): 12 at 40 registers, 110.6 ms per gradient against
-// 112.1 at 8 (64 registers) and 111.3 at 10; 16 (32 registers) spills
-// heavily and took 129 ms.
 #ifndef LBM_CHAN_STEP_MINB
-#define LBM_CHAN_STEP_MINB 12
+#define LBM_CHAN_STEP_MINB 6
 #endif
 
-// Row neighbours of (y, z): y periodic; z - 1 and z + 1 clamped into the
-// box (a pull from outside the box is replaced by the bounce-back of the cut
-// wall link, so the clamped value is never used).
-struct RowNb {
-    int ym, yp, zm, zp;
-    __device__ __forceinline__ RowNb(const ChanGeo &G, int y, int z) {
-        ym = y == 0 ? G.ny - 1 : y - 1;
-        yp = y == G.ny - 1 ? 0 : y + 1;
-        zm = z == 0 ? 0 : z - 1;
-        zp = z == G.nz - 1 ? z : z + 1;
+// A kernel of a channel run is a programmatic dependent of the one before
+// it on the stream: it may start once every block of that one has started,
+// reads the static geometry of its nodes, and touches populations, adjoints
+// and sums only after chan_wait (the completion of the kernel before).
+__device__ __forceinline__ void chan_wait() {
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// The node of a thread of the per-node kernels.  Blocks of the first
+// gridDim.z - nz slabs (`edge`, dispatched first) take the nodes next to the
+// inlet (x = 1) and to the outlet (x = nx - 2), one thread per (side, y, z);
+// the others one node each of the lattice.
+struct ChanNode {
+    int x, y, z, n;
+    int ym, yp;  // element offsets of y - 1 and y + 1 (periodic)
+    bool edge, in;
+    __device__ __forceinline__ explicit ChanNode(const ChanGeo &G) {
+        const int ex = (int)gridDim.z - G.nz;
+        edge = (int)blockIdx.z < ex;
+        if (edge) {
+            const int P = G.ny * G.nz;
+            const int k = ((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * kChanTx + threadIdx.x;
+            const int yz = k < P ? k : k - P;
+            in = k < 2 * P;
+            x = k < P ? 1 : G.nx - 2;
+            z = yz / G.ny;
+            y = yz - z * G.ny;
+        } else {
+            x = blockIdx.x * kChanTx + threadIdx.x;
+            y = blockIdx.y;
+            z = (int)blockIdx.z - ex;
+            in = x < G.nx;
+        }
+        n = x + G.nx * (y + G.ny * z);
+        ym = y == 0 ? G.nx * (G.ny - 1) : -G.nx;
+        yp = y == G.ny - 1 ? -G.nx * (G.ny - 1) : G.nx;
     }
-    // row index y' + ny z' of (y, z) + s (c_iy, c_iz), s = +1 or -1
-    __device__ __forceinline__ int row(const ChanGeo &G, int y, int z, int i, int s) const {
-        const int dy = s * rcy(i), dz = s * rcz(i);
-        const int yy = dy > 0 ? yp : (dy < 0 ? ym : y), zz = dz > 0 ? zp : (dz < 0 ? zm : z);
-        return yy + G.ny * zz;
-    }
-    // node index of (x, y, z) + s c_i (x + s c_ix must be in the box)
-    __device__ __forceinline__ int at(const ChanGeo &G, int x, int y, int z, int i, int s) const {
-        return x + s * rcx(i) + G.nx * row(G, y, z, i, s);
+    // element offset of x + s c_i (s = +1 or -1)
+    __device__ __forceinline__ int off(const ChanGeo &G, int i, int s) const {
+        const int dy = s * cy(i);
+        return s * cx(i) + (dy > 0 ? yp : (dy < 0 ? ym : 0)) + s * cz(i) * G.plane;
     }
 };
 
-// Inlet (x = 0) and outlet (x = nx - 1) planes of a pulled step, one thread
-// per (y, z, side), k in [0, 2 ny nz): the equilibrium of Eq. (9) from the
-// populations pulled at the neighbour plane; G = f there (not collided).
-__device__ __noinline__ void bc_step_body(const ChanGeo G, const Phys ph, const float u_peak,
-                                          const float *__restrict__ Gin, float *__restrict__ frec,
-                                          float *__restrict__ Gout, const int k) {
-    const int P = G.ny * G.nz;
-    const bool inlet = k < P;
-    const int yz = inlet ? k : k - P, y = yz % G.ny, z = yz / G.ny;
-    const int xs = inlet ? 1 : G.nx - 2, ns = xs + G.nx * yz, n = (inlet ? 0 : G.nx - 1) + G.nx * yz;
-    float e[Q], d[Q];
-    const bool cut = G.cutm[ns] != 0;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) e[i] = pull(G, Gin, xs, y, z, ns, i, cut);
-    float rho, jx, jy, jz;
-    moments(e, rho, jx, jy, jz);
-    if (inlet) {
-        const float zh = (z + 0.5f) / G.nz;
-        const float ux = u_peak * 4.f * zh * (1.f - zh);
-#pragma unroll
-        for (int i = 0; i < Q; ++i) d[i] = feq_dev(i, rho, ux, 0.f, 0.f);
-    } else {
-        const float ux = jx / rho + 0.5f * ph.g[0], uy = jy / rho + 0.5f * ph.g[1], uz = jz / rho + 0.5f * ph.g[2];
-#pragma unroll
-        for (int i = 0; i < Q; ++i) d[i] = feq_dev(i, 1.f, ux, uy, uz);
-    }
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        if (frec) frec[i * G.N + n] = d[i];
-        Gout[i * G.N + n] = d[i];
-    }
-}
-
-// Index of a thread of the blocks beyond the lattice (blockIdx.z >= nz: the
-// slabs of extra blocks that a launch carries for the boundary planes).
-__device__ __forceinline__ int extra_index(const ChanGeo &G) {
-    return (((blockIdx.z - G.nz) * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * kChanTx + threadIdx.x;
+// The bounced-back population of each cut link (Eq. 19), into the slot that
+// the node's pull reads: f_i(x) = 2q G_j(x) + (1-2q) G_j(x - c_j) for q < 1/2,
+// else G_j(x)/(2q) + (2q-1)/(2q) G_i(x), i = opp(j).
+constexpr int kLinkTx = 128;
+__global__ void __launch_bounds__(kLinkTx) k_chan_flinks(const uint4 *__restrict__ list, const int count,
+                                                         float *__restrict__ G) {
+    const int t = blockIdx.x * kLinkTx + threadIdx.x;
+    const uint4 r = t < count ? list[t] : make_uint4(0u, 0u, 0u, 0u);
+    chan_wait();
+    if (t >= count) return;
+    const float g0 = G[r.x], g1 = G[r.y], q = __uint_as_float(r.w), q2 = 2.f * q;
+    G[r.z] = q < 0.5f ? __fmaf_rn(q2, g0, __fmul_rn(__fsub_rn(1.f, q2), g1))
+                      : __fmaf_rn(__fdiv_rn(__fsub_rn(q2, 1.f), q2), g1, __fdiv_rn(g0, q2));
 }
 
 // One step at the interior fluid nodes (PULL: f^s pulled from G^{s-1}) or at
 // every fluid node (!PULL: f^s = fin, the stored state): record f^s in frec
 // (may be null), G^s = C(f^s) into Gout (G = f at inlet and outlet nodes),
-// plate drag of G^s added to *drag (may be null).  With PULL the inlet and
-// outlet planes are computed by the launch's extra blocks (blockIdx.z >= nz,
-// bc_step_body).  The pull reads x - c_i for every direction, then replaces
-// the populations of the node's cut links (bounce-back; Eq. 19 with q from
-// the geometry, walls and plate q = 1/2).
+// plate drag of G^s added to *drag (may be null).  With PULL the launch's
+// edge blocks (see ChanNode) pull at the planes next to the inlet and the
+// outlet as well and write the equilibria of Eq. (9) at the inlet (x = 0) and
+// outlet (x = nx - 1) nodes; G = f there.
 template <bool PULL>
 __global__ void __launch_bounds__(kChanTx, LBM_CHAN_STEP_MINB) k_chan_step(const ChanGeo G, const Phys ph, const float u_peak,
                                                        const float *__restrict__ Gin, const float *__restrict__ fin,
                                                        float *__restrict__ frec, float *__restrict__ Gout,
                                                        double *__restrict__ drag, int *__restrict__ status) {
-    if (PULL && (int)blockIdx.z >= G.nz) {  // the inlet and outlet planes (independent of the other blocks)
-        const int k = extra_index(G);
-        if (k < 2 * G.ny * G.nz) bc_step_body(G, ph, u_peak, Gin, frec, Gout, k);
-        return;
-    }
-    const int x = blockIdx.x * kChanTx + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
-    const int n = x + G.nx * (y + G.ny * z);
+    const ChanNode c(G);
+    const int n = c.n;
+    const uint8_t t = c.in ? G.type[n] : (uint8_t)CH_SOLID;
+    const bool live = PULL ? t == CH_FLUID : is_fluid_type(t);
+    const uint32_t pm = live && drag ? G.plate[n] : 0u;
+    chan_wait();
     double D = 0.0;
-    if (x < G.nx) {
-        const uint8_t t = G.type[n];
-        if (PULL ? t == CH_FLUID : is_fluid_type(t)) {
-            float d[Q];
-            if (!PULL) {
+    if (live) {
+        float d[Q];
+        if (!PULL) {
 #pragma unroll
-                for (int i = 0; i < Q; ++i) d[i] = fin[i * G.N + n];
+            for (int i = 0; i < Q; ++i) d[i] = fin[(size_t)i * G.N + n];
+        } else {
+#pragma unroll
+            for (int i = 0; i < Q; ++i) d[i] = Gin[i * G.Ng + (n + G.plane + c.off(G, i, -1))];
+        }
+        if (PULL && c.edge) {
+            float rho, jx, jy, jz;
+            moments(d, rho, jx, jy, jz);
+            if (c.x == 1) {
+                const float zh = (c.z + 0.5f) / G.nz;
+                const float ux = u_peak * 4.f * zh * (1.f - zh);
+#pragma unroll
+                for (int i = 0; i < Q; ++i) d[i] = feq_dev(i, rho, ux, 0.f, 0.f);
             } else {
-                const RowNb nb(G, y, z);
+                const float ux = jx / rho + 0.5f * ph.g[0], uy = jy / rho + 0.5f * ph.g[1], uz = jz / rho + 0.5f * ph.g[2];
 #pragma unroll
-                for (int i = 0; i < Q; ++i) d[i] = Gin[i * G.N + nb.at(G, x, y, z, i, -1)];
-                const uint32_t cm = G.cutm[n];
-                if (cm) {
-                    const uint32_t ma = G.many[n];
-#pragma unroll
-                    for (int i = 1; i < Q; ++i) {
-                        const int j = ropp(i);  // population i arrives from the cut link along c_j
-                        if ((cm >> j) & 1u) {
-                            const float q = G.q[j * G.N + n], gj = Gin[j * G.N + n];
-                            if (q < 0.5f) {
-                                // x - c_j = x + c_i: the second point of the rule, if it is fluid
-                                d[i] = ((ma >> i) & 1u)
-                                           ? 2.f * q * gj + (1.f - 2.f * q) * Gin[j * G.N + nb.at(G, x, y, z, i, 1)]
-                                           : gj;
-                            } else {
-                                d[i] = gj / (2.f * q) + (2.f * q - 1.f) / (2.f * q) * Gin[i * G.N + n];
-                            }
-                        }
-                    }
-                }
+                for (int i = 0; i < Q; ++i) d[i] = feq_dev(i, 1.f, ux, uy, uz);
             }
+            const int nb = c.x == 1 ? n - 1 : n + 1;  // the inlet or outlet node
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                if (frec) __stcs(frec + (size_t)i * G.N + nb, d[i]);
+                Gout[i * G.Ng + (nb + G.plane)] = d[i];
+            }
+        } else {
             if (frec)
 #pragma unroll
-                for (int i = 0; i < Q; ++i) frec[i * G.N + n] = d[i];
+                for (int i = 0; i < Q; ++i) __stcs(frec + (size_t)i * G.N + n, d[i]);
             if (t == CH_FLUID) collide_node(ph, d, status);
 #pragma unroll
-            for (int i = 0; i < Q; ++i) Gout[i * G.N + n] = d[i];
-            const uint32_t pm = G.plate[n];
-            if (pm)
+            for (int i = 0; i < Q; ++i) Gout[i * G.Ng + (n + G.plane)] = d[i];
+            if (pm && !c.edge)
 #pragma unroll
                 for (int j = 1; j < Q; ++j)
                     if (((pm >> j) & 1u) && rcx(j) != 0)
                         D += 2.0 * rcx(j) * ((double)d[j] + (double)rw36(j) / 36.0);
         }
     }
-    if (drag && __any_sync(0xffffffffu, D != 0.0)) warp_add(D, drag);
+    if (__any_sync(0xffffffffu, pm != 0u)) warp_add(D, drag);
 }
 
 // ---- reverse -----------------------------------------------------------------
 
-// Adjoint of the inlet and outlet rows of P at step s + 1 for one row
-// k = y + ny z, given lambda^{s+1} at the row's inlet node (li; bc_adj_inlet)
-// or outlet node (lo; bc_adj_outlet) and f^{s+1} (f1):  rho_bar(y, z) is
-// added to the adjoint of every population pulled at (1, y, z), ext[i](y, z)
-// to that of population i pulled at (nx-2, y, z); gu and gg are the row's
-// parts of dJ/du_peak and dJ/dg_x.
-__device__ __forceinline__ void bc_adj_inlet(const ChanGeo &G, const float u_peak, const float (&li)[Q],
-                                             const float *__restrict__ f1, const int k, float *__restrict__ rho_bar,
-                                             double &gu) {
-    const int z = k / G.ny, n1 = 1 + G.nx * k;
+// Adjoint of the inlet row of P at step s for the row of fluid node n = (1, y,
+// z), given lambda^s at the row's inlet node: that node's populations are
+// read by the pulls of the five directions c_x = 1 only (li; x = 1 holds
+// interior fluid nodes only).  Adds the adjoint of rho(1, y, z) to lambda^s
+// of every population at n (lam), so that the gathers of step s - 1 find it
+// there; returns the row's part of dJ/du_peak.
+__device__ __forceinline__ double fold_inlet(const ChanGeo &G, const float u_peak, const float (&li)[Q],
+                                             const float *__restrict__ f1, const int z, const int n,
+                                             float *__restrict__ lam) {
     // inlet: f_i(0) = rho_1 fe_i(1, u_in)
     const float zh = (z + 0.5f) / G.nz, sh = 4.f * zh * (1.f - zh), ux = u_peak * sh;
     float e[Q];
 #pragma unroll
-    for (int i = 0; i < Q; ++i) e[i] = f1[i * G.N + n1];
+    for (int i = 0; i < Q; ++i) e[i] = f1[(size_t)i * G.N + n];
     float rho1, jx, jy, jz;
     moments(e, rho1, jx, jy, jz);
     float rb = 0.f, ub = 0.f;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
+        if (cx(i) != 1) continue;
         const float w = (float)rw36(i) / 36.f, cu = rcx(i) * ux, l = li[i];
         rb += l * w * (1.f + 3.f * cu + 4.5f * cu * cu - 1.5f * ux * ux);
         ub += l * w * (3.f * rcx(i) + 9.f * cu * rcx(i) - 3.f * ux);
     }
-    rho_bar[k] = rb;
-    gu = (double)ub * rho1 * sh;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) lam[i * G.Ng] += rb;
+    return (double)ub * rho1 * sh;
 }
 
-__device__ __forceinline__ void bc_adj_outlet(const ChanGeo &G, const Phys &ph, const float (&lo)[Q],
-                                              const float *__restrict__ f1, const int k, float *__restrict__ ext,
-                                              double &gg) {
-    const int P = G.ny * G.nz, n2 = G.nx - 2 + G.nx * k;
+// The same for the outlet row of fluid node n = (nx - 2, y, z): the adjoint
+// of u(nx - 2, y, z), by population; returns the row's part of dJ/dg_x.
+__device__ __forceinline__ double fold_outlet(const ChanGeo &G, const Phys &ph, const float (&lo)[Q],
+                                              const float *__restrict__ f1, const int n, float *__restrict__ lam) {
     // outlet: f_i(nx-1) = f^eq_i(1, u(nx-2)), u = j / rho + g / 2
     float e[Q];
 #pragma unroll
-    for (int i = 0; i < Q; ++i) e[i] = f1[i * G.N + n2];
+    for (int i = 0; i < Q; ++i) e[i] = f1[(size_t)i * G.N + n];
     float rho2, jx, jy, jz;
     moments(e, rho2, jx, jy, jz);
     const float ir = 1.f / rho2;
@@ -452,6 +516,7 @@ __device__ __forceinline__ void bc_adj_outlet(const ChanGeo &G, const Phys &ph, 
     float uba[3] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
+        if (cx(i) != -1) continue;
         const float w = (float)rw36(i) / 36.f, l = lo[i];
         const float cu = rcx(i) * u[0] + rcy(i) * u[1] + rcz(i) * u[2];
         uba[0] += l * w * (3.f * rcx(i) + 9.f * cu * rcx(i) - 3.f * u[0]);
@@ -461,8 +526,8 @@ __device__ __forceinline__ void bc_adj_outlet(const ChanGeo &G, const Phys &ph, 
     const float v[3] = {jx * ir, jy * ir, jz * ir};
 #pragma unroll
     for (int i = 0; i < Q; ++i)
-        ext[i * P + k] = ir * (uba[0] * (rcx(i) - v[0]) + uba[1] * (rcy(i) - v[1]) + uba[2] * (rcz(i) - v[2]));
-    gg = 0.5 * (double)uba[0];
+        lam[i * G.Ng] += ir * (uba[0] * (rcx(i) - v[0]) + uba[1] * (rcy(i) - v[1]) + uba[2] * (rcz(i) - v[2]));
+    return 0.5 * (double)uba[0];
 }
 
 // Vector-Jacobian product of collide_node at deviations d: lam = C'(d)^T gb,
@@ -479,20 +544,19 @@ __device__ __forceinline__ void bc_adj_outlet(const ChanGeo &G, const Phys &ph, 
 // opposite pairs (i, i + 9) like the forward collision.  Divisions and
 // square roots use the hardware approximations (a few ulp): the adjoint
 // only has to carry the gradient to well within its 1e-3 tolerance.  The deviations are
-// read pair by pair from f (node n of [Q][N] arrays; null: the rest state)
-// and the result is written to lam (same layout), so that only gb is held
-// whole.
-__device__ __forceinline__ void chan_collide_vjp(const Phys &ph, const float *__restrict__ f, const int n,
-                                                 const int N, const float (&gb)[Q], float *__restrict__ lam,
+// read pair by pair from f (slot stride N; null: the rest state) and the
+// result is written to lam (slot stride Ng), so that only gb is held whole.
+__device__ __forceinline__ void chan_collide_vjp(const Phys &ph, const float *__restrict__ f, const size_t N,
+                                                 const float (&gb)[Q], float *__restrict__ lam, const size_t Ng,
                                                  float &gx_bar, float &smag_bar) {
     // forward intermediates (the moments of d, by opposite pairs)
-    const float d0 = f ? f[n] : 0.f;
+    const float d0 = f ? __ldcs(f) : 0.f;
     float drho = d0, j[3] = {0.f, 0.f, 0.f}, m[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // m: xx yy zz xy xz yz
     float N0 = wf(0) * gb[0], N1[3] = {0.f, 0.f, 0.f}, N2[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, gd = gb[0] * d0;
 #pragma unroll
     for (int i = 1; i <= 9; ++i) {
         const int k = i + 9;  // opp(i)
-        const float di = f ? f[i * N + n] : 0.f, dk = f ? f[k * N + n] : 0.f;
+        const float di = f ? __ldcs(f + i * N) : 0.f, dk = f ? __ldcs(f + k * N) : 0.f;
         const float sp = di + dk, dm = di - dk;
         const float gs = wf(i) * (gb[i] + gb[k]), gm = wf(i) * (gb[i] - gb[k]);
         drho += sp;
@@ -572,7 +636,7 @@ __device__ __forceinline__ void chan_collide_vjp(const Phys &ph, const float *__
     rho_bar -= ir_bar * ir * ir;
     const float dtot = drho_bar + rho_bar;  // rho = 1 + drho
     const float keep = 1.f - om;
-    lam[n] = keep * gb[0] + dtot;
+    lam[0] = keep * gb[0] + dtot;
 #pragma unroll
     for (int i = 1; i <= 9; ++i) {
         const int k = i + 9;
@@ -583,140 +647,106 @@ __device__ __forceinline__ void chan_collide_vjp(const Phys &ph, const float *__
         if (cx(i) * cy(i)) even += cx(i) * cy(i) * mb[3];
         if (cx(i) * cz(i)) even += cx(i) * cz(i) * mb[4];
         if (cy(i) * cz(i)) even += cy(i) * cz(i) * mb[5];
-        lam[i * N + n] = keep * gb[i] + even + odd;
-        lam[k * N + n] = keep * gb[k] + even - odd;
+        lam[i * Ng] = keep * gb[i] + even + odd;
+        lam[k * Ng] = keep * gb[k] + even - odd;
     }
 }
 
-// The inlet / outlet part of the adjoint of the population pulled as k at
-// interior fluid node t at x = xt (row yz): the inlet and outlet rows of P
-// read the pulls at x = 1 and x = nx - 2.
-__device__ __forceinline__ float edge_adj(const ChanGeo &G, const float *__restrict__ rho_bar,
-                                          const float *__restrict__ ext, int xt, int yz, int k) {
-    float v = 0.f;
-    if (xt == 1) v += rho_bar[yz];
-    if (xt == G.nx - 2) v += ext[k * (G.ny * G.nz) + yz];
-    return v;
-}
-
-// Adjoint of the population pulled as k at interior fluid node t (at x = xt,
-// row yz), with the inlet / outlet rows folded in.
-__device__ __forceinline__ float eff(const ChanGeo &G, const float *__restrict__ lam1, const float *__restrict__ rho_bar,
-                                     const float *__restrict__ ext, int t, int xt, int yz, int k) {
-    return lam1[k * G.N + t] + edge_adj(G, rho_bar, ext, xt, yz, k);
-}
-
-// The adjoint gb of G^s at fluid-class node (x, y, z), index n, that the
-// pulls of step s + 1 at the neighbours give: the regular pull of x + c_i
-// (an interior fluid node) and the Bouzidi rule of x + c_i whose link along
-// c_i is cut with q < 1/2 (it reads x).
-__device__ __forceinline__ void gather_adj(const ChanGeo &G, const float *__restrict__ lam1,
-                                           const float *__restrict__ rho_bar, const float *__restrict__ ext, int x,
-                                           int y, int z, int n, float (&gb)[Q]) {
-    const RowNb nb(G, y, z);
-    const uint32_t mf = G.mfl[n], mb = G.mbq[n];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        float v = 0.f;
-        if ((mf >> i) & 1u) {
-            const int xt = x + rcx(i), yzt = nb.row(G, y, z, i, 1), tn = xt + G.nx * yzt;
-            v = eff(G, lam1, rho_bar, ext, tn, xt, yzt, i);
-            if ((mb >> i) & 1u)
-                v += (1.f - 2.f * G.q[i * G.N + tn]) * eff(G, lam1, rho_bar, ext, tn, xt, yzt, ropp(i));
-        }
-        gb[i] = v;
+// Transpose of the bounce-back on lambda^{s+1}, in place (see k_chan_lists):
+// the list's links, then its special records.
+__global__ void __launch_bounds__(kLinkTx) k_chan_rlinks(const uint4 *__restrict__ list, const int count,
+                                                         const ChanSpecial *__restrict__ sp, const int nsp,
+                                                         float *__restrict__ lam) {
+    const int t = blockIdx.x * kLinkTx + threadIdx.x;
+    const uint4 r = t < count ? list[t] : make_uint4(0u, kNoSlot, kNoSlot, 0u);
+    chan_wait();
+    if (t < count) {
+        const float e = lam[r.x], q = __uint_as_float(r.w), q2 = 2.f * q;
+        const float u = r.z != kNoSlot ? lam[r.z] : 0.f;
+        const bool low = q < 0.5f;
+        if (r.y != kNoSlot) lam[r.y] = __fmul_rn(low ? q2 : __fdiv_rn(1.f, q2), e);
+        if (r.z != kNoSlot)
+            lam[r.z] = __fmaf_rn(low ? __fsub_rn(1.f, q2) : __fdiv_rn(__fsub_rn(q2, 1.f), q2), e, u);
+    } else if (t - count < nsp) {
+        const ChanSpecial c = sp[t - count];
+        const float v0 = lam[c.s0], v1 = lam[c.s1];
+        const float v = c.add ? __fmaf_rn(c.c0, v0, lam[c.dst]) : __fmul_rn(c.c0, v0);
+        lam[c.dst] = __fmaf_rn(c.c1, v1, v);
     }
-}
-
-// The inlet / outlet adjoint of step s - 1 for row k (k_chan_adj's extra
-// blocks): lambda^s at the row's inlet and outlet nodes is their gathered gb.
-// Not inlined, so that the node kernel's instruction stream stays short.
-__device__ __noinline__ void adj_extra_row(const ChanGeo G, const Phys ph, const float u_peak,
-                                           const float *__restrict__ lam1, const float *__restrict__ fs,
-                                           const float *__restrict__ rho_bar, const float *__restrict__ ext,
-                                           float *__restrict__ rho_nx, float *__restrict__ ext_nx, const int k,
-                                           double &gup, double &ggx) {
-    const int y = k % G.ny, z = k / G.ny;
-    float l[Q];
-    gather_adj(G, lam1, rho_bar, ext, 0, y, z, G.nx * k, l);
-    bc_adj_inlet(G, u_peak, l, fs, k, rho_nx, gup);
-    gather_adj(G, lam1, rho_bar, ext, G.nx - 1, y, z, G.nx - 1 + G.nx * k, l);
-    bc_adj_outlet(G, ph, l, fs, k, ext_nx, ggx);
 }
 
 // Reverse step s: lambda^s from lambda^{s+1} (lam1) and f^s (fs; null for
-// the rest state f^0 = w), weight wd of D^s in J (0 outside the window),
-// with the inlet / outlet adjoint of step s + 1 in rho_bar and ext.  The
-// parts of dJ/d(u_peak, g_x, smag) of each warp are added to its own slots
-// of gpart (3 per warp, summed over the steps; no atomics).  The launch's
-// extra blocks (blockIdx.z >= nz, present when rho_nx is not null) compute
-// the inlet / outlet adjoint of step s that the next reverse step reads
-// (rho_nx, ext_nx; from lambda^s at the inlet and outlet nodes, where it is
-// the gathered gb, and f^s), independently of the other blocks.
+// the rest state f^0 = w), weight wd of D^s in J (0 outside the window).  The
+// gather gbar_i(x) = lambda_i(x + c_i) is the whole transpose of the pull once
+// k_chan_rlinks has run on lambda^{s+1}; lambda is 0 in the slots of nodes
+// that are neither interior fluid nor the end of a cut link.  lambda^{s+1}
+// also carries the adjoint of its step's inlet and outlet rows at x = 1 and
+// x = nx - 2.  Those two planes are computed by the launch's edge blocks (see
+// ChanNode), which with `fold` also gather lambda^s at the row's inlet or
+// outlet node and fold its adjoint in for the next reverse step.  The parts
+// of dJ/d(u_peak, g_x, smag) of each warp are added to its own slots over the
+// steps (no atomics): FP64 triples of the edge warps in gedge, float-float
+// pairs (g_x, smag) of the others in gpart.
 __global__ void __launch_bounds__(kChanTx, LBM_CHAN_ADJ_MINB) k_chan_adj(
     const ChanGeo G, const Phys ph, const float u_peak, const float *__restrict__ lam1, const float *__restrict__ fs,
-    const float *__restrict__ rho_bar, const float *__restrict__ ext, const float wd, float *__restrict__ lam0,
-    float *__restrict__ rho_nx, float *__restrict__ ext_nx, double *__restrict__ gpart) {
-    double gup = 0.0, ggx = 0.0, gsm = 0.0;
-    if ((int)blockIdx.z >= G.nz) {
-        const int k = extra_index(G);  // row y + ny z
-        if (k < G.ny * G.nz) adj_extra_row(G, ph, u_peak, lam1, fs, rho_bar, ext, rho_nx, ext_nx, k, gup, ggx);
-    } else {
-        const int x = blockIdx.x * kChanTx + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
-        const int n = x + G.nx * (y + G.ny * z);
-        if (x < G.nx) {
-            const uint8_t t = G.type[n];
-            if (!is_fluid_type(t)) {
+    const float wd, float *__restrict__ lam0, const int fold, float4 *__restrict__ gpart, double *__restrict__ gedge) {
+    const ChanNode c(G);
+    // the planes x = 1 and x = nx - 2 belong to the edge blocks
+    const bool in = c.in && (c.edge || !(c.x == 1 || c.x == G.nx - 2));
+    const int n = c.n;
+    float gxb = 0.f, smb = 0.f;
+    double gup = 0.0, ggx = 0.0;
+    const bool live = in && G.type[n] == CH_FLUID;
+    const uint32_t pm = live && wd != 0.f ? G.plate[n] : 0u;
+    chan_wait();
+    if (live) {
+        float gb[Q];
+        const float *l1 = lam1 + (n + G.plane);
 #pragma unroll
-                for (int i = 0; i < Q; ++i) lam0[i * G.N + n] = 0.f;
-            } else {
-                float gb[Q];
-                gather_adj(G, lam1, rho_bar, ext, x, y, z, n, gb);
-                const int yz0 = y + G.ny * z;
-                // the node's own cut links (the adjoint of the populations it pulls itself)
-                const uint32_t cm = t == CH_FLUID ? G.cutm[n] : 0u;
-                if (cm) {
-                    const uint32_t ma = G.many[n];
+        for (int i = 0; i < Q; ++i) gb[i] = l1[(ptrdiff_t)(i * G.Ng) + c.off(G, i, 1)];
+        if (pm)
 #pragma unroll
-                    for (int i = 1; i < Q; ++i) {
-                        if ((cm >> i) & 1u) {  // link along c_i: population opp(i) reads G_i(x)
-                            const float qi = G.q[i * G.N + n];
-                            const float a = qi < 0.5f ? (((ma >> ropp(i)) & 1u) ? 2.f * qi : 1.f) : 1.f / (2.f * qi);
-                            gb[i] += a * eff(G, lam1, rho_bar, ext, n, x, yz0, ropp(i));
-                        }
-                        if ((cm >> ropp(i)) & 1u) {  // link along -c_i with q >= 1/2: population i reads G_i(x)
-                            const float qo = G.q[ropp(i) * G.N + n];
-                            if (qo >= 0.5f) gb[i] += (2.f * qo - 1.f) / (2.f * qo) * eff(G, lam1, rho_bar, ext, n, x, yz0, i);
-                        }
-                    }
-                }
-                const uint32_t pm = G.plate[n];
-                if (wd != 0.f && pm)
+            for (int i = 0; i < Q; ++i)
+                if ((pm >> i) & 1u) gb[i] += wd * 2.f * rcx(i);
+        float *l0 = lam0 + (n + G.plane);
+        chan_collide_vjp(ph, fs ? fs + n : nullptr, (size_t)G.N, gb, l0, G.Ng, gxb, smb);
+        if (c.edge && fold) {
+            const int side = c.x == 1 ? 1 : -1;  // c_x of the pulls that read the row's inlet or outlet node
 #pragma unroll
-                    for (int i = 0; i < Q; ++i)
-                        if ((pm >> i) & 1u) gb[i] += wd * 2.f * rcx(i);
-                if (t == CH_FLUID) {
-                    float gxb, smb;
-                    chan_collide_vjp(ph, fs, n, G.N, gb, lam0, gxb, smb);
-                    ggx = gxb;
-                    gsm = smb;
-                } else {
-#pragma unroll
-                    for (int i = 0; i < Q; ++i) lam0[i * G.N + n] = gb[i];
-                }
-            }
+            for (int i = 0; i < Q; ++i)
+                if (cx(i) == 1 && side == 1) gb[i] = l1[(ptrdiff_t)(i * G.Ng) + c.off(G, i, 1) - 1];
+                else if (cx(i) == -1 && side == -1) gb[i] = l1[(ptrdiff_t)(i * G.Ng) + c.off(G, i, 1) + 1];
+            if (side == 1) gup = fold_inlet(G, u_peak, gb, fs, c.z, n, l0);
+            else ggx = fold_outlet(G, ph, gb, fs, n, l0);
         }
     }
     const int warp = (blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)) * (kChanTx / 32) + (threadIdx.x >> 5);
-    warp_part(gup, ggx, gsm, gpart + 3 * warp);
+    if (c.edge) {
+        warp_part(gup, ggx + (double)gxb, (double)smb, gedge + 3 * warp);
+    } else {
+        const FF a = ff_warp_sum(gxb), b = ff_warp_sum(smb);
+        if ((threadIdx.x & 31) == 0) {
+            const float4 v = gpart[warp];
+            const FF x = ff_add(a, FF{v.x, v.y}), y = ff_add(b, FF{v.z, v.w});
+            gpart[warp] = make_float4(x.h, x.l, y.h, y.l);
+        }
+    }
 }
 
-// grad[0..2] += the sum of the nb warps' parts.
-__global__ void __launch_bounds__(256) k_chan_gsum(const double *__restrict__ gpart, int nb, double *__restrict__ grad) {
+// grad[0..2] += the sums of the warps' parts: ne FP64 triples of the edge
+// warps, nb float-float pairs (g_x, smag) from warp ne on.
+__global__ void __launch_bounds__(256) k_chan_gsum(const double *__restrict__ gedge, int ne,
+                                                   const float4 *__restrict__ gpart, int nb, double *__restrict__ grad) {
+    chan_wait();
     double a[3] = {0.0, 0.0, 0.0};
-    for (int k = threadIdx.x; k < nb; k += blockDim.x)
+    for (int k = threadIdx.x; k < ne; k += blockDim.x)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) a[c] += gpart[3 * k + c];
+        for (int c = 0; c < 3; ++c) a[c] += gedge[3 * k + c];
+    for (int k = ne + threadIdx.x; k < ne + nb; k += blockDim.x) {
+        const float4 v = gpart[k];
+        a[1] += (double)v.x + (double)v.y;
+        a[2] += (double)v.z + (double)v.w;
+    }
     __shared__ double sh[3][8];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -741,17 +771,17 @@ struct lbm_channel_s {
     lbm_channel_params p;
     int N = 0, np = 0, K = 0, nck = 0;
     uint8_t *type = nullptr;
-    uint32_t *cutm = nullptr;
-    float *q = nullptr;
     uint32_t *plate = nullptr;
-    uint32_t *mfl = nullptr, *mbq = nullptr, *many = nullptr;
-    double *gpart = nullptr;  // per-warp parts of dJ/d(u_peak, g_x, smag) (k_chan_adj)
+    uint4 *flist = nullptr, *rlist = nullptr;  // cut links of a forward / reverse step
+    ChanSpecial *special = nullptr;
+    int nlinks = 0, nspecial = 0;
+    float4 *gpart = nullptr;  // per-warp parts of dJ/d(g_x, smag), of the edge warps of dJ/d(u_peak, g_x, smag)
+    double *gedge = nullptr;  // (k_chan_adj)
     double *X = nullptr, *R = nullptr;
     float *G[2] = {nullptr, nullptr}, *lam[2] = {nullptr, nullptr};
     float *seg = nullptr;   // K states f^s of a segment
     float *ckpt = nullptr;  // f^s at s = 0, K, 2K, ...
     float *fend = nullptr;  // f^S of the last forward
-    float *rho_bar[2] = {nullptr, nullptr}, *ext[2] = {nullptr, nullptr};  // inlet / outlet adjoint, by step parity
     double *drag = nullptr, *grad = nullptr;
     int *status = nullptr;
     cudaStream_t stream = nullptr;
@@ -771,12 +801,9 @@ ChanGeo geo_of(const lbm_channel_s *c) {
     g.nz = c->p.nz;
     g.N = c->N;
     g.type = c->type;
-    g.cutm = c->cutm;
-    g.q = c->q;
+    g.plane = c->p.nx * c->p.ny;
+    g.Ng = (size_t)c->N + 2 * (size_t)g.plane;
     g.plate = c->plate;
-    g.mfl = c->mfl;
-    g.mbq = c->mbq;
-    g.many = c->many;
     return g;
 }
 
@@ -801,8 +828,8 @@ int calloc_dev(lbm_channel_s *c, T **p, size_t n) {
 }
 
 void chan_release(lbm_channel_s *c) {
-    void *ptrs[] = {c->type, c->cutm, c->q, c->plate, c->mfl, c->mbq, c->many, c->gpart, c->X, c->R, c->G[0], c->G[1], c->lam[0], c->lam[1], c->seg, c->ckpt,
-                    c->fend, c->rho_bar[0], c->rho_bar[1], c->ext[0], c->ext[1], c->drag, c->grad, c->status};
+    void *ptrs[] = {c->type, c->plate, c->flist, c->rlist, c->special, c->gpart, c->gedge, c->X, c->R, c->G[0], c->G[1], c->lam[0],
+                    c->lam[1], c->seg, c->ckpt, c->fend, c->drag, c->grad, c->status};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
@@ -827,15 +854,35 @@ int chan_check(lbm_channel_s *c, int rc) {
 
 int launch_ok() { return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA; }
 
-// Grid of the per-node kernels (see kChanTx) with extra slabs of blocks for
-// `extra` more threads (the boundary-plane work), and its block count.
-dim3 chan_grid(const lbm_channel_params &p, long long extra) {
-    const long long gx = (p.nx + kChanTx - 1) / kChanTx, per_slab = gx * p.ny * kChanTx;
-    return dim3((unsigned)gx, p.ny, p.nz + (unsigned)((extra + per_slab - 1) / per_slab));
+// Slabs of edge blocks that lead the grid of a per-node launch (see ChanNode),
+// their warps, and the grid.
+int chan_slabs(const lbm_channel_params &p) {
+    const long long per_slab = (long long)((p.nx + kChanTx - 1) / kChanTx) * p.ny * kChanTx, rows = 2ll * p.ny * p.nz;
+    return (int)((rows + per_slab - 1) / per_slab);
 }
-int chan_warps(const lbm_channel_params &p, long long extra) {
-    const dim3 g = chan_grid(p, extra);
-    return (int)(g.x * g.y * g.z) * (kChanTx / 32);
+dim3 chan_grid(const lbm_channel_params &p, int slabs) {
+    return dim3((unsigned)((p.nx + kChanTx - 1) / kChanTx), p.ny, p.nz + slabs);
+}
+int chan_warps(const lbm_channel_params &p, int slabs) {
+    return (int)((p.nx + kChanTx - 1) / kChanTx) * p.ny * slabs * (kChanTx / 32);
+}
+
+// Launch of a channel kernel as a programmatic dependent of the kernel
+// before it on the stream (see chan_wait).
+template <typename... P, typename... A>
+int chan_launch(lbm_channel_s *c, void (*k)(P...), const dim3 grid, const int threads, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.stream = c->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
 }
 
 // Forward from f^{s0} (fin) over steps s0 + 1 .. s1: f^s recorded into
@@ -844,17 +891,16 @@ int chan_warps(const lbm_channel_params &p, long long extra) {
 template <typename Rec>
 int chan_run(lbm_channel_s *c, const float *fin, int s0, int s1, Rec rec, bool with_drag) {
     const ChanGeo g = geo_of(c);
-    const dim3 grid = chan_grid(c->p, 0), grid_bc = chan_grid(c->p, 2ll * c->p.ny * c->p.nz);
+    const dim3 grid = chan_grid(c->p, 0), grid_edge = chan_grid(c->p, chan_slabs(c->p));
     const float up = (float)c->theta[0];
-    k_chan_step<false><<<grid, kChanTx, 0, c->stream>>>(g, c->ph, up, nullptr, fin, nullptr, c->G[s0 & 1],
-                                                      with_drag && s0 >= 1 ? c->drag + (s0 - 1) : nullptr, c->status);
-    int rc = launch_ok();
+    int rc = chan_launch(c, k_chan_step<false>, grid, kChanTx, g, c->ph, up, nullptr, fin, nullptr, c->G[s0 & 1],
+                         with_drag && s0 >= 1 ? c->drag + (s0 - 1) : nullptr, c->status);
     for (int s = s0 + 1; s <= s1 && !rc; ++s) {
-        float *fr = rec(s);
-        k_chan_step<true><<<grid_bc, kChanTx, 0, c->stream>>>(g, c->ph, up, c->G[(s - 1) & 1], nullptr, fr,
-                                                              c->G[s & 1], with_drag ? c->drag + (s - 1) : nullptr,
-                                                              c->status);
-        rc = launch_ok();
+        if (c->nlinks)
+            rc = chan_launch(c, k_chan_flinks, dim3((c->nlinks + kLinkTx - 1) / kLinkTx), kLinkTx, c->flist, c->nlinks,
+                             c->G[(s - 1) & 1]);
+        if (!rc) rc = chan_launch(c, k_chan_step<true>, grid_edge, kChanTx, g, c->ph, up, c->G[(s - 1) & 1], nullptr, rec(s),
+                         c->G[s & 1], with_drag ? c->drag + (s - 1) : nullptr, c->status);
     }
     return rc;
 }
@@ -907,28 +953,20 @@ int lbm_channel_create(const lbm_channel_params *prm, int32_t n, const double *p
             rc = LBM_ERR_CUDA;
         }
     }
-    const size_t NQs = (size_t)c->N * Q, P = (size_t)p.ny * p.nz;
+    const size_t NQs = (size_t)c->N * Q, NQg = NQs + 2 * (size_t)Q * p.nx * p.ny;
     if (!rc) rc = calloc_dev(c, &c->type, (size_t)c->N);
-    if (!rc) rc = calloc_dev(c, &c->cutm, (size_t)c->N);
-    if (!rc) rc = calloc_dev(c, &c->q, NQs);
     if (!rc) rc = calloc_dev(c, &c->plate, (size_t)c->N);
-    if (!rc) rc = calloc_dev(c, &c->mfl, (size_t)c->N);
-    if (!rc) rc = calloc_dev(c, &c->mbq, (size_t)c->N);
-    if (!rc) rc = calloc_dev(c, &c->gpart, 3 * (size_t)chan_warps(p, (long long)p.ny * p.nz));
-    if (!rc) rc = calloc_dev(c, &c->many, (size_t)c->N);
+    if (!rc) rc = calloc_dev(c, &c->gpart, (size_t)chan_warps(p, chan_slabs(p) + p.nz));
+    if (!rc) rc = calloc_dev(c, &c->gedge, 3 * (size_t)chan_warps(p, chan_slabs(p)));
     if (!rc) rc = calloc_dev(c, &c->X, 3 * (size_t)n);
     if (!rc) rc = calloc_dev(c, &c->R, (size_t)n);
     for (int k = 0; k < 2 && !rc; ++k) {
-        rc = calloc_dev(c, &c->G[k], NQs);
-        if (!rc) rc = calloc_dev(c, &c->lam[k], NQs);
+        rc = calloc_dev(c, &c->G[k], NQg);
+        if (!rc) rc = calloc_dev(c, &c->lam[k], NQg);
     }
     if (!rc) rc = calloc_dev(c, &c->seg, NQs * c->K);
     if (!rc) rc = calloc_dev(c, &c->ckpt, NQs * c->nck);
     if (!rc) rc = calloc_dev(c, &c->fend, NQs);
-    for (int k = 0; k < 2 && !rc; ++k) {
-        rc = calloc_dev(c, &c->rho_bar[k], P);
-        if (!rc) rc = calloc_dev(c, &c->ext[k], P * Q);
-    }
     if (!rc) rc = calloc_dev(c, &c->drag, (size_t)p.steps);
     if (!rc) rc = calloc_dev(c, &c->grad, 3);
     if (!rc) rc = calloc_dev(c, &c->status, 1);
@@ -945,14 +983,43 @@ int lbm_channel_create(const lbm_channel_params *prm, int32_t n, const double *p
         const int blocks = (c->N + 255) / 256;
         k_chan_types<<<blocks, 256, 0, c->stream>>>(p.nx, p.ny, p.nz, pb, n, c->X, c->R, c->type);
         rc = launch_ok();
-        if (!rc)
-            k_chan_links<<<blocks, 256, 0, c->stream>>>(p.nx, p.ny, p.nz, n, c->X, c->R, c->type, c->q, c->plate,
-                                                        c->cutm);
-        if (!rc) rc = launch_ok();
+        // link fractions (a temporary), counted and then placed in the lists
+        float *q = nullptr;
+        uint32_t *cursor = nullptr, cnt[Q] = {};
+        if (!rc && (cudaMalloc((void **)&q, sizeof(float) * NQs) != cudaSuccess ||
+                    cudaMalloc((void **)&cursor, sizeof(cnt)) != cudaSuccess)) {
+            cudaGetLastError();
+            rc = LBM_ERR_NOMEM;
+        }
+        auto ok = [](cudaError_t e) { return e == cudaSuccess ? LBM_OK : LBM_ERR_CUDA; };
+        const ChanGeo g = geo_of(c);
         if (!rc) {
-            k_chan_masks<<<blocks, 256, 0, c->stream>>>(geo_of(c), c->mfl, c->mbq, c->many);
+            k_chan_links<<<blocks, 256, 0, c->stream>>>(p.nx, p.ny, p.nz, n, c->X, c->R, c->type, q, c->plate);
             rc = launch_ok();
         }
+        if (!rc) rc = ok(cudaMemsetAsync(cursor, 0, sizeof(cnt), c->stream));
+        if (!rc) {
+            k_chan_lists<false><<<blocks, 256, 0, c->stream>>>(g, q, cursor, nullptr, nullptr, nullptr);
+            rc = launch_ok();
+        }
+        if (!rc) rc = ok(cudaMemcpyAsync(cnt, cursor, sizeof(cnt), cudaMemcpyDeviceToHost, c->stream));
+        if (!rc) rc = ok(cudaStreamSynchronize(c->stream));
+        if (!rc) {
+            c->nspecial = (int)cnt[0];
+            uint32_t at[Q] = {};
+            for (int j = 1; j < Q; ++j) at[j] = (uint32_t)c->nlinks, c->nlinks += (int)cnt[j];
+            rc = calloc_dev(c, &c->flist, (size_t)c->nlinks);
+            if (!rc) rc = calloc_dev(c, &c->rlist, (size_t)c->nlinks);
+            if (!rc) rc = calloc_dev(c, &c->special, (size_t)c->nspecial);
+            if (!rc) rc = ok(cudaMemcpyAsync(cursor, at, sizeof(at), cudaMemcpyHostToDevice, c->stream));
+            if (!rc) {
+                k_chan_lists<true><<<blocks, 256, 0, c->stream>>>(g, q, cursor, c->flist, c->rlist, c->special);
+                rc = launch_ok();
+            }
+            if (!rc) rc = ok(cudaStreamSynchronize(c->stream));
+        }
+        if (q) cudaFree(q);
+        if (cursor) cudaFree(cursor);
     }
     rc = chan_check(c, rc);
     if (rc) {
@@ -1016,21 +1083,20 @@ int lbm_channel_backward(lbm_channel c, double *grad) {
     if (!c || !grad) return LBM_ERR_ARG;
     if (!c->have_forward) return LBM_ERR_ARG;  // the checkpoints belong to another theta
     DeviceScope ds(c->p.device);
-    const size_t NQs = (size_t)c->N * Q, P = (size_t)c->p.ny * c->p.nz;
+    const size_t NQs = (size_t)c->N * Q;
     const int S = c->p.steps, K = c->K;
-    const dim3 grid = chan_grid(c->p, 0), grid_bc = chan_grid(c->p, (long long)P);
-    const int nwarps = chan_warps(c->p, (long long)P);
+    const int slabs = chan_slabs(c->p);
+    const dim3 grid_edge = chan_grid(c->p, slabs);
+    const int nedge = chan_warps(c->p, slabs), nwarps = chan_warps(c->p, c->p.nz);
     const ChanGeo g = geo_of(c);
     const float up = (float)c->theta[0];
     const float wd = (float)(1.0 / (S - c->p.avg_from + 1));
     int rc = cudaMemsetAsync(c->grad, 0, 3 * sizeof(double), c->stream) == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
-    if (!rc && cudaMemsetAsync(c->gpart, 0, 3 * sizeof(double) * nwarps, c->stream) != cudaSuccess)
+    if (!rc && (cudaMemsetAsync(c->gpart, 0, sizeof(float4) * (size_t)(nedge + nwarps), c->stream) != cudaSuccess ||
+                cudaMemsetAsync(c->gedge, 0, 3 * sizeof(double) * (size_t)nedge, c->stream) != cudaSuccess))
         rc = LBM_ERR_CUDA;
-    if (!rc && cudaMemsetAsync(c->lam[(S + 1) & 1], 0, sizeof(float) * NQs, c->stream) != cudaSuccess)
-        rc = LBM_ERR_CUDA;  // lambda^{S+1} = 0
-    // lambda^{S+1} = 0: no inlet / outlet adjoint enters reverse step S
-    if (!rc && (cudaMemsetAsync(c->rho_bar[S & 1], 0, sizeof(float) * P, c->stream) != cudaSuccess ||
-                cudaMemsetAsync(c->ext[S & 1], 0, sizeof(float) * P * Q, c->stream) != cudaSuccess))
+    // lambda^{S+1} = 0, with no inlet / outlet adjoint
+    if (!rc && cudaMemsetAsync(c->lam[(S + 1) & 1], 0, sizeof(float) * g.Ng * Q, c->stream) != cudaSuccess)
         rc = LBM_ERR_CUDA;
     for (int seg = S / K; seg >= 0 && !rc; --seg) {
         const int s0 = seg * K, s1 = std::min(s0 + K - 1, S);  // reverse steps s1 .. s0
@@ -1041,19 +1107,16 @@ int lbm_channel_backward(lbm_channel c, double *grad) {
         for (int s = s1; s >= s0 && !rc; --s) {
             const float *fs = s == s0 ? f0 : c->seg + NQs * (size_t)(s - s0 - 1);
             const float w = (s >= c->p.avg_from && s >= 1) ? wd : 0.f;
-            // the extra blocks of reverse step s > 0 prepare the inlet / outlet adjoint of step s - 1
-            const bool nxt = s > 0;
-            k_chan_adj<<<nxt ? grid_bc : grid, kChanTx, 0, c->stream>>>(
-                g, c->ph, up, c->lam[(s + 1) & 1], s == 0 ? nullptr : fs, c->rho_bar[s & 1], c->ext[s & 1], w,
-                c->lam[s & 1], nxt ? c->rho_bar[(s - 1) & 1] : nullptr, nxt ? c->ext[(s - 1) & 1] : nullptr,
-                c->gpart);
-            rc = launch_ok();
+            // the edge blocks of reverse step s > 0 fold in the inlet / outlet adjoint that step s - 1 reads
+            if (s < S && c->nlinks)
+                rc = chan_launch(c, k_chan_rlinks, dim3((c->nlinks + c->nspecial + kLinkTx - 1) / kLinkTx), kLinkTx,
+                                 c->rlist, c->nlinks, c->special, c->nspecial, c->lam[(s + 1) & 1]);
+            if (!rc)
+                rc = chan_launch(c, k_chan_adj, grid_edge, kChanTx, g, c->ph, up, c->lam[(s + 1) & 1], s == 0 ? nullptr : fs,
+                             w, c->lam[s & 1], s > 0 ? 1 : 0, c->gpart, c->gedge);
         }
     }
-    if (!rc) {
-        k_chan_gsum<<<1, 256, 0, c->stream>>>(c->gpart, nwarps, c->grad);
-        rc = launch_ok();
-    }
+    if (!rc) rc = chan_launch(c, k_chan_gsum, dim3(1), 256, c->gedge, nedge, c->gpart, nwarps, c->grad);
     double gr[3] = {0.0, 0.0, 0.0};
     if (!rc && cudaMemcpyAsync(gr, c->grad, sizeof(gr), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess)
         rc = LBM_ERR_CUDA;
