@@ -312,14 +312,13 @@ int lbm_create(const lbm_params *prm, lbm_handle *out) {
         pt.ulo[a] = (float)p.wall_vel_lo[a];
         pt.uhi[a] = (float)p.wall_vel_hi[a];
     }
-    // a solid node lies within [-ceil(R) + 1, ceil(R)] of floor(X) per axis; the
-    // link tile also holds x = s - c_j and x - c_j, two more nodes out
-    h->tile_ext = (int)std::ceil(M > 0 ? p.max_radius : 1.0) + 2;
+    // half width of the node box of the largest sphere (see LinkTile)
+    h->tile_ext = (int)std::ceil(M > 0 ? p.max_radius : 1.0);
     h->link_cap = link_capacity(M > 0 ? p.max_radius : 1.0);
 
     unsigned char *fixed = nullptr;
     if (!rc) rc = dalloc(h, (unsigned char **)&h->f, (size_t)Q * h->L.S * h->esize);
-    if (!rc) rc = dalloc(h, &h->flag, (size_t)N);
+    if (!rc) rc = dalloc(h, &h->flag, (size_t)N + 16);  // the link kernel reads whole words
     if (!rc) rc = dalloc(h, &h->owner, (size_t)N);
     if (!rc) rc = dalloc(h, &h->status, 1);
     if (!rc) rc = dalloc(h, &h->bar, 1);

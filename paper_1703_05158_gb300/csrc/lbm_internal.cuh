@@ -282,7 +282,7 @@ struct lbm_s {
     double *load_stage[2] = {nullptr, nullptr};
     cudaEvent_t load_ev[2] = {nullptr, nullptr};
     int load_slot = 0;
-    int tile_ext;            // half width of the per-sphere link tile
+    int tile_ext;            // ceil of the largest radius: sizes the per-sphere link tile (LinkTile)
     int link_cap;            // link-list capacity per sphere (shared memory)
     size_t bytes;
     // overlap of the next step's far-node collisions with the link / DEM /

@@ -8,17 +8,21 @@ namespace lbm {
 
 // GI: compiled with the Galilean-invariant momentum exchange (taken where
 // the handle asks for it).
-// The link kernel waits on scattered DRAM accesses: five resident CTAs per
-// SM (48 registers, a few bytes of spills) with two links per thread in
-// flight keep more of them outstanding than four CTAs at 64 registers with
-// three (0.114 against 0.117 ms per launch on 2000 spheres; six CTAs at 40
-// registers spill more and lose).  A thread's links, and so the sums, are
-// in the same order for any batch.
+// Bound by scattered DRAM blocks on thousands of spheres, by latency on a
+// few.  64 registers (4 CTAs per SM, no spills) with three links per thread
+// in flight, link phase in us on 256^3 with 2000 spheres / with 8136 /
+// 512x256x256 with 7911 (FP16): 106.2 / 368 / 466; two links 108.9 / 377 /
+// 476, five 107.4 / 373 / 473; 5 CTAs at 48 registers (spills) 118.7 / 416 /
+// 499 with two and 112.0 / 402 / 514 with one, 6 CTAs 117 / 405 / 504.  With
+// node codes per byte, links found per node and direction and three integer
+// divisions per link, the same took 110.7 / 374 / 467 and 18.3 instead of
+// 15.4 on 64^3 with 31 spheres (the step 60.1 -> 48.4 us there).  A thread's
+// links, and so the sums, are in the same order for any batch.
 #ifndef LBM_LINK_MINB
-#define LBM_LINK_MINB 5  // resident CTAs per SM the register budget is set for
+#define LBM_LINK_MINB 4  // resident CTAs per SM the register budget is set for
 #endif
 #ifndef LBM_LINK_BATCH
-#define LBM_LINK_BATCH 2  // links per thread whose populations are loaded together
+#define LBM_LINK_BATCH 3  // links per thread whose populations are loaded together
 #endif
 
 template <typename T, bool GI>
@@ -31,16 +35,13 @@ __global__ void __launch_bounds__(256, LBM_LINK_MINB) k_links(const Lat L, const
 }
 
 // Batched: instance blockIdx.y; parity P is also the step parity.
-// The batched form (its instance read through a pointer takes more
-// registers): 4 CTAs per SM at 64 registers with two links in flight took
-// the 64-member sweep from 3.846 to 3.407 ms per step against 3 CTAs at 80
-// registers with six (3.482 with three links at 4 CTAs, 3.435 at 5 CTAs
-// and 48 registers, which spill 136 bytes).
+// 64 sweep members, us per step: 2533 at 4 CTAs per SM with three links in
+// flight, 2564 with two, 2587 at 3 CTAs with four.
 #ifndef LBM_LINK_B_MINB
 #define LBM_LINK_B_MINB 4
 #endif
 #ifndef LBM_LINK_B_BATCH
-#define LBM_LINK_B_BATCH 2
+#define LBM_LINK_B_BATCH 3
 #endif
 template <typename T, bool GI>
 __global__ void __launch_bounds__(256, LBM_LINK_B_MINB) k_links_b(const Inst *__restrict__ I, const int P,
@@ -57,8 +58,8 @@ int link_capacity(double max_radius) {
 }
 
 size_t link_smem(int ext, int cap) {
-    const size_t B = 2 * (size_t)ext + 1, B3 = B * B * B;
-    return 4 * (size_t)cap + ((B3 + 15) & ~(size_t)15) + 2 * ((B3 + 1) / 2);
+    const LinkTile tl(ext);
+    return 8 * (size_t)tl.B * tl.B + 4 * ((size_t)cap + tl.ncap(cap));
 }
 
 // Raise (never lower: other handles may need more) a kernel's dynamic
