@@ -56,7 +56,8 @@ void release(lbm_s *h) {
                     (void *)h->pt.fixed, h->pt.Fh, h->pt.Th, h->pt.Fc, h->pt.Fx, h->pt.Tx, h->pt.Xf,
                     h->pt.Xb[0], h->pt.Xb[1], h->pt.Vh[0], h->pt.Vh[1], h->pt.nbr, h->pt.nbr_cnt, h->pt.pairA,
                     h->pt.pairB, h->pt.Xbuild, h->pt.rebuild, h->pt.frame[0], h->pt.frame[1], h->pt.Fcorr,
-                    h->pt.Tcorr, h->pt.Tc, h->pt.pairC, h->pt.tdisp, h->pt.tmask, h->pt.twall, h->zs, h->pt.pairBM, h->pt.nact,
+                    h->pt.Tcorr, h->pt.Tc, h->pt.pairC, h->pt.tdisp, h->pt.tmask, h->pt.twall, h->zs, h->pt.pairBM, h->pt.nact, h->pt.isl_n, h->pt.isl8,
+                    h->pt.isl32, h->pt.big, h->pt.slot, h->pt.inv,
                     h->xbuf,
                     h->zpart, h->zcnt};
     for (void *p : ptrs)
@@ -329,6 +330,7 @@ int lbm_create(const lbm_params *prm, lbm_handle *out) {
     if (!rc) rc = dalloc(h, &pt.R, (size_t)M);
     if (!rc) rc = dalloc(h, &fixed, (size_t)M);
     pt.fixed = fixed;
+    if (!rc) rc = dalloc(h, &pt.inv, 2 * (size_t)M);
     if (!rc) rc = dalloc(h, &pt.Fh, 3 * (size_t)M);
     if (!rc) rc = dalloc(h, &pt.Th, 3 * (size_t)M);
     if (!rc) rc = dalloc(h, &pt.Fc, 3 * (size_t)M);
@@ -364,6 +366,12 @@ int lbm_create(const lbm_params *prm, lbm_handle *out) {
     if (!rc) rc = dalloc(h, &pt.pairBM, (size_t)M * kMaxNbr);
     if (!rc) rc = dalloc(h, &h->xbuf, 2 * 3 * (size_t)M);
     if (!rc) rc = dalloc(h, &pt.nact, (size_t)M);
+    // islands: at most M / 2 in groups of 8, M / 9 in warps
+    if (!rc) rc = dalloc(h, &pt.isl_n, 4);
+    if (!rc) rc = dalloc(h, &pt.isl8, 4 * (size_t)M + 32);
+    if (!rc) rc = dalloc(h, &pt.isl32, 4 * (size_t)M + 32);
+    if (!rc) rc = dalloc(h, &pt.big, (size_t)M);
+    if (!rc) rc = dalloc(h, &pt.slot, (size_t)M);
     if (!rc) rc = dalloc(h, &pt.Xf, (size_t)M);
     for (int b = 0; b < 2 && !rc; ++b) {
         rc = dalloc(h, &pt.Xb[b], 3 * (size_t)M);
@@ -433,6 +441,7 @@ int lbm_create(const lbm_params *prm, lbm_handle *out) {
     if (!rc) {
         *h->status_host = 0;
         bool ok = cudaMemsetAsync(h->f, 0, (size_t)Q * h->L.S * h->esize, h->stream) == cudaSuccess &&
+                  (!M || cudaMemsetAsync(pt.slot, 0, sizeof(int) * (size_t)M, h->stream) == cudaSuccess) &&
                   cudaMemsetAsync(h->flag, 0, (size_t)N, h->stream) == cudaSuccess &&
                   cudaMemsetAsync(h->owner, 0xff, (size_t)N * 4, h->stream) == cudaSuccess &&
                   cudaMemsetAsync(h->status, 0, sizeof(int), h->stream) == cudaSuccess &&

@@ -19,13 +19,16 @@
 // forces are summed in FP32 per sub-step; the spin is advanced once per step
 // (the torque is constant over it).
 //
-// Sub-steps need every sphere's displacement of the previous sub-step.  One
-// thread-block cluster runs all of them: each thread keeps its spheres in
-// registers, publishes (dx, dv) in its CTA's shared memory (double-buffered by
-// sub-step parity) and reads neighbours' through distributed shared memory;
-// a hardware cluster barrier (release / acquire) separates drift and force.
-// More spheres than one cluster holds fall back to a cooperative launch with
-// a bounded software grid barrier.
+// A sub-step needs the displacements of a sphere's contact candidates (the
+// listed pairs that can touch within the step) after the previous one, and of
+// no other sphere.  So the step is split by the components of the candidate
+// graph (k_islands): a sphere without candidates runs all its sub-steps in
+// its own thread, a component of up to 32 spheres in one warp that exchanges
+// (dx, dv) through shared memory, and only larger components need a barrier
+// across CTAs per sub-step: a thread-block cluster (distributed shared memory,
+// hardware barrier) or, for more spheres than one cluster holds well, a
+// cooperative grid (an L2-resident buffer, a bounded software barrier).  The
+// arithmetic of a sphere is the same code in each of them.
 //
 // Tangential contact law (Eqs. 2, 3; on when k_t > 0 and mu > 0, the
 // template argument FRIC of the cluster kernel): the readings of the oracle
@@ -46,6 +49,7 @@
 // error is raised) keeps every pair that can touch within a step in the list.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "lbm_internal.cuh"
@@ -97,6 +101,7 @@ __device__ __forceinline__ void neighbours_body(const Lat &L, const Parts &pt, c
     const int a = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31, wid = (threadIdx.x >> 5) & 7;
     const bool live = a < pt.np;
+    if (blockIdx.x == 0 && threadIdx.x < 3) pt.isl_n[threadIdx.x] = 0;  // for the islands of this step
     const bool rebuild = force || *(volatile int *)(pt.rebuild + sp) != 0;
     if (rebuild) {
         int ocnt = 0;
@@ -112,7 +117,6 @@ __device__ __forceinline__ void neighbours_body(const Lat &L, const Parts &pt, c
             __syncwarp();
         }
         float4 me = live ? pt.Xf[a] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float ra = me.w + (float)pt.skin;
         const float hx = 0.5f * L.nx, hy = 0.5f * L.ny;
         int cnt = 0;
         for (int t0 = 0; t0 < pt.np; t0 += kNbrTile) {
@@ -132,7 +136,7 @@ __device__ __forceinline__ void neighbours_body(const Lat &L, const Parts &pt, c
                     if (dx < -hx) dx += L.nx;
                     if (dy > hy) dy -= L.ny;
                     if (dy < -hy) dy += L.ny;
-                    const float cut = ra + o.w;
+                    const float cut = (me.w + o.w) + (float)pt.skin;  // symmetric: b lists a when a lists b
                     ok = dx * dx + dy * dy + dz * dz < cut * cut;
                 }
                 const unsigned m = __ballot_sync(0xffffffffu, ok);
@@ -309,6 +313,9 @@ __device__ void contact_force(const Lat &L, const Parts &pt, int a, const double
 __global__ void k_contact(const Lat L, const Parts pt) {
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= pt.np) return;
+    const double m = sphere_mass(pt, a), R = pt.R[a];
+    pt.inv[2 * a] = 1.0 / m;  // an FP64 divide costs a sub-step; the masses do not change
+    pt.inv[2 * a + 1] = 1.0 / (0.4 * m * R * R);
     double F[3], T[3] = {0.0, 0.0, 0.0};
     contact_force(L, pt, a, pt.X + 3 * a, pt.V + 3 * a, pt.X, pt.V, F, pt.W + 3 * a, pt.W, T);
     for (int c = 0; c < 3; ++c) {
@@ -408,26 +415,48 @@ __device__ bool grid_barrier(unsigned *bar, unsigned target, int *status) {
     return ok != 0;
 }
 
+// The sub-step arithmetic is written with explicit round-to-nearest
+// operations: the compiler may contract a sum of products either way round,
+// and a sphere has to get the same bits in a warp, a cluster, a grid or a
+// batch.
+__device__ __forceinline__ float dot3(const float3 a, const float3 b) {
+    return __fmaf_rn(a.z, b.z, __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)));
+}
+__device__ __forceinline__ float3 sub3(const float3 a, const float3 b) {
+    return make_float3(__fsub_rn(a.x, b.x), __fsub_rn(a.y, b.y), __fsub_rn(a.z, b.z));
+}
+__device__ __forceinline__ float3 add3(const float3 a, const float3 b) {
+    return make_float3(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y), __fadd_rn(a.z, b.z));
+}
+__device__ __forceinline__ float3 mul3(const float s, const float3 a) {
+    return make_float3(__fmul_rn(s, a.x), __fmul_rn(s, a.y), __fmul_rn(s, a.z));
+}
+// s a + b
+__device__ __forceinline__ float3 fma3(const float s, const float3 a, const float3 b) {
+    return make_float3(__fmaf_rn(s, a.x, b.x), __fmaf_rn(s, a.y, b.y), __fmaf_rn(s, a.z, b.z));
+}
+__device__ __forceinline__ float3 cross3(const float3 a, const float3 b) {
+    return make_float3(__fmaf_rn(a.y, b.z, -__fmul_rn(a.z, b.y)), __fmaf_rn(a.z, b.x, -__fmul_rn(a.x, b.z)),
+                       __fmaf_rn(a.x, b.y, -__fmul_rn(a.y, b.x)));
+}
+__device__ __forceinline__ float3 xyz(const float4 v) { return make_float3(v.x, v.y, v.z); }
+
 // FP32 tangential force of a contact (Eqs. 2, 3) with displacement d (in /
 // out): d turned into the plane normal to n and advanced by v_t h; the trial
 // force -k_t d - gamma_t v_t, capped at mu max(f^n, 0) along -v_t (along the
 // trial force if v_t = 0) with d reset to -f_t / k_t.
 __device__ __forceinline__ float3 tangential_force(float3 &d, const float3 n, const float3 vt, const float fn,
                                                    const float gt, const float kt, const float mu, const float h) {
-    const float dn = d.x * n.x + d.y * n.y + d.z * n.z;
-    d.x += vt.x * h - dn * n.x;
-    d.y += vt.y * h - dn * n.y;
-    d.z += vt.z * h - dn * n.z;
-    float3 f = make_float3(-kt * d.x - gt * vt.x, -kt * d.y - gt * vt.y, -kt * d.z - gt * vt.z);
-    const float t2 = f.x * f.x + f.y * f.y + f.z * f.z;
-    const float cap = mu * fmaxf(fn, 0.f);
-    if (t2 > cap * cap) {
-        const float v2 = vt.x * vt.x + vt.y * vt.y + vt.z * vt.z;
-        const float s = v2 > 0.f ? -cap * rsqrtf(v2) : cap * rsqrtf(t2);
-        const float3 u = v2 > 0.f ? vt : f;
-        f = make_float3(s * u.x, s * u.y, s * u.z);
-        const float ik = -1.f / kt;
-        d = make_float3(f.x * ik, f.y * ik, f.z * ik);
+    const float dn = dot3(d, n);
+    d = add3(d, fma3(h, vt, mul3(-dn, n)));
+    float3 f = fma3(-gt, vt, mul3(-kt, d));
+    const float t2 = dot3(f, f);
+    const float cap = __fmul_rn(mu, fmaxf(fn, 0.f));
+    if (t2 > __fmul_rn(cap, cap)) {
+        const float v2 = dot3(vt, vt);
+        const float s = v2 > 0.f ? __fmul_rn(-cap, rsqrtf(v2)) : __fmul_rn(cap, rsqrtf(t2));
+        f = mul3(s, v2 > 0.f ? vt : f);
+        d = mul3(__fdiv_rn(-1.f, kt), f);
     }
     return f;
 }
@@ -437,281 +466,359 @@ __device__ __forceinline__ float3 tangential_force(float3 &d, const float3 n, co
 __device__ __forceinline__ void friction_add(float3 &F, float3 &T, float3 &d, const float3 n, const float3 vr,
                                              const float l, const float fn, const float gt, const float kt,
                                              const float mu, const float h) {
-    const float vrn = vr.x * n.x + vr.y * n.y + vr.z * n.z;
-    const float3 vt = make_float3(vr.x - vrn * n.x, vr.y - vrn * n.y, vr.z - vrn * n.z);
+    const float3 vt = fma3(-dot3(vr, n), n, vr);
     const float3 f = tangential_force(d, n, vt, fn, gt, kt, mu, h);
-    F.x += f.x;
-    F.y += f.y;
-    F.z += f.z;
-    T.x -= l * (n.y * f.z - n.z * f.y);
-    T.y -= l * (n.z * f.x - n.x * f.z);
-    T.z -= l * (n.x * f.y - n.y * f.x);
+    F = add3(F, f);
+    T = fma3(-l, cross3(n, f), T);
 }
 
-__device__ __forceinline__ float3 cross3(const float3 a, const float3 b) {
-    return make_float3(a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x);
+// Islands of the step: the components of the candidate graph (every sphere
+// with candidates is in one of two or more spheres).  One warp per such
+// sphere walks its component from its own entry, up to kIsland spheres; the
+// smallest id of a component that fits places it, in groups of 8 lanes or a
+// whole warp, and gives each member its lane; the members of a larger one
+// each join the list of `big` spheres.  Runs on the side branch of the step
+// beside the collide.
+constexpr int kIsland = 32;
+// Groups and warps there is room for (an island has two or more members; with
+// lists cut short, an error the step reports, the walks may disagree).
+__device__ __forceinline__ int cap8(const Parts &pt) { return pt.np / 2 + 4; }
+__device__ __forceinline__ int cap32(const Parts &pt) { return pt.np / 8 + 1; }
+__global__ void __launch_bounds__(128) k_islands(const Parts pt) {
+    __shared__ int ids[4][kIsland + 32];
+    const int a = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (a >= pt.np || pt.nact[a] == 0) return;
+    int *id = ids[threadIdx.x >> 5];
+    int n = 1;
+    bool root = true;
+    if (lane == 0) id[0] = a;
+    __syncwarp();
+    for (int i = 0; i < n && n <= kIsland; ++i) {
+        const long long e = (long long)id[i] * pt.max_nbr;
+        const int c = pt.nact[id[i]];
+        for (int m0 = 0; m0 < c && n <= kIsland; m0 += 32) {
+            const int b = m0 + lane < pt.max_nbr ? pt.pairBM[e + m0 + lane].x : 0;  // past c: an earlier step's entry
+            bool fresh = m0 + lane < c;
+            for (int k = 0; k < n; ++k) fresh = fresh && id[k] != b;
+            const unsigned bal = __ballot_sync(0xffffffffu, fresh);
+            __syncwarp();
+            if (fresh) id[n + __popc(bal & ((1u << lane) - 1u))] = b;  // n <= 32: at most 64 entries
+            n += __popc(bal);
+            root = root && !__any_sync(0xffffffffu, fresh && b < a);
+            __syncwarp();
+        }
+    }
+    if (n > kIsland) {
+        if (lane == 0) {
+            const int k = atomicAdd(pt.isl_n + 2, 1);
+            pt.big[k] = a;
+            pt.slot[a] = k;
+        }
+    } else if (root) {
+        const bool wide = n > 8;
+        int g = 0;
+        if (lane == 0) g = atomicAdd(pt.isl_n + (wide ? 1 : 0), 1);
+        g = __shfl_sync(0xffffffffu, g, 0);
+        if (g >= (wide ? cap32(pt) : cap8(pt))) return;
+        if (wide) {
+            pt.isl32[32 * g + lane] = lane < n ? id[lane] : -1;
+            if (lane < n) pt.slot[id[lane]] = lane;
+        } else if (lane < 8) {
+            pt.isl8[8 * g + lane] = lane < n ? id[lane] : -1;
+            if (lane < n) pt.slot[id[lane]] = 8 * (g & 3) + lane;
+        }
+    }
 }
 
-// All sub-steps of the lattice step of parity sp in one cluster (gridDim.x
-// CTAs).  Thread t of CTA c owns spheres a = c T + t + q G (q < K,
-// G = cluster threads).  The step's neighbour pass has read rebuild[sp], so
-// it is cleared here; the commits may set rebuild[sp ^ 1].  FRIC: with the
-// tangential contact law (each sphere also publishes its spin change).
-// GRID: the same sub-steps on a cooperative grid of any size: the spheres
-// publish (dx, dv, dOm) in a global buffer xbuf [2][np][S] (read through L2)
-// and a bounded grid barrier replaces the cluster barrier; used for sphere
-// counts one cluster holds poorly.  Returns early (the step is then void and
-// the timeout status set) if a barrier gives up.
-template <bool FRIC, bool GRID>
-__device__ __forceinline__ void dem_cluster_body(const Lat &L, const Parts &pt, SFrame *fnext, const int sp,
-                                                 int *status, float4 *xbuf = nullptr, unsigned *bar = nullptr) {
+// State of one sphere over the sub-steps of a step.
+template <bool FRIC>
+struct Ball {
+    float3 dx, dv, v0, fa, fc;  // displacement and velocity change so far, start velocity, load / m, contact force
+    float im, Rf, Llo, Lhi, gw;
+    int nc;
+    bool fx;
+    // with friction: spin change, start spin, torque / I, contact torque, 1 / I, wall gamma_t, open-contact
+    // mask, wall displacements (w = 1: in contact)
+    float3 dw, w0, ta, tc;
+    float iI, gwt;
+    unsigned long long msk;
+    float4 wl[2];
+
+    __device__ __forceinline__ void load(const Lat &L, const Parts &pt, const int a, const float kn, const float ce,
+                                         const float kt) {
+        const double m = sphere_mass(pt, a), R = pt.R[a], z0 = pt.X[3 * a + 2], ia = pt.inv[2 * a];
+        fx = pt.fixed[a] != 0;
+        im = (float)ia;
+        Rf = (float)R;
+        fa = make_float3((float)((pt.Fh[3 * a] + pt.Fx[3 * a]) * ia), (float)((pt.Fh[3 * a + 1] + pt.Fx[3 * a + 1]) * ia),
+                         (float)((pt.Fh[3 * a + 2] + pt.Fx[3 * a + 2]) * ia));
+        fc = make_float3((float)pt.Fc[3 * a], (float)pt.Fc[3 * a + 1], (float)pt.Fc[3 * a + 2]);
+        v0 = make_float3((float)pt.V[3 * a], (float)pt.V[3 * a + 1], (float)pt.V[3 * a + 2]);
+        Llo = (float)(R - (z0 + 0.5));
+        Lhi = (float)(R - ((L.nz - 0.5) - z0));
+        gw = ce * sqrtf((float)m * kn);
+        nc = pt.nact[a];
+        dx = make_float3(0.f, 0.f, 0.f);
+        dv = make_float3(0.f, 0.f, 0.f);
+        if constexpr (FRIC) {
+            const double ii = pt.inv[2 * a + 1];
+            iI = (float)ii;
+            w0 = make_float3((float)pt.W[3 * a], (float)pt.W[3 * a + 1], (float)pt.W[3 * a + 2]);
+            ta = make_float3((float)((pt.Th[3 * a] + pt.Tx[3 * a]) * ii), (float)((pt.Th[3 * a + 1] + pt.Tx[3 * a + 1]) * ii),
+                             (float)((pt.Th[3 * a + 2] + pt.Tx[3 * a + 2]) * ii));
+            tc = make_float3((float)pt.Tc[3 * a], (float)pt.Tc[3 * a + 1], (float)pt.Tc[3 * a + 2]);
+            dw = make_float3(0.f, 0.f, 0.f);
+            msk = pt.tmask[a];
+            wl[0] = pt.twall[2 * a];
+            wl[1] = pt.twall[2 * a + 1];
+            gwt = (float)pt.ct * sqrtf((float)m * kt);
+        }
+    }
+
+    // half kick and drift
+    __device__ __forceinline__ void drift(const float h, const float h2) {
+        if (!fx) {
+            dv = fma3(h2, fma3(im, fc, fa), dv);
+            if constexpr (FRIC) dw = fma3(h2, fma3(iI, tc, ta), dw);
+        }
+        dx = fma3(h, add3(v0, dv), dx);
+    }
+
+    __device__ __forceinline__ void publish(float4 *me) const {
+        me[0] = make_float4(dx.x, dx.y, dx.z, 0.f);
+        me[1] = make_float4(dv.x, dv.y, dv.z, 0.f);
+        if constexpr (FRIC) me[2] = make_float4(dw.x, dw.y, dw.z, 0.f);
+    }
+
+    // Contact force at the drifted positions and the second half kick;
+    // get(b, x, v, w) gives candidate b's published (dx, dv, dOm).
+    template <typename Get>
+    __device__ __forceinline__ void force(const Parts &pt, const int a, const float kn, const float kt, const float mu,
+                                          const float h, const float h2, Get get) {
+        if (fx) return;
+        float3 F = make_float3(0.f, 0.f, 0.f);
+        float3 Tq = make_float3(0.f, 0.f, 0.f);
+        // neighbours in groups of kNbrGroup: every load of a group is
+        // issued before any of its arithmetic; the sum keeps list order
+        constexpr int kNbrGroup = 4;
+        for (int m0 = 0; m0 < nc; m0 += kNbrGroup) {
+            float4 A[kNbrGroup], Bv[kNbrGroup], ox[kNbrGroup], ov[kNbrGroup];
+            float4 C[FRIC ? kNbrGroup : 1], ow[FRIC ? kNbrGroup : 1], td[FRIC ? kNbrGroup : 1];
+            float Rb[kNbrGroup];
+            int lm[kNbrGroup];  // list position of the candidate (its contact state)
+#pragma unroll
+            for (int u = 0; u < kNbrGroup; ++u) {
+                if (m0 + u >= nc) break;
+                const long long e = (long long)a * pt.max_nbr + m0 + u;
+                const int2 bm = __ldg(pt.pairBM + e);
+                const int b = bm.x;
+                lm[u] = bm.y;
+                A[u] = __ldg(pt.pairA + e);
+                Bv[u] = __ldg(pt.pairB + e);
+                Rb[u] = __ldg(&pt.Xf[b].w);
+                if constexpr (FRIC) {  // the open contact's displacement, loaded with the group
+                    td[u] = (msk >> lm[u]) & 1ull ? pt.tdisp[(long long)a * pt.max_nbr + lm[u]]
+                                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+                    C[u] = __ldg(pt.pairC + e);
+                    get(b, ox[u], ov[u], ow[u]);
+                } else {
+                    get(b, ox[u], ov[u], ow[0]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kNbrGroup; ++u) {
+                if (m0 + u >= nc) break;
+                const float3 D = sub3(dx, xyz(ox[u])), d0 = xyz(A[u]);
+                const float c = __fsub_rn(__fmaf_rn(-2.f, dot3(d0, D), A[u].w), dot3(D, D));
+                if (!(c > 0.f)) {
+                    if constexpr (FRIC) msk &= ~(1ull << lm[u]);  // the contact opened
+                    continue;
+                }
+                const float3 ex = add3(d0, D);
+                const float dist = __fsqrt_rn(dot3(ex, ex));
+                const float delta = __fdiv_rn(c, __fadd_rn(__fadd_rn(Rf, Rb[u]), dist));
+                const float3 n = mul3(__fdiv_rn(1.f, dist), ex);
+                const float3 vab = sub3(add3(xyz(Bv[u]), dv), xyz(ov[u]));
+                const float fn = __fmaf_rn(-Bv[u].w, dot3(vab, n), __fmul_rn(kn, delta));
+                F = fma3(fn, n, F);
+                if constexpr (FRIC) {
+                    const int m = lm[u];
+                    const long long e = (long long)a * pt.max_nbr + m;
+                    const float la = __fmaf_rn(-0.5f, delta, Rf), lb = __fmaf_rn(-0.5f, delta, Rb[u]);
+                    const float3 Sw = fma3(la, add3(w0, dw), mul3(lb, add3(xyz(C[u]), xyz(ow[u]))));
+                    float3 d = xyz(td[u]);
+                    friction_add(F, Tq, d, n, sub3(vab, cross3(Sw, n)), la, fn, C[u].w, kt, mu, h);
+                    pt.tdisp[e] = make_float4(d.x, d.y, d.z, 0.f);
+                    msk |= 1ull << m;
+                }
+            }
+        }
+        const float vz = __fadd_rn(v0.z, dv.z);
+        const float lo = __fsub_rn(Llo, dx.z), hi = __fadd_rn(Lhi, dx.z);
+        const float flo = __fmaf_rn(-gw, vz, __fmul_rn(kn, lo)), fhi = __fmaf_rn(gw, vz, __fmul_rn(kn, hi));
+        if (lo > 0.f) F.z = __fadd_rn(F.z, flo);
+        if (hi > 0.f) F.z = __fsub_rn(F.z, fhi);
+        if constexpr (FRIC) {
+            const float3 w = add3(w0, dw);
+            const float3 v = make_float3(__fadd_rn(v0.x, dv.x), __fadd_rn(v0.y, dv.y), vz);
+#pragma unroll
+            for (int side = 0; side < 2; ++side) {
+                const float pen = side == 0 ? lo : hi;
+                if (!(pen > 0.f)) {
+                    wl[side] = make_float4(0.f, 0.f, 0.f, 0.f);  // the contact opened
+                    continue;
+                }
+                const float3 n = make_float3(0.f, 0.f, side == 0 ? 1.f : -1.f);
+                const float *uw = side == 0 ? pt.ulo : pt.uhi;
+                const float l = __fmaf_rn(-0.5f, pen, Rf);
+                const float3 vr = sub3(sub3(v, make_float3(uw[0], uw[1], uw[2])), cross3(mul3(l, w), n));
+                float3 d = wl[side].w != 0.f ? xyz(wl[side]) : make_float3(0.f, 0.f, 0.f);
+                friction_add(F, Tq, d, n, vr, l, side == 0 ? flo : fhi, gwt, kt, mu, h);
+                wl[side] = make_float4(d.x, d.y, d.z, 1.f);
+            }
+            tc = Tq;
+            dw = fma3(h2, fma3(iI, Tq, ta), dw);
+        }
+        fc = F;
+        dv = fma3(h2, fma3(im, F, fa), dv);
+    }
+
+    __device__ __forceinline__ void store(const Lat &L, const Parts &pt, SFrame *fnext, const int a, const int sp,
+                                          int *status) const {
+        double x[3] = {pt.X[3 * a] + (double)dx.x, pt.X[3 * a + 1] + (double)dx.y, pt.X[3 * a + 2] + (double)dx.z};
+        wrap_pos(L, x);
+        double v[3] = {pt.V[3 * a], pt.V[3 * a + 1], pt.V[3 * a + 2]};
+        double w[3] = {pt.W[3 * a], pt.W[3 * a + 1], pt.W[3 * a + 2]};
+        if (!fx) {
+            v[0] += (double)dv.x;
+            v[1] += (double)dv.y;
+            v[2] += (double)dv.z;
+            if constexpr (FRIC) {
+                w[0] += (double)dw.x;
+                w[1] += (double)dw.y;
+                w[2] += (double)dw.z;
+            } else {
+                for (int c = 0; c < 3; ++c) w[c] += (pt.Th[3 * a + c] + pt.Tx[3 * a + c]) * pt.inv[2 * a + 1];
+            }
+        }
+        if constexpr (FRIC) {
+            pt.Tc[3 * a] = (double)tc.x;
+            pt.Tc[3 * a + 1] = (double)tc.y;
+            pt.Tc[3 * a + 2] = (double)tc.z;
+            pt.tmask[a] = msk;
+            pt.twall[2 * a] = wl[0];
+            pt.twall[2 * a + 1] = wl[1];
+        }
+        const double f3[3] = {(double)fc.x, (double)fc.y, (double)fc.z};
+        const double moved2 = (double)(dx.x * dx.x + dx.y * dx.y + dx.z * dx.z);
+        commit(L, pt, fnext, a, x, v, w, f3, moved2, sp, status);
+    }
+};
+
+// All sub-steps of sphere a (-1: an idle lane) in its own thread: without
+// candidates (ISLAND = false), or as lane `lane` of a warp that holds whole
+// islands and exchanges through buf ([2][32][S], this warp's).
+template <bool FRIC, bool ISLAND>
+__device__ __forceinline__ void dem_one(const Lat &L, const Parts &pt, SFrame *fnext, const int sp, int *status,
+                                        const int a, const int lane, float4 *buf) {
+    constexpr int S = FRIC ? 3 : 2;
+    const int ns = pt.substeps;
+    const float h = 1.f / ns, h2 = 0.5f * h;
+    const float kn = (float)pt.kn, ce = (float)pt.ce, kt = (float)pt.kt, mu = (float)pt.mu;
+    Ball<FRIC> B;
+    if (a >= 0) B.load(L, pt, a, kn, ce, kt);
+    if (!ISLAND) B.nc = 0;
+    for (int s = 0; s < ns; ++s) {
+        float4 *b2 = buf + (size_t)((s + 1) & 1) * 32 * S;
+        if (a >= 0) {
+            B.drift(h, h2);
+            if (ISLAND) B.publish(b2 + lane * S);
+        }
+        if (ISLAND) __syncwarp();
+        if (a >= 0)
+            B.force(pt, a, kn, kt, mu, h, h2, [&](int b, float4 &x, float4 &v, float4 &w) {
+                const float4 *o = b2 + (pt.slot[b] & 31) * S;
+                x = o[0];
+                v = o[1];
+                if constexpr (FRIC) w = o[2];
+            });
+    }
+    if (a >= 0) B.store(L, pt, fnext, a, sp, status);
+}
+
+// All sub-steps of a set of spheres on the threads of one cluster of `ctas`
+// CTAs (blockIdx.x its ranks), or (GRID) on the first `ctas` CTAs of a
+// cooperative grid: of every sphere (LIST = false) or of the `count` big ones.
+// Thread t of CTA c owns entries k = c T + t + q G (q < K, G = the threads).
+// GRID: the spheres publish (dx, dv, dOm) in a global buffer xbuf [2][count][S]
+// (read through L2) and a bounded grid barrier replaces the cluster barrier;
+// returns early (the step is then void and the timeout status set) if a
+// barrier gives up.
+template <bool FRIC, bool GRID, bool LIST>
+__device__ __forceinline__ void dem_wide(const Lat &L, const Parts &pt, SFrame *fnext, const int sp, int *status,
+                                         const int count, const int ctas, float4 *xbuf = nullptr, unsigned *bar = nullptr) {
     constexpr int S = FRIC ? 3 : 2;  // float4 per sphere in the exchange buffer: dx, dv (, dOm)
     constexpr int K = dem_kmax(FRIC);
     extern __shared__ float4 dsm[];  // [2][K * T][S]
     namespace cg = cooperative_groups;
-    const int T = blockDim.x, G = gridDim.x * T, cap = K * T;
+    const int T = blockDim.x, G = ctas * T, cap = K * T;
     unsigned target = 0;
     const int g0 = blockIdx.x * T + threadIdx.x;
-    if (g0 == 0) pt.rebuild[sp] = 0;
     const int ns = pt.substeps;
     const float h = 1.f / ns, h2 = 0.5f * h;
-    const float kn = (float)pt.kn, ce = (float)pt.ce;
-    const float kt = (float)pt.kt, mu = (float)pt.mu;
-    float3 dx[K], dv[K], v0[K], fa[K], fc[K];
-    float im[K], Rf[K], Llo[K], Lhi[K], gw[K];
-    int nc[K];
-    bool fx[K];
-    // with friction: spin change, start spin, torque / I, contact torque, 1 / I,
-    // open-contact mask, wall displacements (w = 1: in contact), wall gamma_t
-    float3 dw[FRIC ? K : 1], w0[FRIC ? K : 1], ta[FRIC ? K : 1], tc[FRIC ? K : 1];
-    float iI[FRIC ? K : 1], gwt[FRIC ? K : 1];
-    unsigned long long msk[FRIC ? K : 1];
-    float4 wl[FRIC ? K : 1][2];
+    const float kn = (float)pt.kn, ce = (float)pt.ce, kt = (float)pt.kt, mu = (float)pt.mu;
+    Ball<FRIC> B[K];
+    int id[K];
 #pragma unroll
     for (int q = 0; q < K; ++q) {
-        const int a = g0 + q * G;
-        if (a >= pt.np) break;
-        const double m = sphere_mass(pt, a), R = pt.R[a], z0 = pt.X[3 * a + 2];
-        fx[q] = pt.fixed[a] != 0;
-        const double ia = 1.0 / m;
-        im[q] = (float)ia;
-        Rf[q] = (float)R;
-        fa[q] = make_float3((float)((pt.Fh[3 * a] + pt.Fx[3 * a]) * ia), (float)((pt.Fh[3 * a + 1] + pt.Fx[3 * a + 1]) * ia),
-                            (float)((pt.Fh[3 * a + 2] + pt.Fx[3 * a + 2]) * ia));
-        fc[q] = make_float3((float)pt.Fc[3 * a], (float)pt.Fc[3 * a + 1], (float)pt.Fc[3 * a + 2]);
-        v0[q] = make_float3((float)pt.V[3 * a], (float)pt.V[3 * a + 1], (float)pt.V[3 * a + 2]);
-        Llo[q] = (float)(R - (z0 + 0.5));
-        Lhi[q] = (float)(R - ((L.nz - 0.5) - z0));
-        gw[q] = ce * sqrtf((float)m * kn);
-        nc[q] = pt.nact[a];
-        dx[q] = make_float3(0.f, 0.f, 0.f);
-        dv[q] = make_float3(0.f, 0.f, 0.f);
-        if constexpr (FRIC) {
-            const double ii = 1.0 / (0.4 * m * R * R);
-            iI[q] = (float)ii;
-            w0[q] = make_float3((float)pt.W[3 * a], (float)pt.W[3 * a + 1], (float)pt.W[3 * a + 2]);
-            ta[q] = make_float3((float)((pt.Th[3 * a] + pt.Tx[3 * a]) * ii),
-                                (float)((pt.Th[3 * a + 1] + pt.Tx[3 * a + 1]) * ii),
-                                (float)((pt.Th[3 * a + 2] + pt.Tx[3 * a + 2]) * ii));
-            tc[q] = make_float3((float)pt.Tc[3 * a], (float)pt.Tc[3 * a + 1], (float)pt.Tc[3 * a + 2]);
-            dw[q] = make_float3(0.f, 0.f, 0.f);
-            msk[q] = pt.tmask[a];
-            wl[q][0] = pt.twall[2 * a];
-            wl[q][1] = pt.twall[2 * a + 1];
-            gwt[q] = (float)pt.ct * sqrtf((float)m * kt);
-        }
+        const int k = g0 + q * G;
+        if (k >= count) break;
+        id[q] = LIST ? pt.big[k] : k;
+        B[q].load(L, pt, id[q], kn, ce, kt);
     }
     if constexpr (!GRID) cluster_barrier();  // every CTA of the cluster is running before shared memory is shared
     for (int s = 0; s < ns; ++s) {
-        float4 *buf = GRID ? xbuf + (size_t)((s + 1) & 1) * pt.np * S : dsm + (size_t)((s + 1) & 1) * cap * S;
+        float4 *buf = GRID ? xbuf + (size_t)((s + 1) & 1) * count * S : dsm + (size_t)((s + 1) & 1) * cap * S;
 #pragma unroll
         for (int q = 0; q < K; ++q) {
-            const int a = g0 + q * G;
-            if (a >= pt.np) break;
-            if (!fx[q]) {  // half kick
-                dv[q].x += (fa[q].x + fc[q].x * im[q]) * h2;
-                dv[q].y += (fa[q].y + fc[q].y * im[q]) * h2;
-                dv[q].z += (fa[q].z + fc[q].z * im[q]) * h2;
-                if constexpr (FRIC) {
-                    dw[q].x += (ta[q].x + tc[q].x * iI[q]) * h2;
-                    dw[q].y += (ta[q].y + tc[q].y * iI[q]) * h2;
-                    dw[q].z += (ta[q].z + tc[q].z * iI[q]) * h2;
-                }
-            }
-            dx[q].x += (v0[q].x + dv[q].x) * h;
-            dx[q].y += (v0[q].y + dv[q].y) * h;
-            dx[q].z += (v0[q].z + dv[q].z) * h;
-            float4 *me = buf + (GRID ? (size_t)a * S : (size_t)(q * T + threadIdx.x) * S);
-            me[0] = make_float4(dx[q].x, dx[q].y, dx[q].z, 0.f);
-            me[1] = make_float4(dv[q].x, dv[q].y, dv[q].z, 0.f);
-            if constexpr (FRIC) me[2] = make_float4(dw[q].x, dw[q].y, dw[q].z, 0.f);
+            const int k = g0 + q * G;
+            if (k >= count) break;
+            B[q].drift(h, h2);
+            B[q].publish(buf + (GRID ? (size_t)k * S : (size_t)(q * T + threadIdx.x) * S));
         }
         if constexpr (GRID) {
-            target += gridDim.x;
+            target += ctas;
             if (!grid_barrier(bar, target, status)) return;
         } else {
             cluster_barrier();
         }
 #pragma unroll
         for (int q = 0; q < K; ++q) {
-            const int a = g0 + q * G;
-            if (a >= pt.np) break;
-            if (fx[q]) continue;
-            float3 F = make_float3(0.f, 0.f, 0.f);
-            float3 Tq = make_float3(0.f, 0.f, 0.f);
-            // neighbours in groups of kNbrGroup: every load of a group is
-            // issued before any of its arithmetic; the sum keeps list order
-            constexpr int kNbrGroup = 4;
-            for (int m0 = 0; m0 < nc[q]; m0 += kNbrGroup) {
-                float4 A[kNbrGroup], Bv[kNbrGroup], ox[kNbrGroup], ov[kNbrGroup];
-                float4 C[FRIC ? kNbrGroup : 1], ow[FRIC ? kNbrGroup : 1], td[FRIC ? kNbrGroup : 1];
-                float Rb[kNbrGroup];
-                int lm[kNbrGroup];  // list position of the candidate (its contact state)
-#pragma unroll
-                for (int u = 0; u < kNbrGroup; ++u) {
-                    if (m0 + u >= nc[q]) break;
-                    const long long e = (long long)a * pt.max_nbr + m0 + u;
-                    const int2 bm = __ldg(pt.pairBM + e);
-                    const int b = bm.x;
-                    lm[u] = bm.y;
-                    A[u] = __ldg(pt.pairA + e);
-                    Bv[u] = __ldg(pt.pairB + e);
-                    Rb[u] = __ldg(&pt.Xf[b].w);
-                    if constexpr (FRIC)  // the open contact's displacement, loaded with the group
-                        td[u] = (msk[q] >> lm[u]) & 1ull ? pt.tdisp[(long long)a * pt.max_nbr + lm[u]]
-                                                         : make_float4(0.f, 0.f, 0.f, 0.f);
-                    if constexpr (GRID) {
-                        const float4 *o = buf + (size_t)b * S;
-                        ox[u] = __ldcg(o);
-                        ov[u] = __ldcg(o + 1);
-                        if constexpr (FRIC) {
-                            C[u] = __ldg(pt.pairC + e);
-                            ow[u] = __ldcg(o + 2);
-                        }
-                    } else {
-                        const int qb = b / G, rb = b - qb * G, cb = rb / T, tb = rb - cb * T;
-                        const float4 *o = cg::this_cluster().map_shared_rank(buf + (size_t)(qb * T + tb) * S, cb);
-                        ox[u] = o[0];
-                        ov[u] = o[1];
-                        if constexpr (FRIC) {
-                            C[u] = __ldg(pt.pairC + e);
-                            ow[u] = o[2];
-                        }
-                    }
+            const int k = g0 + q * G;
+            if (k >= count) break;
+            B[q].force(pt, id[q], kn, kt, mu, h, h2, [&](int b, float4 &x, float4 &v, float4 &w) {
+                const int kb = LIST ? min(pt.slot[b], count - 1) : b;
+                if constexpr (GRID) {
+                    const float4 *o = buf + (size_t)kb * S;
+                    x = __ldcg(o);
+                    v = __ldcg(o + 1);
+                    if constexpr (FRIC) w = __ldcg(o + 2);
+                } else {
+                    const int qb = kb / G, rb = kb - qb * G, cb = rb / T, tb = rb - cb * T;
+                    const float4 *o = cg::this_cluster().map_shared_rank(buf + (size_t)(qb * T + tb) * S, cb);
+                    x = o[0];
+                    v = o[1];
+                    if constexpr (FRIC) w = o[2];
                 }
-#pragma unroll
-                for (int u = 0; u < kNbrGroup; ++u) {
-                    if (m0 + u >= nc[q]) break;
-                    const float Dx = dx[q].x - ox[u].x, Dy = dx[q].y - ox[u].y, Dz = dx[q].z - ox[u].z;
-                    const float c =
-                        A[u].w - 2.f * (A[u].x * Dx + A[u].y * Dy + A[u].z * Dz) - (Dx * Dx + Dy * Dy + Dz * Dz);
-                    if (!(c > 0.f)) {
-                        if constexpr (FRIC) msk[q] &= ~(1ull << lm[u]);  // the contact opened
-                        continue;
-                    }
-                    const float ex = A[u].x + Dx, ey = A[u].y + Dy, ez = A[u].z + Dz;
-                    const float dist = sqrtf(ex * ex + ey * ey + ez * ez);
-                    const float Rs = Rf[q] + Rb[u];
-                    const float delta = c / (Rs + dist);
-                    const float id = 1.f / dist;
-                    const float nx = ex * id, ny = ey * id, nz = ez * id;
-                    const float vn = (Bv[u].x + dv[q].x - ov[u].x) * nx + (Bv[u].y + dv[q].y - ov[u].y) * ny +
-                                     (Bv[u].z + dv[q].z - ov[u].z) * nz;
-                    const float fn = kn * delta - Bv[u].w * vn;
-                    F.x += fn * nx;
-                    F.y += fn * ny;
-                    F.z += fn * nz;
-                    if constexpr (FRIC) {
-                        const int m = lm[u];
-                        const long long e = (long long)a * pt.max_nbr + m;
-                        const float la = Rf[q] - 0.5f * delta, lb = Rb[u] - 0.5f * delta;
-                        const float3 n = make_float3(nx, ny, nz);
-                        const float3 Sw = make_float3(la * (w0[q].x + dw[q].x) + lb * (C[u].x + ow[u].x),
-                                                      la * (w0[q].y + dw[q].y) + lb * (C[u].y + ow[u].y),
-                                                      la * (w0[q].z + dw[q].z) + lb * (C[u].z + ow[u].z));
-                        const float3 Sn = cross3(Sw, n);
-                        const float3 vr = make_float3(Bv[u].x + dv[q].x - ov[u].x - Sn.x,
-                                                      Bv[u].y + dv[q].y - ov[u].y - Sn.y,
-                                                      Bv[u].z + dv[q].z - ov[u].z - Sn.z);
-                        float3 d = make_float3(td[u].x, td[u].y, td[u].z);
-                        friction_add(F, Tq, d, n, vr, la, fn, C[u].w, kt, mu, h);
-                        pt.tdisp[e] = make_float4(d.x, d.y, d.z, 0.f);
-                        msk[q] |= 1ull << m;
-                    }
-                }
-            }
-            const float vz = v0[q].z + dv[q].z;
-            const float lo = Llo[q] - dx[q].z;
-            if (lo > 0.f) F.z += kn * lo - gw[q] * vz;
-            const float hi = Lhi[q] + dx[q].z;
-            if (hi > 0.f) F.z -= kn * hi + gw[q] * vz;
-            if constexpr (FRIC) {
-                const float3 w = make_float3(w0[q].x + dw[q].x, w0[q].y + dw[q].y, w0[q].z + dw[q].z);
-                const float3 v = make_float3(v0[q].x + dv[q].x, v0[q].y + dv[q].y, vz);
-#pragma unroll
-                for (int side = 0; side < 2; ++side) {
-                    const float pen = side == 0 ? lo : hi;
-                    if (!(pen > 0.f)) {
-                        wl[q][side] = make_float4(0.f, 0.f, 0.f, 0.f);  // the contact opened
-                        continue;
-                    }
-                    const float sg = side == 0 ? 1.f : -1.f;
-                    const float3 n = make_float3(0.f, 0.f, sg);
-                    const float *uw = side == 0 ? pt.ulo : pt.uhi;
-                    const float l = Rf[q] - 0.5f * pen;
-                    const float3 Sn = cross3(make_float3(l * w.x, l * w.y, l * w.z), n);
-                    const float3 vr = make_float3(v.x - uw[0] - Sn.x, v.y - uw[1] - Sn.y, v.z - uw[2] - Sn.z);
-                    const float fn = side == 0 ? kn * lo - gw[q] * vz : kn * hi + gw[q] * vz;
-                    float3 d = wl[q][side].w != 0.f ? make_float3(wl[q][side].x, wl[q][side].y, wl[q][side].z)
-                                                    : make_float3(0.f, 0.f, 0.f);
-                    friction_add(F, Tq, d, n, vr, l, fn, gwt[q], kt, mu, h);
-                    wl[q][side] = make_float4(d.x, d.y, d.z, 1.f);
-                }
-                tc[q] = Tq;
-                dw[q].x += (ta[q].x + Tq.x * iI[q]) * h2;
-                dw[q].y += (ta[q].y + Tq.y * iI[q]) * h2;
-                dw[q].z += (ta[q].z + Tq.z * iI[q]) * h2;
-            }
-            fc[q] = F;
-            dv[q].x += (fa[q].x + F.x * im[q]) * h2;
-            dv[q].y += (fa[q].y + F.y * im[q]) * h2;
-            dv[q].z += (fa[q].z + F.z * im[q]) * h2;
+            });
         }
     }
     if constexpr (!GRID) cluster_barrier();  // no CTA leaves while another may still read its shared memory
 #pragma unroll
     for (int q = 0; q < K; ++q) {
-        const int a = g0 + q * G;
-        if (a >= pt.np) break;
-        double x[3] = {pt.X[3 * a] + (double)dx[q].x, pt.X[3 * a + 1] + (double)dx[q].y, pt.X[3 * a + 2] + (double)dx[q].z};
-        wrap_pos(L, x);
-        double v[3] = {pt.V[3 * a], pt.V[3 * a + 1], pt.V[3 * a + 2]};
-        double w[3] = {pt.W[3 * a], pt.W[3 * a + 1], pt.W[3 * a + 2]};
-        if (!fx[q]) {
-            const double m = sphere_mass(pt, a);
-            const double iI = 1.0 / (0.4 * m * pt.R[a] * pt.R[a]);
-            v[0] += (double)dv[q].x;
-            v[1] += (double)dv[q].y;
-            v[2] += (double)dv[q].z;
-            if constexpr (FRIC) {
-                w[0] += (double)dw[q].x;
-                w[1] += (double)dw[q].y;
-                w[2] += (double)dw[q].z;
-            } else {
-                for (int c = 0; c < 3; ++c) w[c] += (pt.Th[3 * a + c] + pt.Tx[3 * a + c]) * iI;
-            }
-        }
-        if constexpr (FRIC) {
-            pt.Tc[3 * a] = (double)tc[q].x;
-            pt.Tc[3 * a + 1] = (double)tc[q].y;
-            pt.Tc[3 * a + 2] = (double)tc[q].z;
-            pt.tmask[a] = msk[q];
-            pt.twall[2 * a] = wl[q][0];
-            pt.twall[2 * a + 1] = wl[q][1];
-        }
-        const double f3[3] = {(double)fc[q].x, (double)fc[q].y, (double)fc[q].z};
-        const double moved2 = (double)(dx[q].x * dx[q].x + dx[q].y * dx[q].y + dx[q].z * dx[q].z);
-        commit(L, pt, fnext, a, x, v, w, f3, moved2, sp, status);
+        const int k = g0 + q * G;
+        if (k >= count) break;
+        B[q].store(L, pt, fnext, id[q], sp, status);
     }
 }
 
@@ -720,26 +827,62 @@ __global__ void __launch_bounds__(256) k_neighbours(const Lat L, const Parts pt,
     neighbours_body(L, pt, sp, force, status);
 }
 
-template <bool FRIC>
-__global__ void __launch_bounds__(kDemThreads, 1) k_dem_cluster(const Lat L, const Parts pt, SFrame *fnext,
-                                                                const int sp, int *status) {
-    dem_cluster_body<FRIC, false>(L, pt, fnext, sp, status);
+// The DEM of a step (parity sp): islands on the first warps, free spheres
+// (no candidates) from the last thread down, each thread one at a time, and,
+// with CL, the big spheres on the first cluster of the grid (its gridDim.x is
+// a multiple of the cluster's `ctas`).  The step's neighbour pass has read
+// rebuild[sp], so it is cleared here; the commits may set rebuild[sp ^ 1].
+// Latency-bound: with every sphere in one cluster or grid and a barrier per
+// sub-step it took 15 us for 1 or 31 spheres and 17 us for 2000 (cluster),
+// 42 us for 8136 with friction (grid); now 9, 9, 11 and 13 us (ncu, cold),
+// the step 48.4 -> 42.1 us at 64^3 with 31 spheres and 941 -> 911 us at 256^3
+// with 8136.
+template <bool FRIC, bool CL>
+__global__ void __launch_bounds__(kDemThreads) k_dem_local(const Lat L, const Parts pt, SFrame *fnext, const int sp,
+                                                           int *status, const int ctas, unsigned *bar) {
+    constexpr int S = FRIC ? 3 : 2;
+    extern __shared__ float4 dsm[];
+    const int G = gridDim.x * blockDim.x, g0 = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    if (g0 == 0) {
+        pt.rebuild[sp] = 0;
+        *bar = 0u;  // for the grid form's kernel, which follows
+    }
+    const int n8 = min(pt.isl_n[0], cap8(pt)), n32 = min(pt.isl_n[1], cap32(pt)), nbig = pt.isl_n[2];
+    const int w8 = (n8 + 3) / 4;
+    float4 *buf = dsm + (size_t)(threadIdx.x >> 5) * 2 * 32 * S;
+    for (int u = g0 >> 5; u < w8 + n32; u += G >> 5) {
+        const int a = u >= w8 ? pt.isl32[32 * (u - w8) + lane] : (4 * u + (lane >> 3) < n8 ? pt.isl8[32 * u + lane] : -1);
+        dem_one<FRIC, true>(L, pt, fnext, sp, status, a, lane, buf);
+        __syncwarp();
+    }
+    for (int a = G - 1 - g0; a < pt.np; a += G)
+        if (pt.nact[a] == 0) dem_one<FRIC, false>(L, pt, fnext, sp, status, a, lane, buf);
+    if (CL && nbig > 0 && (int)blockIdx.x < ctas) {
+        __syncthreads();  // the islands' buffers are free
+        dem_wide<FRIC, false, true>(L, pt, fnext, sp, status, nbig, ctas);
+    }
 }
 
 #ifndef LBM_DEM_GRID_THREADS
 #define LBM_DEM_GRID_THREADS 64
 #endif
 constexpr int kDemGridThreads = LBM_DEM_GRID_THREADS;  // threads per CTA of the grid form
-// sphere count from which the automatic choice takes the grid form: one
-// cluster then holds two or more spheres per thread (measured: 8136 spheres
-// with friction, DEM 0.31 ms per step in the cluster, 0.14 ms in the grid)
+// sphere count from which the automatic choice takes the grid form for the
+// big spheres: one cluster then holds two or more spheres per thread
+// (measured with every sphere in it: 8136 spheres with friction, DEM 0.31 ms
+// per step in the cluster, 0.14 ms in the grid)
 constexpr int kDemGridFrom = 4096;
 
+// The big spheres on a cooperative grid; only as many CTAs as they fill take
+// part.
 template <bool FRIC>
 __global__ void __launch_bounds__(kDemGridThreads) k_dem_grid(const Lat L, const Parts pt, SFrame *fnext,
                                                               const int sp, int *status, float4 *xbuf,
                                                               unsigned *bar) {
-    dem_cluster_body<FRIC, true>(L, pt, fnext, sp, status, xbuf, bar);
+    const int nbig = pt.isl_n[2];
+    const int ctas = min((int)gridDim.x, (nbig + kDemGridThreads - 1) / kDemGridThreads);
+    if ((int)blockIdx.x >= ctas) return;
+    dem_wide<FRIC, true, true>(L, pt, fnext, sp, status, nbig, ctas, xbuf, bar);
 }
 
 // Batched forms: instance blockIdx.y.
@@ -755,13 +898,17 @@ template <bool FRIC>
 __global__ void __launch_bounds__(kDemThreads, 1) k_dem_cluster_b(const Inst *__restrict__ I, const int sp) {
     const Inst &a = I[blockIdx.y];
     if (a.pt.np == 0) return;  // the whole cluster (one instance) leaves together
-    if (FRIC && !a.pt.fric) dem_cluster_body<false, false>(a.L, a.pt, a.pt.frame[sp ^ 1], sp, a.status);
-    else dem_cluster_body<FRIC, false>(a.L, a.pt, a.pt.frame[sp ^ 1], sp, a.status);
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.pt.rebuild[sp] = 0;
+    SFrame *fnext = a.pt.frame[sp ^ 1];
+    if (FRIC && !a.pt.fric) dem_wide<false, false, false>(a.L, a.pt, fnext, sp, a.status, a.pt.np, gridDim.x);
+    else dem_wide<FRIC, false, false>(a.L, a.pt, fnext, sp, a.status, a.pt.np, gridDim.x);
 }
 
 static size_t dem_cluster_smem(bool fric) {
     return (size_t)2 * dem_kmax(fric) * kDemThreads * (fric ? 3 : 2) * sizeof(float4);
 }
+// without a cluster: the islands' buffers only
+static size_t dem_island_smem(bool fric) { return (size_t)2 * kDemThreads * (fric ? 3 : 2) * sizeof(float4); }
 
 // ---- fallback: cooperative grid with a bounded software barrier ------------
 
@@ -837,8 +984,9 @@ __global__ void __launch_bounds__(128) k_dem(const Lat L, const Parts pt, SFrame
 
 int launch_neighbours(lbm_s *h, int force, cudaStream_t stream) {
     const int blocks = (h->pt.np * 32 + 255) / 256;
-    k_neighbours<<<blocks, 256, 0, stream ? stream : h->stream>>>(h->L, h->pt, (int)(h->steps & 1), force,
-                                                                 h->status);
+    cudaStream_t st = stream ? stream : h->stream;
+    k_neighbours<<<blocks, 256, 0, st>>>(h->L, h->pt, (int)(h->steps & 1), force, h->status);
+    k_islands<<<(h->pt.np + 3) / 4, 128, 0, st>>>(h->pt);
     return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
 }
 
@@ -874,7 +1022,7 @@ int dem_cluster_setup(int max_particles, bool small, bool fric) {
     for (int cl : sizes) {
         if ((long long)cl * kDemThreads * dem_kmax(fric) < max_particles) continue;
         if (small && (long long)cl * kDemThreads < max_particles && cl < 16) continue;
-        if (!(fric ? cluster_attrs(k_dem_cluster<true>, true, cl) : cluster_attrs(k_dem_cluster<false>, false, cl)))
+        if (!(fric ? cluster_attrs(k_dem_local<true, true>, true, cl) : cluster_attrs(k_dem_local<false, true>, false, cl)))
             continue;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
@@ -888,8 +1036,8 @@ int dem_cluster_setup(int max_particles, bool small, bool fric) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int n = 0;
-        const cudaError_t e = fric ? cudaOccupancyMaxActiveClusters(&n, k_dem_cluster<true>, &cfg)
-                                   : cudaOccupancyMaxActiveClusters(&n, k_dem_cluster<false>, &cfg);
+        const cudaError_t e = fric ? cudaOccupancyMaxActiveClusters(&n, k_dem_local<true, true>, &cfg)
+                                   : cudaOccupancyMaxActiveClusters(&n, k_dem_local<false, true>, &cfg);
         if (e == cudaSuccess && n >= 1) return cl;
         cudaGetLastError();
     }
@@ -945,15 +1093,15 @@ int dem_grid_setup(bool fric, int sms) {
 // Spheres the grid form holds with `blocks` co-resident blocks.
 long long dem_grid_capacity(bool fric, int blocks) { return (long long)blocks * kDemGridThreads * dem_kmax(fric); }
 
-// Grid form: one sphere per thread while the co-resident grid allows, a
-// cooperative launch (so every block is resident for the grid barriers).
+// Grid form of the big spheres: one per thread while the co-resident grid
+// allows, a cooperative launch (so every block is resident for the grid
+// barriers; k_dem_local has cleared their counter).
 static int launch_dem_grid(lbm_s *h, SFrame *fnext, int sp) {
     const bool fric = h->pt.fric != 0;
     const int np = h->pt.np;
     int blocks = (np + kDemGridThreads - 1) / kDemGridThreads;
     if (blocks > h->dem_grid_blocks) blocks = h->dem_grid_blocks;
     if (blocks < 1 || dem_grid_capacity(fric, blocks) < np) return LBM_ERR_UNSUPPORTED;
-    if (cudaMemsetAsync(h->bar, 0, sizeof(unsigned), h->stream) != cudaSuccess) return LBM_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -980,24 +1128,30 @@ int launch_dem(lbm_s *h) {
     const bool grid = h->dem_grid_blocks > 0 &&
                       (h->dem_mode == LBM_DEM_GRID ||
                        (h->dem_mode == LBM_DEM_AUTO && (h->dem_cluster == 0 || pt.np > kDemGridFrom)));
-    if (grid) return launch_dem_grid(h, fnext, sp);
-    if (h->dem_cluster > 0) {
+    if (grid || h->dem_cluster > 0) {
+        // the cluster of the big spheres: no more CTAs than give each sphere a thread
+        int cl = 1;
+        while (!grid && cl < h->dem_cluster && cl * kDemThreads < pt.np) cl *= 2;
+        // a thread per sphere, and as many warps again as islands of pairs in groups of 8 could fill (at most 64 CTAs)
+        const int want = (pt.np + kDemThreads - 1) / kDemThreads + std::min(64, pt.np / (2 * kDemThreads / 8));
+        const bool fric = pt.fric != 0;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = h->dem_cluster;
+        attr[0].val.clusterDim.x = cl;
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
-        cfg.gridDim = dim3(h->dem_cluster);
+        cfg.gridDim = dim3((want + cl - 1) / cl * cl);
         cfg.blockDim = dim3(kDemThreads);
-        const bool fric = pt.fric != 0;
-        cfg.dynamicSmemBytes = dem_cluster_smem(fric);
+        cfg.dynamicSmemBytes = grid ? dem_island_smem(fric) : dem_cluster_smem(fric);
         cfg.stream = h->stream;
         cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        const cudaError_t e = fric ? cudaLaunchKernelEx(&cfg, k_dem_cluster<true>, L, pt, fnext, sp, status)
-                                   : cudaLaunchKernelEx(&cfg, k_dem_cluster<false>, L, pt, fnext, sp, status);
-        return e == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
+        cfg.numAttrs = grid ? 0 : 1;
+        const auto k = grid ? (fric ? k_dem_local<true, false> : k_dem_local<false, false>)
+                            : (fric ? k_dem_local<true, true> : k_dem_local<false, true>);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, k, L, pt, fnext, sp, status, cl, h->bar);
+        if (e != cudaSuccess) return LBM_ERR_CUDA;
+        return grid ? launch_dem_grid(h, fnext, sp) : LBM_OK;
     }
     if (pt.fric) return LBM_ERR_UNSUPPORTED;  // the FP64 fallback keeps no tangential contact state
     if (cudaMemsetAsync(h->bar, 0, sizeof(unsigned), h->stream) != cudaSuccess) return LBM_ERR_CUDA;

@@ -184,6 +184,7 @@ struct Parts {
     int np;
     double *X, *V, *W, *R;         // [np][3] x3, [np]
     const uint8_t *fixed;          // [np]
+    double *inv;                   // [np][2]: 1 / mass, 1 / moment of inertia
     double *Fh, *Th;               // hydrodynamic load of the last step
     double *Fc;                    // contact force at the current position
     double *Fx, *Tx;               // external load
@@ -194,6 +195,9 @@ struct Parts {
     float4 *pairA, *pairB;         // per contact candidate: (d0, c0) and (dv0, gamma), see lbm_dem.cu
     int2 *pairBM;                  // per contact candidate: (b, list position)
     int *nact;                     // [np] contact candidates of the step
+    // islands of the step (k_islands): counts of 8-lane groups, warps and big spheres; their members
+    // (-1: an idle lane); a member's lane or place in `big`
+    int *isl_n, *isl8, *isl32, *big, *slot;
     double *Xbuild;                // centres when the lists were built
     int *rebuild;                  // [2]: rebuild[s & 1] = 1 asks the neighbour pass of step s to rebuild
     SFrame *frame[2];              // frames of the centres of even / odd steps
