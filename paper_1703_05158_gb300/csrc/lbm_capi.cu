@@ -540,7 +540,7 @@ int lbm_set_particles(lbm_handle h, int32_t n, const double *pos, const double *
     h->steps = 0;
     if (!rc && h->zieb) rc = zieb_reset(h, h->zvp);  // the cylinder starts at rest with the fluid
     if (!rc && n) rc = launch_neighbours(h, 1);
-    if (!rc && n) rc = launch_mark(h, h->parity, 0);
+    if (!rc && n) rc = launch_mark(h, h->parity, true);
     if (!rc && n) rc = launch_contact(h);
     if (!rc && n && h->overlap) {
         // near set of step 0 from the initial centres; events in a recorded state
@@ -640,7 +640,7 @@ namespace {
 int serial_step_launches(lbm_s *h) {
     const int P = h->parity;
     auto ok = [](cudaError_t e) { return e == cudaSuccess ? LBM_OK : LBM_ERR_CUDA; };
-    int rc = launch_mark(h, P, h->pt.corr);
+    int rc = launch_mark(h, P);
     if (!rc) rc = ok(cudaEventRecord(h->ev_fork, h->stream));
     if (!rc) rc = ok(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
     if (!rc) rc = launch_neighbours(h, 0, h->side);
@@ -767,7 +767,7 @@ int lbm_step(lbm_handle h, int32_t nsteps) {
             if (!rc) rc = ok(cudaEventRecord(h->ev_cf, Bs));
         }
         if (!rc) rc = prof_mark(h, E0, A);
-        if (!rc && parts) rc = launch_mark(h, P, h->pt.corr);
+        if (!rc && parts) rc = launch_mark(h, P);
         if (!rc && parts) rc = launch_refill(h, P);
         if (!rc) rc = prof_mark(h, E1, A);
         if (ovl) {

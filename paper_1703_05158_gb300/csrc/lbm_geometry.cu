@@ -5,20 +5,27 @@
 //   0       fluid
 //   1 or 3  solid, owner[n] = its sphere: the marks of a step of even step
 //           count write 1, those of an odd step 3 (the mark value `cur` of
-//           the step), so a solid node of the previous geometry that the
-//           current marks did not take keeps the other value
-//   2       fluid now, solid at the previous step (the refill turns nodes of
-//           the other mark value into 2; the collide kernel turns 2 into 0)
+//           the step)
+//   2       fluid now, solid at the previous step (the refill turns uncovered
+//           nodes into 2; the collide kernel turns 2 into 0)
 //
 //   mark:   nodes inside sphere p at the current centre, unless a
 //           neighbouring sphere that also contains the node has a smaller
 //           |x - X| - R (ties to the smaller index) -> cur, owner p
-//   refill: nodes of sphere p left at the previous step's mark value take
-//           the equilibrium (Eq. 9) at the surface velocity of p and at the
-//           mean density of the neighbours fluid before and after (flag 0),
-//           then become 2.
-// After the refill every solid node carries the current mark value, and
-// bit 0 is the fluid / solid class for every reader.
+//   refill: nodes of sphere p that it no longer contains and nobody else took
+//           take the equilibrium (Eq. 9) at the surface velocity of p and at
+//           the mean density of the neighbours fluid before and after (flag
+//           0), then become 2.
+//
+// Spheres that can contain a node together are contact candidates of the
+// previous neighbour pass (its reach covers a step's motion), so only those
+// are asked; a sphere without candidates keeps its nodes between steps and
+// writes the ones its motion adds.  Which nodes a motion adds and drops
+// follows from the two centres alone, so memory is read at those only (about
+// one node per sphere and step): marks + refill of 2000 spheres read 1.5M
+// flags and owners before.  The momentum correction visits every node of a
+// sphere each step: there a solid node of the previous geometry that the
+// current marks did not take is known by the other mark value.
 //
 // Inside tests and keys are FP32 on relative coordinates
 // (float)(x - b) - (float)(X - b), b = floor(X) (the sphere frames written
@@ -78,6 +85,18 @@ struct BoxWalk {
 // of FP32 radius R: offsets lie in [-ceil(R) + 1, ceil(R)].
 __device__ __forceinline__ int ext_of(float R) { return (int)ceilf(R); }
 
+// Whether the node at offset (ox, oy, oz) from floor(X) lies in the sphere.
+__device__ __forceinline__ bool inside(const SFrame &F, const int ox, const int oy, const int oz) {
+    return dist2(rel(ox, F.fr[0]), rel(oy, F.fr[1]), rel(oz, F.fr[2])) < F.R2;
+}
+
+// floor(X) of frame a relative to that of frame b (x and y periodic).
+struct Shift {
+    int x, y, z;
+    __device__ __forceinline__ Shift(const Lat &L, const SFrame &a, const SFrame &b)
+        : x(fold(a.b[0], b.b[0], L.nx)), y(fold(a.b[1], b.b[1], L.ny)), z(a.b[2] - b.b[2]) {}
+};
+
 constexpr int MAX_NBR_SMEM = 64;
 
 // Momentum m of a node and its moment l x m, accumulated into acc[0..5]
@@ -115,24 +134,39 @@ __device__ __forceinline__ int mark_node(const Lat &L, const SFrame &F, const SF
     return x + L.nx * (y + L.ny * z);
 }
 
-// The plain marks: flag cur and owner p on every node sphere p wins.
+// The plain marks: flag cur and owner p on the nodes sphere p wins; without
+// contact candidates and not `full` (the first marks of a placement) only on
+// those it did not contain at the previous step's centre (fprev).
 __device__ __forceinline__ void mark_body(const Lat &L, const Parts &pt, const SFrame *__restrict__ fcur,
-                                          uint8_t *__restrict__ flag, int32_t *__restrict__ owner, const uint8_t cur) {
+                                          const SFrame *__restrict__ fprev, uint8_t *__restrict__ flag,
+                                          int32_t *__restrict__ owner, const uint8_t cur, const int full) {
     const int p = blockIdx.x;
     __shared__ SFrame nf[MAX_NBR_SMEM];
     __shared__ int nid[MAX_NBR_SMEM];
-    const int cnt = min(pt.nbr_cnt[p], MAX_NBR_SMEM);
+    const SFrame F = fcur[p];
+    const int cnt = min(pt.nact[p], MAX_NBR_SMEM);
+    const int e = ext_of(F.R), E = 2 * e, E3 = E * E * E, lo = 1 - e;
+    BoxWalk w(threadIdx.x, blockDim.x, E);
+    if (cnt == 0 && !full) {
+        const SFrame G = fprev[p];
+        const Shift d(L, F, G);
+        for (int t = threadIdx.x; t < E3; t += blockDim.x, w.next()) {
+            const int ox = w.ox + lo, oy = w.oy + lo, oz = w.oz + lo, z = F.b[2] + oz;
+            if (!inside(F, ox, oy, oz) || inside(G, ox + d.x, oy + d.y, oz + d.z) || z < 0 || z >= L.nz) continue;
+            const int n = wrapi(F.b[0] + ox, L.nx) + L.nx * (wrapi(F.b[1] + oy, L.ny) + L.ny * z);
+            flag[n] = cur;
+            owner[n] = p;
+        }
+        return;
+    }
     for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-        const int q = pt.nbr[(long long)p * pt.max_nbr + t];
+        const int q = pt.pairBM[(long long)p * pt.max_nbr + t].x;
         nid[t] = q;
         nf[t] = fcur[q];
     }
-    const SFrame F = fcur[p];
     __syncthreads();
-    const int e = ext_of(F.R), B = 2 * e + 1, B3 = B * B * B;
-    BoxWalk w(threadIdx.x, blockDim.x, B);
-    for (int t = threadIdx.x; t < B3; t += blockDim.x, w.next()) {
-        const int n = mark_node(L, F, nf, nid, cnt, p, w.ox - e, w.oy - e, w.oz - e);
+    for (int t = threadIdx.x; t < E3; t += blockDim.x, w.next()) {
+        const int n = mark_node(L, F, nf, nid, cnt, p, w.ox + lo, w.oy + lo, w.oz + lo);
         if (n < 0) continue;
         flag[n] = cur;
         owner[n] = p;
@@ -254,12 +288,12 @@ constexpr int kGeomThreads = LBM_GEOM_THREADS;
 // are resident at once (one wave): 32 registers for the marks, 40 for the
 // refill.
 template <typename T, bool CORR>
-__global__ void __launch_bounds__(CORR ? 256 : kGeomThreads, CORR ? 4 : 2048 / kGeomThreads) k_mark(const Lat L, const Parts pt, const SFrame *__restrict__ fcur,
-                                              uint8_t *__restrict__ flag, int32_t *__restrict__ owner,
-                                              const T *__restrict__ f, const int P, const int corr,
-                                              const uint8_t cur) {
-    if (CORR && corr) mark_corr_body<T>(L, pt, fcur, flag, owner, f, P, cur);
-    else mark_body(L, pt, fcur, flag, owner, cur);
+__global__ void __launch_bounds__(CORR ? 256 : kGeomThreads, CORR ? 4 : 2048 / kGeomThreads)
+    k_mark(const Lat L, const Parts pt, const SFrame *__restrict__ fcur, const SFrame *__restrict__ fprev,
+           uint8_t *__restrict__ flag, int32_t *__restrict__ owner, const T *__restrict__ f, const int P,
+           const uint8_t cur, const int full) {
+    if (CORR) mark_corr_body<T>(L, pt, fcur, flag, owner, f, P, cur);
+    else mark_body(L, pt, fcur, fprev, flag, owner, cur, full);
 }
 
 // Batched: instance blockIdx.y at step parity sp (also the population
@@ -271,7 +305,7 @@ __global__ void __launch_bounds__(256, CORR ? 4 : 8) k_mark_b(const Inst *__rest
     if ((int)blockIdx.x >= a.pt.np) return;
     const uint8_t cur = mark_value(sp);
     if (CORR && a.pt.corr) mark_corr_body<T>(a.L, a.pt, a.pt.frame[sp], a.flag, a.owner, (const T *)a.f, sp, cur);
-    else mark_body(a.L, a.pt, a.pt.frame[sp], a.flag, a.owner, cur);
+    else mark_body(a.L, a.pt, a.pt.frame[sp], a.pt.frame[sp ^ 1], a.flag, a.owner, cur, 0);
 }
 
 // One CTA per sphere: collect the uncovered nodes of its previous bounding
@@ -287,41 +321,57 @@ __device__ __forceinline__ void refill_body(const Lat &L, const SFrame *__restri
                                             const int P, unsigned long long *__restrict__ ctr,
                                             int *__restrict__ status, const Parts &pt, const uint8_t cur) {
     __shared__ int list[kRefillCap];
-    const uint8_t prev_mark = (uint8_t)(4 - cur);  // the other mark value: the previous step's geometry
     __shared__ int count;
     const int p = blockIdx.x;
     const SFrame Fp = fprev[p];  // the node geometry of the previous step was built from this centre
-    const int e = ext_of(Fp.R), B = 2 * e + 1;
+    const SFrame F = fcur[p];    // current centre, velocity and spin
+    const int e = ext_of(Fp.R);
     const int bx = Fp.b[0], by = Fp.b[1], bz = Fp.b[2];
     if (threadIdx.x == 0) count = 0;
     __syncthreads();
-    // the box is scanned kScanBatch offsets per thread at a time, their
-    // flags and owners loaded together (one memory round trip per batch)
-    constexpr int kScanBatch = 4;
-    const int B3 = B * B * B;
-    BoxWalk w(threadIdx.x, blockDim.x, B);
-    for (int t0 = threadIdx.x; t0 < B3; t0 += kScanBatch * blockDim.x) {
-        int n[kScanBatch];
+    auto take = [&](int n) {
+        const int k = atomicAdd(&count, 1);
+        if (k < kRefillCap) list[k] = n;
+        else atomicOr(status, ST_TILE);
+    };
+    if (CORR && pt.corr) {
+        const uint8_t prev_mark = (uint8_t)(4 - cur);  // the other mark value: the previous step's geometry
+        // the box is scanned kScanBatch offsets per thread at a time, their
+        // flags and owners loaded together (one memory round trip per batch)
+        constexpr int kScanBatch = 4;
+        const int B = 2 * e + 1, B3 = B * B * B;
+        BoxWalk w(threadIdx.x, blockDim.x, B);
+        for (int t0 = threadIdx.x; t0 < B3; t0 += kScanBatch * blockDim.x) {
+            int n[kScanBatch];
 #pragma unroll
-        for (int j = 0; j < kScanBatch; ++j) {
-            const int z = bz + w.oz - e;
-            const bool in = t0 + j * (int)blockDim.x < B3 && z >= 0 && z < L.nz;
-            n[j] = in ? wrapi(bx + w.ox - e, L.nx) + L.nx * (wrapi(by + w.oy - e, L.ny) + L.ny * z) : -1;
-            w.next();
+            for (int j = 0; j < kScanBatch; ++j) {
+                const int z = bz + w.oz - e;
+                const bool in = t0 + j * (int)blockDim.x < B3 && z >= 0 && z < L.nz;
+                n[j] = in ? wrapi(bx + w.ox - e, L.nx) + L.nx * (wrapi(by + w.oy - e, L.ny) + L.ny * z) : -1;
+                w.next();
+            }
+            uint8_t fl[kScanBatch];
+            int32_t ow[kScanBatch];
+#pragma unroll
+            for (int j = 0; j < kScanBatch; ++j) {
+                fl[j] = n[j] >= 0 ? flag[n[j]] : 0;
+                ow[j] = n[j] >= 0 ? owner[n[j]] : -1;
+            }
+#pragma unroll
+            for (int j = 0; j < kScanBatch; ++j)  // prev_mark is 1 or 3, never the 0 of a skipped offset
+                if (fl[j] == prev_mark && ow[j] == p) take(n[j]);
         }
-        uint8_t fl[kScanBatch];
-        int32_t ow[kScanBatch];
-#pragma unroll
-        for (int j = 0; j < kScanBatch; ++j) {
-            fl[j] = n[j] >= 0 ? flag[n[j]] : 0;
-            ow[j] = n[j] >= 0 ? owner[n[j]] : -1;
-        }
-#pragma unroll
-        for (int j = 0; j < kScanBatch; ++j) {
-            if (fl[j] != prev_mark || ow[j] != p) continue;  // prev_mark is 1 or 3, never the 0 of a skipped offset
-            const int k = atomicAdd(&count, 1);
-            if (k < kRefillCap) list[k] = n[j];
-            else atomicOr(status, ST_TILE);
+    } else {
+        // in the sphere at the previous centre, not at the current one, and
+        // still p's: then p owned it and no other sphere has taken it
+        const int E = 2 * e, E3 = E * E * E, lo = 1 - e;
+        const Shift d(L, Fp, F);
+        BoxWalk w(threadIdx.x, blockDim.x, E);
+        for (int t = threadIdx.x; t < E3; t += blockDim.x, w.next()) {
+            const int ox = w.ox + lo, oy = w.oy + lo, oz = w.oz + lo, z = bz + oz;
+            if (!inside(Fp, ox, oy, oz) || inside(F, ox + d.x, oy + d.y, oz + d.z) || z < 0 || z >= L.nz) continue;
+            const int n = wrapi(bx + ox, L.nx) + L.nx * (wrapi(by + oy, L.ny) + L.ny * z);
+            if ((flag[n] & 1) && owner[n] == p) take(n);
         }
     }
     __syncthreads();
@@ -349,7 +399,6 @@ __device__ __forceinline__ void refill_body(const Lat &L, const SFrame *__restri
     }
     const int total = min(count, kRefillCap);
     if (total == 0) return;
-    const SFrame F = fcur[p];  // current centre, velocity and spin, for the surface velocity
     const float *V = F.V, *W = F.W;
     const int lane = threadIdx.x & 31;
     __shared__ double wacc[8][6];  // with CORR, per warp: the momentum its refilled nodes take, in node order
@@ -566,31 +615,31 @@ int launch_near_mark(lbm_s *h, uint8_t *near, uint8_t tag, const SFrame *frames,
 }
 
 template <bool CORR>
-int mark_launch(lbm_s *h, int P, int corr) {
-    const SFrame *fcur = h->pt.frame[h->steps & 1];
+int mark_launch(lbm_s *h, int P, int full) {
+    const SFrame *fcur = h->pt.frame[h->steps & 1], *fprev = h->pt.frame[(h->steps + 1) & 1];
     const uint8_t cur = mark_value((int)(h->steps & 1));
     const dim3 g(h->pt.np);
     const int nt = CORR ? 256 : kGeomThreads;
     switch (h->precision) {
         case LBM_FP32:
-            k_mark<float, CORR><<<g, nt, 0, h->stream>>>(h->L, h->pt, fcur, h->flag, h->owner,
-                                                           (const float *)h->f, P, corr, cur);
+            k_mark<float, CORR><<<g, nt, 0, h->stream>>>(h->L, h->pt, fcur, fprev, h->flag, h->owner, (const float *)h->f,
+                                                         P, cur, full);
             break;
         case LBM_BF16_DEV:
-            k_mark<__nv_bfloat16, CORR><<<g, nt, 0, h->stream>>>(h->L, h->pt, fcur, h->flag, h->owner,
-                                                                   (const __nv_bfloat16 *)h->f, P, corr, cur);
+            k_mark<__nv_bfloat16, CORR><<<g, nt, 0, h->stream>>>(h->L, h->pt, fcur, fprev, h->flag, h->owner,
+                                                                 (const __nv_bfloat16 *)h->f, P, cur, full);
             break;
         case LBM_FP16_DEV:
-            k_mark<__half, CORR><<<g, nt, 0, h->stream>>>(h->L, h->pt, fcur, h->flag, h->owner,
-                                                            (const __half *)h->f, P, corr, cur);
+            k_mark<__half, CORR><<<g, nt, 0, h->stream>>>(h->L, h->pt, fcur, fprev, h->flag, h->owner,
+                                                          (const __half *)h->f, P, cur, full);
             break;
         default: return LBM_ERR_ARG;
     }
     return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
 }
 
-int launch_mark(lbm_s *h, int P, int corr) {
-    return corr ? mark_launch<true>(h, P, corr) : mark_launch<false>(h, P, 0);
+int launch_mark(lbm_s *h, int P, bool first) {
+    return h->pt.corr && !first ? mark_launch<true>(h, P, 0) : mark_launch<false>(h, P, first);
 }
 
 template <typename T, bool CORR>
