@@ -51,18 +51,37 @@ int dalloc(lbm_s *h, T **p, size_t n) {
     return LBM_OK;
 }
 
+// Requests that one allocation serves (each on a 256-byte boundary): a handle
+// has some forty small arrays, and every cudaMalloc costs its creation tens of
+// microseconds.
+struct Arena {
+    struct Req {
+        void **p;
+        size_t at;
+    };
+    std::vector<Req> reqs;
+    size_t total = 0;
+    template <class T>
+    void add(T **p, size_t n) {
+        *p = nullptr;
+        if (n == 0) return;
+        reqs.push_back({(void **)p, total});
+        total += (n * sizeof(T) + 255) & ~(size_t)255;
+    }
+    int make(lbm_s *h, unsigned char **base) {
+        const int rc = dalloc(h, base, total);
+        if (!rc)
+            for (const Req &r : reqs) *r.p = *base + r.at;
+        return rc;
+    }
+};
+
 void release(lbm_s *h) {
-    void *ptrs[] = {h->f, h->flag, h->owner, h->status, h->bar, h->ctr, h->pt.X, h->pt.V, h->pt.W, h->pt.R,
-                    (void *)h->pt.fixed, h->pt.Fh, h->pt.Th, h->pt.Fc, h->pt.Fx, h->pt.Tx, h->pt.Xf,
-                    h->pt.Xb[0], h->pt.Xb[1], h->pt.Vh[0], h->pt.Vh[1], h->pt.nbr, h->pt.nbr_cnt, h->pt.pairA,
-                    h->pt.pairB, h->pt.Xbuild, h->pt.rebuild, h->pt.frame[0], h->pt.frame[1], h->pt.Fcorr,
-                    h->pt.Tcorr, h->pt.Tc, h->pt.pairC, h->pt.tdisp, h->pt.tmask, h->pt.twall, h->zs, h->pt.pairBM, h->pt.nact, h->pt.isl_n, h->pt.isl8,
-                    h->pt.isl32, h->pt.big, h->pt.slot, h->pt.inv,
-                    h->xbuf,
-                    h->zpart, h->zcnt};
+    void *ptrs[] = {h->f, h->arena};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (h->status_host) cudaFreeHost(h->status_host);
+    if (h->state_host) cudaFreeHost(h->state_host);
     for (int k = 0; k < 2; ++k) {
         if (h->load_stage[k]) cudaFreeHost(h->load_stage[k]);
         if (h->load_ev[k]) cudaEventDestroy(h->load_ev[k]);
@@ -133,6 +152,19 @@ int settle(lbm_s *h) {
     return h->sticky;
 }
 
+// The same after work on the stream that has already left the status word in
+// status_host (the output kernels).
+int settle_posted(lbm_s *h) {
+    if (cudaStreamSynchronize(h->stream) != cudaSuccess) {
+        cudaGetLastError();
+        if (!h->sticky) h->sticky = LBM_ERR_CUDA;
+        return h->sticky;
+    }
+    const int c = status_to_code(*(volatile int *)h->status_host);
+    if (c && !h->sticky) h->sticky = c;
+    return h->sticky;
+}
+
 bool finite3(const double *v, int n) {
     for (int i = 0; i < 3 * n; ++i)
         if (!std::isfinite(v[i])) return false;
@@ -150,6 +182,47 @@ int copy_out(lbm_s *h, void *dst, const void *src, size_t n, int where) {
     if (n == 0 || !dst) return LBM_OK;
     const cudaMemcpyKind k = where == LBM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     return cudaMemcpyAsync(dst, src, n, k, h->stream) == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
+}
+
+// Pinned memory for the loads and state of all spheres: made with the handle
+// up to this many spheres, with the first host read beyond it.
+constexpr int kStateHostNow = 1 << 15;
+double *state_stage(lbm_s *h) {
+    if (!h->state_host &&
+        cudaMallocHost((void **)&h->state_host, 15 * sizeof(double) * (size_t)h->p.max_particles) != cudaSuccess) {
+        cudaGetLastError();
+        h->state_host = nullptr;
+    }
+    return h->state_host;
+}
+
+// F, T, X, V, Omega of the spheres to the caller's five arrays (any may be
+// null), then the stream settled.  Device arrays are written by one kernel
+// (a place that is not a whole double's needs the byte copies), host arrays
+// through pinned memory (without it, by pageable copies).
+int state_out(lbm_s *h, double *const *out, int where) {
+    const size_t n3 = 3 * (size_t)h->pt.np, v3 = n3 * sizeof(double);
+    bool any = false, whole = true;
+    for (int k = 0; k < 5; ++k) {
+        any = any || out[k];
+        whole = whole && ((uintptr_t)out[k] & 7) == 0;
+    }
+    if (!any || n3 == 0) return settle(h);
+    int rc = LBM_OK;
+    if (where == LBM_DEVICE ? !whole : !state_stage(h)) {
+        const double *src[5] = {h->pt.Fh, h->pt.Th, h->pt.X, h->pt.V, h->pt.W};
+        for (int k = 0; k < 5 && !rc; ++k) rc = copy_out(h, out[k], src[k], v3, where);
+        const int s = settle(h);
+        return rc ? rc : s;
+    }
+    double *to[5];
+    for (int k = 0; k < 5; ++k) to[k] = where == LBM_DEVICE ? out[k] : (out[k] ? h->state_host + n3 * k : nullptr);
+    rc = launch_state(h, to);
+    const int s = rc ? settle(h) : settle_posted(h);
+    if (!rc && where == LBM_HOST)
+        for (int k = 0; k < 5; ++k)
+            if (out[k]) std::memcpy(out[k], to[k], v3);
+    return rc ? rc : s;
 }
 
 // ZIEB cylinder at rest: rho = 1 and H_p = 0 in both parity slots, piston
@@ -318,71 +391,61 @@ int lbm_create(const lbm_params *prm, lbm_handle *out) {
     h->link_cap = link_capacity(M > 0 ? p.max_radius : 1.0);
 
     unsigned char *fixed = nullptr;
-    if (!rc) rc = dalloc(h, (unsigned char **)&h->f, (size_t)Q * h->L.S * h->esize);
-    if (!rc) rc = dalloc(h, &h->flag, (size_t)N + 16);  // the link kernel reads whole words
-    if (!rc) rc = dalloc(h, &h->owner, (size_t)N);
-    if (!rc) rc = dalloc(h, &h->status, 1);
-    if (!rc) rc = dalloc(h, &h->bar, 1);
-    if (!rc) rc = dalloc(h, &h->ctr, 4);
-    if (!rc) rc = dalloc(h, &pt.X, 3 * (size_t)M);
-    if (!rc) rc = dalloc(h, &pt.V, 3 * (size_t)M);
-    if (!rc) rc = dalloc(h, &pt.W, 3 * (size_t)M);
-    if (!rc) rc = dalloc(h, &pt.R, (size_t)M);
-    if (!rc) rc = dalloc(h, &fixed, (size_t)M);
-    pt.fixed = fixed;
-    if (!rc) rc = dalloc(h, &pt.inv, 2 * (size_t)M);
-    if (!rc) rc = dalloc(h, &pt.Fh, 3 * (size_t)M);
-    if (!rc) rc = dalloc(h, &pt.Th, 3 * (size_t)M);
-    if (!rc) rc = dalloc(h, &pt.Fc, 3 * (size_t)M);
-    if (!rc) rc = dalloc(h, &pt.Fx, 3 * (size_t)M);
-    if (!rc) rc = dalloc(h, &pt.Tx, 3 * (size_t)M);
-    if (!rc) rc = dalloc(h, &pt.Xbuild, 3 * (size_t)M);
-    if (!rc) rc = dalloc(h, &pt.rebuild, 2);
-    if (!rc) rc = dalloc(h, &pt.Fcorr, 3 * (size_t)M);
-    if (!rc) rc = dalloc(h, &pt.Tcorr, 3 * (size_t)M);
-    if (!rc) rc = dalloc(h, &pt.Tc, 3 * (size_t)M);
-    if (!rc && p.zieb) {
+    Arena a;
+    a.add(&h->flag, (size_t)N + 16);  // the link kernel reads whole words
+    a.add(&h->owner, (size_t)N);
+    a.add(&h->status, 1);
+    a.add(&h->bar, 1);
+    a.add(&h->ctr, 4);
+    double **d3[] = {&pt.X, &pt.V, &pt.W, &pt.Fh, &pt.Th, &pt.Fc, &pt.Fx, &pt.Tx, &pt.Xbuild, &pt.Fcorr, &pt.Tcorr, &pt.Tc,
+                     &pt.Xb[0], &pt.Xb[1], &pt.Vh[0], &pt.Vh[1]};
+    for (double **p3 : d3) a.add(p3, 3 * (size_t)M);
+    a.add(&pt.R, (size_t)M);
+    a.add(&fixed, (size_t)M);
+    a.add(&pt.inv, 2 * (size_t)M);
+    a.add(&pt.rebuild, 2);
+    if (p.zieb) {
         h->zieb = 1;
         h->zA = p.zieb_area;
         h->zV0 = p.zieb_volume;
         h->zblocks = (int)(((long long)p.nx * p.ny + 255) / 256);
-        rc = dalloc(h, &h->zs, 5);
-        if (!rc) rc = dalloc(h, &h->zpart, 2 * (size_t)h->zblocks);
-        if (!rc) rc = dalloc(h, &h->zcnt, 2 * (size_t)h->zblocks);
         h->zvp = p.zieb_piston_velocity;
-        if (!rc) rc = zieb_reset(h, h->zvp);
+        a.add(&h->zs, 5);
+        a.add(&h->zpart, 2 * (size_t)h->zblocks);
+        a.add(&h->zcnt, 2 * (size_t)h->zblocks);
     }
-    if (!rc && pt.fric) {
-        rc = dalloc(h, &pt.pairC, (size_t)M * kMaxNbr);
-        if (!rc) rc = dalloc(h, &pt.tdisp, (size_t)M * kMaxNbr);
-        if (!rc) rc = dalloc(h, &pt.tmask, (size_t)M);
-        if (!rc) rc = dalloc(h, &pt.twall, 2 * (size_t)M);
+    if (pt.fric) {
+        a.add(&pt.pairC, (size_t)M * kMaxNbr);
+        a.add(&pt.tdisp, (size_t)M * kMaxNbr);
+        a.add(&pt.tmask, (size_t)M);
+        a.add(&pt.twall, 2 * (size_t)M);
     }
     pt.corr = p.momentum_correction;
-    if (!rc) rc = dalloc(h, &pt.frame[0], (size_t)M);
-    if (!rc) rc = dalloc(h, &pt.frame[1], (size_t)M);
-    if (!rc) rc = dalloc(h, &pt.pairA, (size_t)M * kMaxNbr);
-    if (!rc) rc = dalloc(h, &pt.pairB, (size_t)M * kMaxNbr);
-    if (!rc) rc = dalloc(h, &pt.pairBM, (size_t)M * kMaxNbr);
-    if (!rc) rc = dalloc(h, &h->xbuf, 2 * 3 * (size_t)M);
-    if (!rc) rc = dalloc(h, &pt.nact, (size_t)M);
+    a.add(&pt.frame[0], (size_t)M);
+    a.add(&pt.frame[1], (size_t)M);
+    a.add(&pt.pairA, (size_t)M * kMaxNbr);
+    a.add(&pt.pairB, (size_t)M * kMaxNbr);
+    a.add(&pt.pairBM, (size_t)M * kMaxNbr);
+    a.add(&h->xbuf, 2 * 3 * (size_t)M);
+    a.add(&pt.nact, (size_t)M);
     // islands: at most M / 2 in groups of 8, M / 9 in warps
-    if (!rc) rc = dalloc(h, &pt.isl_n, 4);
-    if (!rc) rc = dalloc(h, &pt.isl8, 4 * (size_t)M + 32);
-    if (!rc) rc = dalloc(h, &pt.isl32, 4 * (size_t)M + 32);
-    if (!rc) rc = dalloc(h, &pt.big, (size_t)M);
-    if (!rc) rc = dalloc(h, &pt.slot, (size_t)M);
-    if (!rc) rc = dalloc(h, &pt.Xf, (size_t)M);
-    for (int b = 0; b < 2 && !rc; ++b) {
-        rc = dalloc(h, &pt.Xb[b], 3 * (size_t)M);
-        if (!rc) rc = dalloc(h, &pt.Vh[b], 3 * (size_t)M);
-    }
-    if (!rc) rc = dalloc(h, &pt.nbr, (size_t)M * kMaxNbr);
-    if (!rc) rc = dalloc(h, &pt.nbr_cnt, (size_t)M);
+    a.add(&pt.isl_n, 4);
+    a.add(&pt.isl8, 4 * (size_t)M + 32);
+    a.add(&pt.isl32, 4 * (size_t)M + 32);
+    a.add(&pt.big, (size_t)M);
+    a.add(&pt.slot, (size_t)M);
+    a.add(&pt.Xf, (size_t)M);
+    a.add(&pt.nbr, (size_t)M * kMaxNbr);
+    a.add(&pt.nbr_cnt, (size_t)M);
+    if (!rc) rc = dalloc(h, (unsigned char **)&h->f, (size_t)Q * h->L.S * h->esize);
+    if (!rc) rc = a.make(h, &h->arena);
+    pt.fixed = fixed;
+    if (!rc && p.zieb) rc = zieb_reset(h, h->zvp);
     if (!rc && cudaMallocHost((void **)&h->status_host, sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         rc = LBM_ERR_NOMEM;
     }
+    if (!rc && M > 0 && M <= kStateHostNow) state_stage(h);
     if (!rc && M > 0 && links_setup(h->tile_ext, h->link_cap) != LBM_OK) rc = LBM_ERR_CUDA;
     // overlapped schedule (spheres only): near tags, second stream, events
     h->overlap = M > 0 && p.schedule == LBM_SCHEDULE_OVERLAP;
@@ -591,15 +654,16 @@ int lbm_set_particle_load(lbm_handle h, const double *force, const double *torqu
         if (force) std::memcpy(stage, force, v3);
         if (torque) std::memcpy(stage + 3 * (size_t)h->pt.np, torque, v3);
     }
-    if (force)
-        rc = copy_in(h, h->pt.Fx, stage ? stage : force, v3, where);
-    else if (v3 && cudaMemsetAsync(h->pt.Fx, 0, v3, h->stream) != cudaSuccess)
-        rc = LBM_ERR_CUDA;
-    if (!rc) {
-        if (torque)
-            rc = copy_in(h, h->pt.Tx, stage ? stage + 3 * (size_t)h->pt.np : torque, v3, where);
-        else if (v3 && cudaMemsetAsync(h->pt.Tx, 0, v3, h->stream) != cudaSuccess)
-            rc = LBM_ERR_CUDA;
+    const double *F = stage && force ? stage : force;
+    const double *T = stage && torque ? stage + 3 * (size_t)h->pt.np : torque;
+    if (v3 && ((uintptr_t)F & 7) == 0 && ((uintptr_t)T & 7) == 0) {
+        rc = launch_load(h, F, T);
+    } else if (v3) {  // device arrays that do not start at a whole double
+        rc = F ? copy_in(h, h->pt.Fx, F, v3, where)
+               : (cudaMemsetAsync(h->pt.Fx, 0, v3, h->stream) == cudaSuccess ? LBM_OK : LBM_ERR_CUDA);
+        if (!rc)
+            rc = T ? copy_in(h, h->pt.Tx, T, v3, where)
+                   : (cudaMemsetAsync(h->pt.Tx, 0, v3, h->stream) == cudaSuccess ? LBM_OK : LBM_ERR_CUDA);
     }
     if (!rc && stage) {
         if (cudaEventRecord(h->load_ev[h->load_slot], h->stream) != cudaSuccess) rc = LBM_ERR_CUDA;
@@ -736,9 +800,7 @@ int lbm_step(lbm_handle h, int32_t nsteps) {
     if (!rc && parts && !ovl && !h->prof && nsteps >= 1 && h->stream) {
         if (h->graph_stale || !h->graph[0] || !h->graph[1]) rc = capture_step_graphs(h);
         for (int it = 0; it < nsteps && !rc; ++it) {
-            // the link / refill counters report the last step of the call
-            if (it == nsteps - 1) rc = ok(cudaMemsetAsync(h->ctr, 0, 2 * sizeof(unsigned long long), A));
-            if (!rc) rc = ok(cudaGraphLaunch(h->graph[h->parity], A));
+            rc = ok(cudaGraphLaunch(h->graph[h->parity], A));
             if (!rc) {
                 h->parity ^= 1;
                 ++h->steps;
@@ -754,7 +816,6 @@ int lbm_step(lbm_handle h, int32_t nsteps) {
         const long long s = h->steps;
         const int cur = (int)(s & 1), nxt = (int)((s + 1) & 1);
         if (h->prof && h->ev_used == h->ev_cap) rc = prof_flush(h);
-        if (!rc && it == nsteps - 1) rc = ok(cudaMemsetAsync(h->ctr, 0, 2 * sizeof(unsigned long long), A));
         if (ovl) {
             // second stream: the far-node collisions of step s, once the
             // near tags of step s exist (recorded after step s-1's near
@@ -818,36 +879,23 @@ int lbm_step(lbm_handle h, int32_t nsteps) {
 int lbm_forces(lbm_handle h, double *F, double *T, int32_t where) {
     if (!h || (where != LBM_HOST && where != LBM_DEVICE)) return LBM_ERR_ARG;
     DeviceScope ds(h->device);
-    const size_t v3 = 3 * sizeof(double) * (size_t)h->pt.np;
-    int rc = copy_out(h, F, h->pt.Fh, v3, where);
-    if (!rc) rc = copy_out(h, T, h->pt.Th, v3, where);
-    const int s = settle(h);
-    return rc ? rc : s;
+    double *const out[5] = {F, T, nullptr, nullptr, nullptr};
+    return state_out(h, out, where);
 }
 
 int lbm_particles(lbm_handle h, double *pos, double *vel, double *omega, int32_t where) {
     if (!h || (where != LBM_HOST && where != LBM_DEVICE)) return LBM_ERR_ARG;
     DeviceScope ds(h->device);
-    const size_t v3 = 3 * sizeof(double) * (size_t)h->pt.np;
-    int rc = copy_out(h, pos, h->pt.X, v3, where);
-    if (!rc) rc = copy_out(h, vel, h->pt.V, v3, where);
-    if (!rc) rc = copy_out(h, omega, h->pt.W, v3, where);
-    const int s = settle(h);
-    return rc ? rc : s;
+    double *const out[5] = {nullptr, nullptr, pos, vel, omega};
+    return state_out(h, out, where);
 }
 
 int lbm_particle_state(lbm_handle h, double *F, double *T, double *pos, double *vel, double *omega,
                        int32_t where) {
     if (!h || (where != LBM_HOST && where != LBM_DEVICE)) return LBM_ERR_ARG;
     DeviceScope ds(h->device);
-    const size_t v3 = 3 * sizeof(double) * (size_t)h->pt.np;
-    int rc = copy_out(h, F, h->pt.Fh, v3, where);
-    if (!rc) rc = copy_out(h, T, h->pt.Th, v3, where);
-    if (!rc) rc = copy_out(h, pos, h->pt.X, v3, where);
-    if (!rc) rc = copy_out(h, vel, h->pt.V, v3, where);
-    if (!rc) rc = copy_out(h, omega, h->pt.W, v3, where);
-    const int s = settle(h);
-    return rc ? rc : s;
+    double *const out[5] = {F, T, pos, vel, omega};
+    return state_out(h, out, where);
 }
 
 int lbm_fields(lbm_handle h, float *rho, float *u, int32_t where) {
@@ -868,7 +916,7 @@ int lbm_fields(lbm_handle h, float *rho, float *u, int32_t where) {
         if (!rc && u) rc = copy_out(h, u, tmp + N, 3 * sizeof(float) * (size_t)N, LBM_HOST);
         cudaFreeAsync(tmp, h->stream);
     }
-    const int s = settle(h);
+    const int s = rc ? settle(h) : settle_posted(h);
     return rc ? rc : s;
 }
 
@@ -877,7 +925,7 @@ int lbm_populations(lbm_handle h, double *f, int32_t where) {
     DeviceScope ds(h->device);
     const size_t n = (size_t)Q * h->L.N * sizeof(double);
     int rc = with_out_buffer(h, f, n, where, [&](void *d) { return launch_get_populations(h, (double *)d, h->parity); });
-    const int s = settle(h);
+    const int s = rc ? settle(h) : settle_posted(h);
     return rc ? rc : s;
 }
 
@@ -886,7 +934,7 @@ int lbm_geometry(lbm_handle h, int32_t *owner, int32_t where) {
     DeviceScope ds(h->device);
     const size_t n = (size_t)h->L.N * sizeof(int32_t);
     int rc = with_out_buffer(h, owner, n, where, [&](void *d) { return launch_owner(h, (int32_t *)d); });
-    const int s = settle(h);
+    const int s = rc ? settle(h) : settle_posted(h);
     return rc ? rc : s;
 }
 

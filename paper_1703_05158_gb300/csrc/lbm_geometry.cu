@@ -291,7 +291,8 @@ template <typename T, bool CORR>
 __global__ void __launch_bounds__(CORR ? 256 : kGeomThreads, CORR ? 4 : 2048 / kGeomThreads)
     k_mark(const Lat L, const Parts pt, const SFrame *__restrict__ fcur, const SFrame *__restrict__ fprev,
            uint8_t *__restrict__ flag, int32_t *__restrict__ owner, const T *__restrict__ f, const int P,
-           const uint8_t cur, const int full) {
+           const uint8_t cur, const int full, unsigned long long *__restrict__ ctr) {
+    if (blockIdx.x == 0 && threadIdx.x < 2) ctr[threadIdx.x] = 0ull;  // links and refilled nodes of this step
     if (CORR) mark_corr_body<T>(L, pt, fcur, flag, owner, f, P, cur);
     else mark_body(L, pt, fcur, fprev, flag, owner, cur, full);
 }
@@ -623,15 +624,15 @@ int mark_launch(lbm_s *h, int P, int full) {
     switch (h->precision) {
         case LBM_FP32:
             k_mark<float, CORR><<<g, nt, 0, h->stream>>>(h->L, h->pt, fcur, fprev, h->flag, h->owner, (const float *)h->f,
-                                                         P, cur, full);
+                                                         P, cur, full, h->ctr);
             break;
         case LBM_BF16_DEV:
             k_mark<__nv_bfloat16, CORR><<<g, nt, 0, h->stream>>>(h->L, h->pt, fcur, fprev, h->flag, h->owner,
-                                                                 (const __nv_bfloat16 *)h->f, P, cur, full);
+                                                                 (const __nv_bfloat16 *)h->f, P, cur, full, h->ctr);
             break;
         case LBM_FP16_DEV:
             k_mark<__half, CORR><<<g, nt, 0, h->stream>>>(h->L, h->pt, fcur, fprev, h->flag, h->owner,
-                                                          (const __half *)h->f, P, cur, full);
+                                                          (const __half *)h->f, P, cur, full, h->ctr);
             break;
         default: return LBM_ERR_ARG;
     }

@@ -260,10 +260,12 @@ struct lbm_s {
     int precision;
     size_t esize;  // bytes per stored population
     void *f;       // populations
+    unsigned char *arena;  // the allocation behind the other arrays
     uint8_t *flag;  // 0 fluid, 1 solid, 3 solid at the previous geometry, 2 refilled (see lbm_geometry.cu)
     int32_t *owner;
     int *status;             // device status word
     int *status_host;        // pinned mirror
+    double *state_host;      // pinned [5][max_particles][3]: loads and state on their way to the caller
     unsigned *bar;           // DEM grid-barrier counter
     unsigned long long *ctr; // [0] links, [1] refilled, [2] fluid-count scratch
     int parity;              // parity of the next step
@@ -397,6 +399,8 @@ int launch_set_populations(lbm_s *h, const double *f_dev, int parity);
 int launch_get_populations(lbm_s *h, double *f_dev, int parity);
 int launch_fields(lbm_s *h, float *rho, float *u, int parity);
 int launch_owner(lbm_s *h, int32_t *owner);
+int launch_state(lbm_s *h, double *const *out);  // F, T, X, V, Omega, each to out[k] (null: skipped)
+int launch_load(lbm_s *h, const double *F, const double *T);
 int launch_count_fluid(lbm_s *h);
 int dem_max_blocks(int threads, int *blocks_per_sm);
 int dem_cluster_setup(int max_particles, bool small = false, bool fric = false);
