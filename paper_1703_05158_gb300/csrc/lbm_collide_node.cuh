@@ -7,6 +7,18 @@
 
 namespace lbm {
 
+// c_i . v for a direction known at compile time: the zero components cost
+// nothing (a product with 0.f is an instruction the compiler must keep), and
+// what is left rounds as the full sum does.
+__device__ __forceinline__ float dot_c(const int i, const float x, const float y, const float z) {
+    float s = 0.f;
+    bool any = false;
+    if (cx(i)) s = cx(i) > 0 ? x : -x, any = true;
+    if (cy(i)) s = !any ? (cy(i) > 0 ? y : -y) : (cy(i) > 0 ? __fadd_rn(s, y) : __fsub_rn(s, y)), any = true;
+    if (cz(i)) s = !any ? (cz(i) > 0 ? z : -z) : (cz(i) > 0 ? __fadd_rn(s, z) : __fsub_rn(s, z)), any = true;
+    return s;
+}
+
 // Collision of one node (deviations in d, in place): rho (Eq. 5), the
 // force-shifted velocity (Eq. 6), Pi^neq and the Smagorinsky relaxation
 // time (Eq. 18), BGK relaxation towards Eq. (9) by opposite pairs, and the
@@ -15,7 +27,7 @@ namespace lbm {
 // __fmaf_rn), so the compiler cannot contract differently in different
 // kernels and a node gets bitwise the same result from any of them; the
 // products with lattice-vector components (0 or +-1) round the same either
-// way and are left to the compiler.
+// way (dot_c).
 __device__ __forceinline__ void collide_node(const Phys &ph, float (&d)[Q], int *status) {
     // moments from the sums and differences of opposite pairs (i, i + 9):
     // rho and the second moments take sp_i = d_i + d_i+9, the momentum
@@ -37,7 +49,7 @@ __device__ __forceinline__ void collide_node(const Phys &ph, float (&d)[Q], int 
     }
     const float rho = __fadd_rn(1.f, drho);
     if (!(rho > 0.f)) atomicOr(status, ST_DIVERGED);
-    const float ir = __fdiv_rn(1.f, rho);
+    const float ir = __frcp_rn(rho);
     const float ux = __fmaf_rn(jx, ir, 0.5f * ph.g[0]);  // g/2 is exact
     const float uy = __fmaf_rn(jy, ir, 0.5f * ph.g[1]);
     const float uz = __fmaf_rn(jz, ir, 0.5f * ph.g[2]);
@@ -67,7 +79,7 @@ __device__ __forceinline__ void collide_node(const Phys &ph, float (&d)[Q], int 
         const float inner = __fmaf_rn(__fmul_rn(ph.smag, __fsqrt_rn(q2)), ir, __fmul_rn(ph.tau0, ph.tau0));
         tau = __fmaf_rn(0.5f, __fsub_rn(__fsqrt_rn(inner), ph.tau0), ph.tau0);
     }
-    const float om = __fdiv_rn(1.f, tau);
+    const float om = __frcp_rn(tau);
 
     // Relaxation towards Eq. (9) (deviation form), by opposite pairs (i, i+9):
     // f^eq - w = w [drho + rho (4.5 (c.u)^2 - 1.5 u^2)]  +/-  3 w rho (c.u),
@@ -94,14 +106,14 @@ __device__ __forceinline__ void collide_node(const Phys &ph, float (&d)[Q], int 
     for (int i = 1; i <= 9; ++i) {
         const int k = i + 9;  // opp(i)
         const int c = w36(i) == 2 ? 0 : 1;
-        const float cu = cx(i) * ux + cy(i) * uy + cz(i) * uz;
+        const float cu = dot_c(i, ux, uy, uz);
         const float sym = __fmaf_rn(__fmul_rn(ow45[c], cu), cu, owb[c]);  // om (f^eq - w), even part
         const float asym = __fmul_rn(ow3[c], cu);                           // odd part
         d[i] = __fmaf_rn(keep, d[i], __fadd_rn(sym, asym));
         d[k] = __fmaf_rn(keep, d[k], __fsub_rn(sym, asym));
         if (forced) {
             // Guo source: w [3 (c - u).F + 9 (c.u)(c.F)], even and odd parts
-            const float cF = cx(i) * fx + cy(i) * fy + cz(i) * fz;
+            const float cF = dot_c(i, fx, fy, fz);
             const float skw = __fmul_rn(sk, wf(i));
             const float se = __fmul_rn(skw, __fmaf_rn(__fmul_rn(9.f, cu), cF, __fmul_rn(-3.f, uF)));
             const float so = __fmul_rn(__fmul_rn(3.f, skw), cF);
