@@ -20,6 +20,9 @@
 //
 // Roofline: HBM-bound.  Algorithmic traffic per fluid node and step is
 // 19 loads + 19 stores of the stored type plus one flag byte.
+#include <algorithm>
+
+#include "lbm_rows.cuh"
 #include "lbm_stream.cuh"
 
 namespace lbm {
@@ -92,6 +95,57 @@ __global__ void __launch_bounds__(256, 4) k_collide_list2(const Lat L, const Phy
     }
 }
 
+// Rows through shared memory (lbm_rows.cuh), three CTAs per SM of 256
+// consumers (two for buffers of 2 KB).  HBM-bound in FP32: 256^3 with 2000
+// spheres, us per launch at even / odd parity 394 / 394 (6.4 TB/s, 94% of a
+// copy) where a thread per node with global loads took 385 / 452; collide
+// phase 422 -> 396 us at 256^3, two CTAs 464, four (56 registers) 477.
+//
+// Where: the lattice has to exceed L2 (256x256x16, 80 MB: 26.6 us per step
+// node-wise, 28.7 by rows; x 24: 45.4 and 43.6; 128^3: 57.7 both) and whole
+// rows of 112 nodes or more fill 7/8 of a buffer (128x256x256: 213 -> 208,
+// 240x200x200 260 -> 253; four rows of 64: 106.6 -> 109.0, 160 of 256
+// nodes filled: 110.5 -> 130; one row of 512 in 2 KB buffers: 112.6 -> 159).
+// 16-bit storage is bound by instruction issue, and the pair kernel does the
+// conversions of two nodes from one word: at rows of 512 bytes it stays ahead
+// (297 us against 320 at four CTAs, 325 at three), at rows of 1 KB or more the
+// copies win (512x256x256 FP16: 613 against 700 us).
+constexpr long long kRowsFrom = 1ll << 21;
+constexpr int rows_minb(int pitch) { return pitch > 1024 ? 2 : 3; }
+constexpr int rows_smem(int pitch) { return 226 * 1024 / rows_minb(pitch) - 1536; }
+constexpr int kRowThreads = 256;  // consumers at most
+
+template <int ODD, typename T, int PITCH>
+__global__ void __launch_bounds__(kRowThreads + 32, rows_minb(PITCH))
+    k_collide_rows(const Lat L, const Phys ph, T *__restrict__ f, uint8_t *__restrict__ flag, int *__restrict__ status,
+                   const RowPlan pl) {
+    asm volatile("griddepcontrol.launch_dependents;");  // as in k_stream_collide
+    rows_body<ODD, T, PITCH>(
+        [&](int u) {
+            return RowUnit<T>(L, ph, f, flag, status, pl.dnx, pl.dpp, pl.per_plane, pl.rows, u);
+        },
+        pl.units, pl.stages, pl.consumers);
+}
+
+// The plan of a lattice whose rows can be copied whole (16-byte multiples)
+// and fill a buffer (see above), else stages = 0.
+static RowPlan rows_plan(const Lat &L, size_t esize) {
+    RowPlan p{};
+    const int bytes = L.nx * (int)esize, rows = std::max(1, kRowThreads / L.nx);
+    if (bytes % 16 != 0 || L.N < kRowsFrom) return p;
+    if (esize == 4 ? L.nx < 112 || rows * L.nx < 224 || L.nx > kRowThreads : bytes < 1024 || bytes > 2048) return p;
+    p.rows = std::min(rows, L.ny);
+    const int U = p.rows * L.nx, passes = (U + kRowThreads - 1) / kRowThreads;
+    p.consumers = ((U + passes - 1) / passes + 31) / 32 * 32;
+    p.pitch = U * (int)esize <= 1024 ? 1024 : 2048;
+    p.stages = std::min(kRowStages, rows_smem(p.pitch) / (Q * p.pitch));
+    p.per_plane = (L.ny + p.rows - 1) / p.rows;
+    p.units = p.per_plane * L.nz;
+    p.dpp = FastDiv((unsigned)p.per_plane);
+    p.dnx = FastDiv((unsigned)L.nx);
+    return p;
+}
+
 // Batched form: every node of every instance, one persistent launch.  Chunk
 // c = (instance, first node) covers TPB consecutive nodes of one instance
 // (a block's threads, coalesced); block b takes the contiguous chunk range
@@ -157,6 +211,23 @@ __global__ void __launch_bounds__(128, 8) k_stream_collide2(const Lat L, const P
     sc_pair<ODD, T>(L, ph, f, flag, status, xp, blockIdx.y, blockIdx.z);
 }
 
+template <int ODD, typename T, int PITCH>
+static int launch_rows_p(lbm_s *h, const RowPlan &p, cudaStream_t st) {
+    constexpr int kSmem = rows_smem(PITCH);
+    const auto k = k_collide_rows<ODD, T, PITCH>;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess) return LBM_ERR_CUDA;
+    const int grid = std::min(p.units, h->sms * rows_minb(PITCH));
+    k<<<grid, p.consumers + 32, p.stages * Q * PITCH, st>>>(h->L, h->ph, (T *)h->f, h->flag, h->status, p);
+    return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
+}
+
+template <int ODD, typename T>
+static int launch_rows(lbm_s *h, const RowPlan &p, cudaStream_t st) {
+    if constexpr (sizeof(T) == 2)
+        if (p.pitch == 2048) return launch_rows_p<ODD, T, 2048>(h, p, st);
+    return launch_rows_p<ODD, T, 1024>(h, p, st);
+}
+
 template <int ODD, typename T>
 static int launch_sc(lbm_s *h, cudaStream_t st) {
     const int bx = h->L.nx >= 256 ? 256 : ((h->L.nx + 31) / 32) * 32;
@@ -176,6 +247,8 @@ static int launch_sc2(lbm_s *h, cudaStream_t st) {
 
 template <int ODD, typename T>
 static int launch_parity(lbm_s *h, cudaStream_t st) {
+    const RowPlan p = rows_plan(h->L, sizeof(T));
+    if (p.stages >= 2) return launch_rows<ODD, T>(h, p, st);
     if constexpr (sizeof(T) == 2) {
         if ((h->L.nx % 2) == 0) return launch_sc2<ODD, T>(h, st);
     }
