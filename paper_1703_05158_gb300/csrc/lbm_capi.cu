@@ -434,6 +434,8 @@ int lbm_create(const lbm_params *prm, lbm_handle *out) {
     a.add(&pt.isl32, 4 * (size_t)M + 32);
     a.add(&pt.big, (size_t)M);
     a.add(&pt.slot, (size_t)M);
+    a.add(&pt.order, (size_t)M);
+    a.add(&pt.order_new, (size_t)M);
     a.add(&pt.Xf, (size_t)M);
     a.add(&pt.nbr, (size_t)M * kMaxNbr);
     a.add(&pt.nbr_cnt, (size_t)M);

@@ -118,7 +118,7 @@ __device__ __forceinline__ void neighbours_body(const Lat &L, const Parts &pt, c
         }
         float4 me = live ? pt.Xf[a] : make_float4(0.f, 0.f, 0.f, 0.f);
         const float hx = 0.5f * L.nx, hy = 0.5f * L.ny;
-        int cnt = 0;
+        int cnt = 0, above = 0;
         for (int t0 = 0; t0 < pt.np; t0 += kNbrTile) {
             const int tn = min(kNbrTile, pt.np - t0);
             __syncthreads();
@@ -130,6 +130,7 @@ __device__ __forceinline__ void neighbours_body(const Lat &L, const Parts &pt, c
                 bool ok = false;
                 if (i < tn && b != a) {
                     const float4 o = tile[i];
+                    above += o.z > me.z || (o.z == me.z && b < a);  // rank in descending z
                     float dx = me.x - o.x, dy = me.y - o.y;
                     const float dz = me.z - o.z;
                     if (dx > hx) dx -= L.nx;
@@ -147,7 +148,9 @@ __device__ __forceinline__ void neighbours_body(const Lat &L, const Parts &pt, c
                 cnt += __popc(m);
             }
         }
+        above = __reduce_add_sync(0xffffffffu, above);
         if (live && lane == 0) {
+            pt.order_new[above] = a;  // the ranks of distinct (z, id) are a permutation
             pt.nbr_cnt[a] = min(cnt, pt.max_nbr);
             if (cnt > pt.max_nbr) atomicOr(status, ST_NBR_OVERFLOW);
         }
@@ -314,6 +317,7 @@ __global__ void k_contact(const Lat L, const Parts pt) {
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= pt.np) return;
     const double m = sphere_mass(pt, a), R = pt.R[a];
+    pt.order[a] = pt.order_new[a];
     pt.inv[2 * a] = 1.0 / m;  // an FP64 divide costs a sub-step; the masses do not change
     pt.inv[2 * a + 1] = 1.0 / (0.4 * m * R * R);
     double F[3], T[3] = {0.0, 0.0, 0.0};
@@ -855,8 +859,10 @@ __global__ void __launch_bounds__(kDemThreads) k_dem_local(const Lat L, const Pa
         dem_one<FRIC, true>(L, pt, fnext, sp, status, a, lane, buf);
         __syncwarp();
     }
-    for (int a = G - 1 - g0; a < pt.np; a += G)
+    for (int a = G - 1 - g0; a < pt.np; a += G) {
+        pt.order[a] = pt.order_new[a];
         if (pt.nact[a] == 0) dem_one<FRIC, false>(L, pt, fnext, sp, status, a, lane, buf);
+    }
     if (CL && nbig > 0 && (int)blockIdx.x < ctas) {
         __syncthreads();  // the islands' buffers are free
         dem_wide<FRIC, false, true>(L, pt, fnext, sp, status, nbig, ctas);
@@ -899,6 +905,8 @@ __global__ void __launch_bounds__(kDemThreads, 1) k_dem_cluster_b(const Inst *__
     const Inst &a = I[blockIdx.y];
     if (a.pt.np == 0) return;  // the whole cluster (one instance) leaves together
     if (blockIdx.x == 0 && threadIdx.x == 0) a.pt.rebuild[sp] = 0;
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < a.pt.np; k += gridDim.x * blockDim.x)
+        a.pt.order[k] = a.pt.order_new[k];
     SFrame *fnext = a.pt.frame[sp ^ 1];
     if (FRIC && !a.pt.fric) dem_wide<false, false, false>(a.L, a.pt, fnext, sp, a.status, a.pt.np, gridDim.x);
     else dem_wide<FRIC, false, false>(a.L, a.pt, fnext, sp, a.status, a.pt.np, gridDim.x);

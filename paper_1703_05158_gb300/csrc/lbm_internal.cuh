@@ -198,6 +198,7 @@ struct Parts {
     // islands of the step (k_islands): counts of 8-lane groups, warps and big spheres; their members
     // (-1: an idle lane); a member's lane or place in `big`
     int *isl_n, *isl8, *isl32, *big, *slot;
+    int *order, *order_new;        // [np] spheres by z at the last list build (this step's, the next step's)
     double *Xbuild;                // centres when the lists were built
     int *rebuild;                  // [2]: rebuild[s & 1] = 1 asks the neighbour pass of step s to rebuild
     SFrame *frame[2];              // frames of the centres of even / odd steps

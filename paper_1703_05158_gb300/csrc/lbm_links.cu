@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(256, LBM_LINK_MINB) k_links(const Lat L, const
                                                uint8_t *__restrict__ flag, const int32_t *__restrict__ owner,
                                                const int P, const int ext, const int cap, int *__restrict__ status,
                                                unsigned long long *__restrict__ ctr) {
-    links_body<T, GI, LBM_LINK_BATCH>(L, pt, fcur, f, flag, owner, P, ext, cap, status, ctr, blockIdx.x);
+    links_body<T, GI, LBM_LINK_BATCH>(L, pt, fcur, f, flag, owner, P, ext, cap, status, ctr, pt.order[blockIdx.x]);
 }
 
 // Batched: instance blockIdx.y; parity P is also the step parity.
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(256, LBM_LINK_B_MINB) k_links_b(const Inst *__
     const Inst &a = I[blockIdx.y];
     if ((int)blockIdx.x >= a.pt.np) return;
     links_body<T, GI, LBM_LINK_B_BATCH>(a.L, a.pt, a.pt.frame[P], (T *)a.f, a.flag, a.owner, P, ext, cap, a.status,
-                                        a.ctr, blockIdx.x);
+                                        a.ctr, a.pt.order[blockIdx.x]);
 }
 
 int link_capacity(double max_radius) {
