@@ -41,12 +41,12 @@ namespace lbm {
 #endif
 template <int ODD, typename T>
 __global__ void __launch_bounds__(256, ODD ? LBM_SC_MINB_ODD : LBM_SC_MINB_EVEN) k_stream_collide(const Lat L, const Phys ph, T *__restrict__ f,
-                                                        uint8_t *__restrict__ flag, int *__restrict__ status) {
+                                                        uint8_t *__restrict__ flag, int *__restrict__ status, const int down) {
     // a programmatic dependent (the link kernel) may launch once every block
     // has started; it waits for this grid's completion before its reads
     asm volatile("griddepcontrol.launch_dependents;");
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y, z = blockIdx.z;
+    const int y = blockIdx.y, z = down ? L.nz - 1 - (int)blockIdx.z : (int)blockIdx.z;
     if (x >= L.nx) return;
     const int row = y + L.ny * z;
     const int n = x + L.nx * row;
@@ -118,11 +118,12 @@ constexpr int kRowThreads = 256;  // consumers at most
 template <int ODD, typename T, int PITCH>
 __global__ void __launch_bounds__(kRowThreads + 32, rows_minb(PITCH))
     k_collide_rows(const Lat L, const Phys ph, T *__restrict__ f, uint8_t *__restrict__ flag, int *__restrict__ status,
-                   const RowPlan pl) {
+                   const RowPlan pl, const int down) {
     asm volatile("griddepcontrol.launch_dependents;");  // as in k_stream_collide
     rows_body<ODD, T, PITCH>(
         [&](int u) {
-            return RowUnit<T>(L, ph, f, flag, status, pl.dnx, pl.dpp, pl.per_plane, pl.rows, u);
+            return RowUnit<T>(L, ph, f, flag, status, pl.dnx, pl.dpp, pl.per_plane, pl.rows,
+                              down ? pl.units - 1 - u : u);
         },
         pl.units, pl.stages, pl.consumers);
 }
@@ -204,11 +205,24 @@ __global__ void __launch_bounds__(TPB, MINB) k_collide_batch_tab(const __grid_co
 // 16-bit storage: two nodes per thread (sc_pair).  Requires even nx.
 template <int ODD, typename T>
 __global__ void __launch_bounds__(128, 8) k_stream_collide2(const Lat L, const Phys ph, T *__restrict__ f,
-                                                            uint8_t *__restrict__ flag, int *__restrict__ status) {
+                                                            uint8_t *__restrict__ flag, int *__restrict__ status,
+                                                            const int down) {
     asm volatile("griddepcontrol.launch_dependents;");  // as in k_stream_collide
     const int xp = blockIdx.x * blockDim.x + threadIdx.x;
     if (xp >= (L.nx >> 1)) return;
-    sc_pair<ODD, T>(L, ph, f, flag, status, xp, blockIdx.y, blockIdx.z);
+    sc_pair<ODD, T>(L, ph, f, flag, status, xp, blockIdx.y, down ? L.nz - 1 - (int)blockIdx.z : (int)blockIdx.z);
+}
+
+// Whether the collide of this parity goes through the planes from the top
+// down: the planes the step before ended with are still in L2.  Us per step
+// one way / alternating: 201x150x101 91.8 / 81.1, 160^3 110.5 / 101.2, 256^3
+// 404 / 401, 256^3 BF16 312 / 308; lattices that fit L2 the same.  The link
+// kernel in between takes L2 for its own scattered blocks (158 bytes per
+// link): 160^3 with 400 spheres 158.7 / 155.7, 256^3 with 2000 533.6 / 534.8,
+// so the sweep alternates while that is less than L2.
+static int sweep_down(const lbm_s *h, int parity) {
+    const double r = h->p.max_radius, link_bytes = h->pt.np * 72.0 * r * r * 158.0;
+    return parity && link_bytes < 120e6;
 }
 
 template <int ODD, typename T, int PITCH>
@@ -217,7 +231,7 @@ static int launch_rows_p(lbm_s *h, const RowPlan &p, cudaStream_t st) {
     const auto k = k_collide_rows<ODD, T, PITCH>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess) return LBM_ERR_CUDA;
     const int grid = std::min(p.units, h->sms * rows_minb(PITCH));
-    k<<<grid, p.consumers + 32, p.stages * Q * PITCH, st>>>(h->L, h->ph, (T *)h->f, h->flag, h->status, p);
+    k<<<grid, p.consumers + 32, p.stages * Q * PITCH, st>>>(h->L, h->ph, (T *)h->f, h->flag, h->status, p, sweep_down(h, ODD));
     return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
 }
 
@@ -232,7 +246,7 @@ template <int ODD, typename T>
 static int launch_sc(lbm_s *h, cudaStream_t st) {
     const int bx = h->L.nx >= 256 ? 256 : ((h->L.nx + 31) / 32) * 32;
     dim3 grid((h->L.nx + bx - 1) / bx, h->L.ny, h->L.nz);
-    k_stream_collide<ODD, T><<<grid, bx, 0, st>>>(h->L, h->ph, (T *)h->f, h->flag, h->status);
+    k_stream_collide<ODD, T><<<grid, bx, 0, st>>>(h->L, h->ph, (T *)h->f, h->flag, h->status, sweep_down(h, ODD));
     return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
 }
 
@@ -241,7 +255,7 @@ static int launch_sc2(lbm_s *h, cudaStream_t st) {
     const int hx = h->L.nx / 2;
     const int bx = hx >= 128 ? 128 : ((hx + 31) / 32) * 32;
     dim3 grid((hx + bx - 1) / bx, h->L.ny, h->L.nz);
-    k_stream_collide2<ODD, T><<<grid, bx, 0, st>>>(h->L, h->ph, (T *)h->f, h->flag, h->status);
+    k_stream_collide2<ODD, T><<<grid, bx, 0, st>>>(h->L, h->ph, (T *)h->f, h->flag, h->status, sweep_down(h, ODD));
     return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
 }
 
