@@ -706,24 +706,36 @@ namespace {
 int serial_step_launches(lbm_s *h) {
     const int P = h->parity;
     auto ok = [](cudaError_t e) { return e == cudaSuccess ? LBM_OK : LBM_ERR_CUDA; };
-    int rc = launch_mark(h, P);
+    int rc = launch_mark(h, P, false, true);
     if (!rc) rc = ok(cudaEventRecord(h->ev_fork, h->stream));
     if (!rc) rc = ok(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
     if (!rc) rc = launch_neighbours(h, 0, h->side);
     if (!rc) rc = ok(cudaEventRecord(h->ev_nbr, h->side));
-    if (!rc) rc = launch_refill(h, P);
-    if (!rc) rc = launch_stream_collide(h, P);
-    if (!rc) rc = launch_links(h, P, true);
+    if (!rc) rc = launch_refill(h, P, true);
+    if (!rc) rc = launch_stream_collide(h, P, true);
+    // the row form fills the registers to its last block: nothing to overlap
+    // with (with every launch programmatic 256^3 with 2000 spheres took 639 us
+    // per step, with this one ordinary 527, with only this one so 532)
+    if (!rc) rc = launch_links(h, P, !collides_by_rows(h));
     if (!rc && h->zieb) rc = launch_zieb(h, P);
     if (!rc) rc = ok(cudaStreamWaitEvent(h->stream, h->ev_nbr, 0));
-    if (!rc) rc = launch_dem(h);
+    if (!rc) rc = launch_dem(h, true);
     return rc;
 }
 
-// Capture the serial step of each parity into a graph (the launchers read
-// the parity and the step parity from the handle, so both are set for the
-// capture and restored).
-int capture_step_graphs(lbm_s *h) {
+void drop_step_graphs(lbm_s *h) {
+    for (cudaGraphExec_t &g : h->graph)
+        if (g) {
+            cudaGraphExecDestroy(g);
+            g = nullptr;
+        }
+}
+
+// Capture graph k: one serial step from parity k (k < 2), or two from parity
+// 0, whose second one starts without the gap between two graphs (the
+// launchers read the parity and the step parity from the handle, so both are
+// set for the capture and restored).
+int capture_step_graph(lbm_s *h, int k) {
     if (!h->side) {
         if (cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
@@ -732,42 +744,30 @@ int capture_step_graphs(lbm_s *h) {
             return LBM_ERR_CUDA;
         }
     }
-    for (cudaGraphExec_t &g : h->graph)
-        if (g) {
-            cudaGraphExecDestroy(g);
-            g = nullptr;
-        }
     const int P0 = h->parity;
     const long long s0 = h->steps;
-    int rc = LBM_OK;
-    for (int k = 0; k < 2 && !rc; ++k) {
-        const int P = P0 ^ k;
+    int rc = LBM_OK, r = LBM_OK;
+    cudaGraph_t g = nullptr;
+    if (cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+        cudaGetLastError();
+        return LBM_ERR_CUDA;
+    }
+    for (int P = k & 1; P <= (k == 2 ? 1 : k) && !r; ++P) {
         h->parity = P;
-        h->steps = s0 + k;
-        cudaGraph_t g = nullptr;
-        if (cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-            rc = LBM_ERR_CUDA;
-            break;
-        }
-        const int r = serial_step_launches(h);
-        const cudaError_t e = cudaStreamEndCapture(h->stream, &g);
-        if (r || e != cudaSuccess) rc = r ? r : LBM_ERR_CUDA;
-        if (!rc && cudaGraphInstantiate(&h->graph[P], g, 0) != cudaSuccess) rc = LBM_ERR_CUDA;
-        if (g) cudaGraphDestroy(g);
+        h->steps = P;  // the step parity is the parity
+        r = serial_step_launches(h);
     }
     h->parity = P0;
     h->steps = s0;
+    const cudaError_t e = cudaStreamEndCapture(h->stream, &g);
+    if (r || e != cudaSuccess) rc = r ? r : LBM_ERR_CUDA;
+    if (!rc && cudaGraphInstantiate(&h->graph[k], g, 0) != cudaSuccess) rc = LBM_ERR_CUDA;
+    if (g) cudaGraphDestroy(g);
     if (rc) {
         cudaGetLastError();
-        for (cudaGraphExec_t &g : h->graph)
-            if (g) {
-                cudaGraphExecDestroy(g);
-                g = nullptr;
-            }
-        return rc;
+        drop_step_graphs(h);
     }
-    h->graph_stale = false;
-    return LBM_OK;
+    return rc;
 }
 
 }  // namespace
@@ -800,12 +800,16 @@ int lbm_step(lbm_handle h, int32_t nsteps) {
     // are kept until the spheres are set again, so single steps replay them
     // too).
     if (!rc && parts && !ovl && !h->prof && nsteps >= 1 && h->stream) {
-        if (h->graph_stale || !h->graph[0] || !h->graph[1]) rc = capture_step_graphs(h);
-        for (int it = 0; it < nsteps && !rc; ++it) {
-            rc = ok(cudaGraphLaunch(h->graph[h->parity], A));
+        if (h->graph_stale) drop_step_graphs(h);
+        h->graph_stale = false;
+        for (int left = nsteps; left > 0 && !rc;) {
+            const int k = h->parity == 0 && left >= 2 ? 2 : h->parity, n = k == 2 ? 2 : 1;
+            if (!h->graph[k]) rc = capture_step_graph(h, k);
+            if (!rc) rc = ok(cudaGraphLaunch(h->graph[k], A));
             if (!rc) {
-                h->parity ^= 1;
-                ++h->steps;
+                h->parity ^= n & 1;
+                h->steps += n;
+                left -= n;
             }
         }
         nsteps = 0;  // done

@@ -42,9 +42,10 @@ namespace lbm {
 template <int ODD, typename T>
 __global__ void __launch_bounds__(256, ODD ? LBM_SC_MINB_ODD : LBM_SC_MINB_EVEN) k_stream_collide(const Lat L, const Phys ph, T *__restrict__ f,
                                                         uint8_t *__restrict__ flag, int *__restrict__ status, const int down) {
-    // a programmatic dependent (the link kernel) may launch once every block
-    // has started; it waits for this grid's completion before its reads
-    asm volatile("griddepcontrol.launch_dependents;");
+    // the link kernel reads the marks before its wait: it may start once every
+    // block here has seen the refill (and so the marks) complete
+    step_wait();
+    step_next();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y, z = down ? L.nz - 1 - (int)blockIdx.z : (int)blockIdx.z;
     if (x >= L.nx) return;
@@ -119,7 +120,8 @@ template <int ODD, typename T, int PITCH>
 __global__ void __launch_bounds__(kRowThreads + 32, rows_minb(PITCH))
     k_collide_rows(const Lat L, const Phys ph, T *__restrict__ f, uint8_t *__restrict__ flag, int *__restrict__ status,
                    const RowPlan pl, const int down) {
-    asm volatile("griddepcontrol.launch_dependents;");  // as in k_stream_collide
+    step_wait();  // as in k_stream_collide
+    step_next();
     rows_body<ODD, T, PITCH>(
         [&](int u) {
             return RowUnit<T>(L, ph, f, flag, status, pl.dnx, pl.dpp, pl.per_plane, pl.rows,
@@ -207,7 +209,8 @@ template <int ODD, typename T>
 __global__ void __launch_bounds__(128, 8) k_stream_collide2(const Lat L, const Phys ph, T *__restrict__ f,
                                                             uint8_t *__restrict__ flag, int *__restrict__ status,
                                                             const int down) {
-    asm volatile("griddepcontrol.launch_dependents;");  // as in k_stream_collide
+    step_wait();  // as in k_stream_collide
+    step_next();
     const int xp = blockIdx.x * blockDim.x + threadIdx.x;
     if (xp >= (L.nx >> 1)) return;
     sc_pair<ODD, T>(L, ph, f, flag, status, xp, blockIdx.y, down ? L.nz - 1 - (int)blockIdx.z : (int)blockIdx.z);
@@ -226,60 +229,69 @@ static int sweep_down(const lbm_s *h, int parity) {
 }
 
 template <int ODD, typename T, int PITCH>
-static int launch_rows_p(lbm_s *h, const RowPlan &p, cudaStream_t st) {
+static int launch_rows_p(lbm_s *h, const RowPlan &p, bool pdl) {
     constexpr int kSmem = rows_smem(PITCH);
     const auto k = k_collide_rows<ODD, T, PITCH>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess) return LBM_ERR_CUDA;
     const int grid = std::min(p.units, h->sms * rows_minb(PITCH));
-    k<<<grid, p.consumers + 32, p.stages * Q * PITCH, st>>>(h->L, h->ph, (T *)h->f, h->flag, h->status, p, sweep_down(h, ODD));
-    return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
+    return launch_step(k, dim3(grid), dim3(p.consumers + 32), p.stages * Q * PITCH, h->stream, pdl, h->L, h->ph, (T *)h->f,
+                       h->flag, h->status, p, sweep_down(h, ODD)) == cudaSuccess
+               ? LBM_OK
+               : LBM_ERR_CUDA;
 }
 
 template <int ODD, typename T>
-static int launch_rows(lbm_s *h, const RowPlan &p, cudaStream_t st) {
+static int launch_rows(lbm_s *h, const RowPlan &p, bool pdl) {
     if constexpr (sizeof(T) == 2)
-        if (p.pitch == 2048) return launch_rows_p<ODD, T, 2048>(h, p, st);
-    return launch_rows_p<ODD, T, 1024>(h, p, st);
+        if (p.pitch == 2048) return launch_rows_p<ODD, T, 2048>(h, p, pdl);
+    return launch_rows_p<ODD, T, 1024>(h, p, pdl);
 }
 
 template <int ODD, typename T>
-static int launch_sc(lbm_s *h, cudaStream_t st) {
+static int launch_sc(lbm_s *h, bool pdl) {
     const int bx = h->L.nx >= 256 ? 256 : ((h->L.nx + 31) / 32) * 32;
-    dim3 grid((h->L.nx + bx - 1) / bx, h->L.ny, h->L.nz);
-    k_stream_collide<ODD, T><<<grid, bx, 0, st>>>(h->L, h->ph, (T *)h->f, h->flag, h->status, sweep_down(h, ODD));
-    return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
+    const dim3 grid((h->L.nx + bx - 1) / bx, h->L.ny, h->L.nz);
+    return launch_step(k_stream_collide<ODD, T>, grid, dim3(bx), 0, h->stream, pdl, h->L, h->ph, (T *)h->f, h->flag,
+                       h->status, sweep_down(h, ODD)) == cudaSuccess
+               ? LBM_OK
+               : LBM_ERR_CUDA;
 }
 
 template <int ODD, typename T>
-static int launch_sc2(lbm_s *h, cudaStream_t st) {
+static int launch_sc2(lbm_s *h, bool pdl) {
     const int hx = h->L.nx / 2;
     const int bx = hx >= 128 ? 128 : ((hx + 31) / 32) * 32;
-    dim3 grid((hx + bx - 1) / bx, h->L.ny, h->L.nz);
-    k_stream_collide2<ODD, T><<<grid, bx, 0, st>>>(h->L, h->ph, (T *)h->f, h->flag, h->status, sweep_down(h, ODD));
-    return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
+    const dim3 grid((hx + bx - 1) / bx, h->L.ny, h->L.nz);
+    return launch_step(k_stream_collide2<ODD, T>, grid, dim3(bx), 0, h->stream, pdl, h->L, h->ph, (T *)h->f, h->flag,
+                       h->status, sweep_down(h, ODD)) == cudaSuccess
+               ? LBM_OK
+               : LBM_ERR_CUDA;
 }
 
 template <int ODD, typename T>
-static int launch_parity(lbm_s *h, cudaStream_t st) {
+static int launch_parity(lbm_s *h, bool pdl) {
     const RowPlan p = rows_plan(h->L, sizeof(T));
-    if (p.stages >= 2) return launch_rows<ODD, T>(h, p, st);
+    if (p.stages >= 2) return launch_rows<ODD, T>(h, p, pdl);
     if constexpr (sizeof(T) == 2) {
-        if ((h->L.nx % 2) == 0) return launch_sc2<ODD, T>(h, st);
+        if ((h->L.nx % 2) == 0) return launch_sc2<ODD, T>(h, pdl);
     }
-    return launch_sc<ODD, T>(h, st);
+    return launch_sc<ODD, T>(h, pdl);
 }
 
 template <typename T>
-static int launch_type(lbm_s *h, int parity, cudaStream_t st) {
-    return parity ? launch_parity<1, T>(h, st) : launch_parity<0, T>(h, st);
+static int launch_type(lbm_s *h, int parity, bool pdl) {
+    const int rc = parity ? launch_parity<1, T>(h, pdl) : launch_parity<0, T>(h, pdl);
+    if (rc) cudaGetLastError();
+    return rc;
 }
 
-int launch_stream_collide(lbm_s *h, int parity, cudaStream_t stream) {
-    cudaStream_t st = stream ? stream : h->stream;
+bool collides_by_rows(const lbm_s *h) { return rows_plan(h->L, h->esize).stages >= 2; }
+
+int launch_stream_collide(lbm_s *h, int parity, bool pdl) {
     switch (h->precision) {
-        case LBM_FP32: return launch_type<float>(h, parity, st);
-        case LBM_BF16_DEV: return launch_type<__nv_bfloat16>(h, parity, st);
-        case LBM_FP16_DEV: return launch_type<__half>(h, parity, st);
+        case LBM_FP32: return launch_type<float>(h, parity, pdl);
+        case LBM_BF16_DEV: return launch_type<__nv_bfloat16>(h, parity, pdl);
+        case LBM_FP16_DEV: return launch_type<__half>(h, parity, pdl);
     }
     return LBM_ERR_ARG;
 }

@@ -847,6 +847,8 @@ __global__ void __launch_bounds__(kDemThreads) k_dem_local(const Lat L, const Pa
     constexpr int S = FRIC ? 3 : 2;
     extern __shared__ float4 dsm[];
     const int G = gridDim.x * blockDim.x, g0 = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    step_next();
+    step_wait();
     if (g0 == 0) {
         pt.rebuild[sp] = 0;
         *bar = 0u;  // for the grid form's kernel, which follows
@@ -1127,7 +1129,7 @@ static int launch_dem_grid(lbm_s *h, SFrame *fnext, int sp) {
     return e == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
 }
 
-int launch_dem(lbm_s *h) {
+int launch_dem(lbm_s *h, bool pdl) {
     Lat L = h->L;
     Parts pt = h->pt;
     int *status = h->status;
@@ -1144,17 +1146,19 @@ int launch_dem(lbm_s *h) {
         const int want = (pt.np + kDemThreads - 1) / kDemThreads + std::min(64, pt.np / (2 * kDemThreads / 8));
         const bool fric = pt.fric != 0;
         cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = cl;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = pdl;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = cl;
+        attr[1].val.clusterDim.y = 1;
+        attr[1].val.clusterDim.z = 1;
         cfg.gridDim = dim3((want + cl - 1) / cl * cl);
         cfg.blockDim = dim3(kDemThreads);
         cfg.dynamicSmemBytes = grid ? dem_island_smem(fric) : dem_cluster_smem(fric);
         cfg.stream = h->stream;
         cfg.attrs = attr;
-        cfg.numAttrs = grid ? 0 : 1;
+        cfg.numAttrs = grid ? 1 : 2;
         const auto k = grid ? (fric ? k_dem_local<true, false> : k_dem_local<false, false>)
                             : (fric ? k_dem_local<true, true> : k_dem_local<false, true>);
         const cudaError_t e = cudaLaunchKernelEx(&cfg, k, L, pt, fnext, sp, status, cl, h->bar);

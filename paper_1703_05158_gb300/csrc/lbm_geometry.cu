@@ -292,6 +292,8 @@ __global__ void __launch_bounds__(CORR ? 256 : kGeomThreads, CORR ? 4 : 2048 / k
     k_mark(const Lat L, const Parts pt, const SFrame *__restrict__ fcur, const SFrame *__restrict__ fprev,
            uint8_t *__restrict__ flag, int32_t *__restrict__ owner, const T *__restrict__ f, const int P,
            const uint8_t cur, const int full, unsigned long long *__restrict__ ctr) {
+    step_wait();  // first: the refill reads the frames before its own wait
+    step_next();
     if (blockIdx.x == 0 && threadIdx.x < 2) ctr[threadIdx.x] = 0ull;  // links and refilled nodes of this step
     if (CORR) mark_corr_body<T>(L, pt, fcur, flag, owner, f, P, cur);
     else mark_body(L, pt, fcur, fprev, flag, owner, cur, full);
@@ -321,20 +323,21 @@ __device__ __forceinline__ void refill_body(const Lat &L, const SFrame *__restri
                                             uint8_t *__restrict__ flag, const int32_t *__restrict__ owner,
                                             const int P, unsigned long long *__restrict__ ctr,
                                             int *__restrict__ status, const Parts &pt, const uint8_t cur) {
-    __shared__ int list[kRefillCap];
-    __shared__ int count;
+    __shared__ int list[kRefillCap], cand[CORR ? 1 : kRefillCap];
+    __shared__ int count, ncand;
     const int p = blockIdx.x;
     const SFrame Fp = fprev[p];  // the node geometry of the previous step was built from this centre
     const SFrame F = fcur[p];    // current centre, velocity and spin
     const int e = ext_of(Fp.R);
     const int bx = Fp.b[0], by = Fp.b[1], bz = Fp.b[2];
-    if (threadIdx.x == 0) count = 0;
+    if (threadIdx.x == 0) count = ncand = 0;
     __syncthreads();
     auto take = [&](int n) {
         const int k = atomicAdd(&count, 1);
         if (k < kRefillCap) list[k] = n;
         else atomicOr(status, ST_TILE);
     };
+    if (CORR) step_wait();
     if (CORR && pt.corr) {
         const uint8_t prev_mark = (uint8_t)(4 - cur);  // the other mark value: the previous step's geometry
         // the box is scanned kScanBatch offsets per thread at a time, their
@@ -372,7 +375,19 @@ __device__ __forceinline__ void refill_body(const Lat &L, const SFrame *__restri
             const int ox = w.ox + lo, oy = w.oy + lo, oz = w.oz + lo, z = bz + oz;
             if (!inside(Fp, ox, oy, oz) || inside(F, ox + d.x, oy + d.y, oz + d.z) || z < 0 || z >= L.nz) continue;
             const int n = wrapi(bx + ox, L.nx) + L.nx * (wrapi(by + oy, L.ny) + L.ny * z);
-            if ((flag[n] & 1) && owner[n] == p) take(n);
+            if constexpr (CORR) {
+                if ((flag[n] & 1) && owner[n] == p) take(n);
+            } else {
+                const int k = atomicAdd(&ncand, 1);
+                if (k < kRefillCap) cand[k] = n;
+                else atomicOr(status, ST_TILE);
+            }
+        }
+        if constexpr (!CORR) {  // which nodes follows from the frames, beside the marks; the rest after them
+            step_wait();
+            __syncthreads();
+            for (int k = threadIdx.x; k < min(ncand, kRefillCap); k += blockDim.x)
+                if ((flag[cand[k]] & 1) && owner[cand[k]] == p) take(cand[k]);
         }
     }
     __syncthreads();
@@ -480,6 +495,7 @@ __global__ void __launch_bounds__(CORR ? 256 : kGeomThreads, CORR ? 4 : 1280 / k
                                                 uint8_t *__restrict__ flag, const int32_t *__restrict__ owner,
                                                 const int P, unsigned long long *__restrict__ ctr,
                                                 int *__restrict__ status, const Parts pt, const uint8_t cur) {
+    step_next();
     refill_body<T, CORR>(L, fcur, fprev, f, flag, owner, P, ctr, status, pt, cur);
 }
 
@@ -615,54 +631,50 @@ int launch_near_mark(lbm_s *h, uint8_t *near, uint8_t tag, const SFrame *frames,
     return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
 }
 
-template <bool CORR>
-int mark_launch(lbm_s *h, int P, int full) {
+template <typename T, bool CORR>
+static cudaError_t mark_launch(lbm_s *h, int P, int full, bool pdl) {
     const SFrame *fcur = h->pt.frame[h->steps & 1], *fprev = h->pt.frame[(h->steps + 1) & 1];
-    const uint8_t cur = mark_value((int)(h->steps & 1));
-    const dim3 g(h->pt.np);
-    const int nt = CORR ? 256 : kGeomThreads;
-    switch (h->precision) {
-        case LBM_FP32:
-            k_mark<float, CORR><<<g, nt, 0, h->stream>>>(h->L, h->pt, fcur, fprev, h->flag, h->owner, (const float *)h->f,
-                                                         P, cur, full, h->ctr);
-            break;
-        case LBM_BF16_DEV:
-            k_mark<__nv_bfloat16, CORR><<<g, nt, 0, h->stream>>>(h->L, h->pt, fcur, fprev, h->flag, h->owner,
-                                                                 (const __nv_bfloat16 *)h->f, P, cur, full, h->ctr);
-            break;
-        case LBM_FP16_DEV:
-            k_mark<__half, CORR><<<g, nt, 0, h->stream>>>(h->L, h->pt, fcur, fprev, h->flag, h->owner,
-                                                          (const __half *)h->f, P, cur, full, h->ctr);
-            break;
-        default: return LBM_ERR_ARG;
-    }
-    return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
-}
-
-int launch_mark(lbm_s *h, int P, bool first) {
-    return h->pt.corr && !first ? mark_launch<true>(h, P, 0) : mark_launch<false>(h, P, first);
+    return launch_step(k_mark<T, CORR>, dim3(h->pt.np), dim3(CORR ? 256 : kGeomThreads), 0, h->stream, pdl, h->L, h->pt,
+                       fcur, fprev, h->flag, h->owner, (const T *)h->f, P, mark_value((int)(h->steps & 1)), full, h->ctr);
 }
 
 template <typename T, bool CORR>
-void refill_launch(lbm_s *h, int parity) {
+static cudaError_t refill_launch(lbm_s *h, int P, bool pdl) {
     const SFrame *fcur = h->pt.frame[h->steps & 1], *fprev = h->pt.frame[(h->steps + 1) & 1];
-    k_refill<T, CORR><<<h->pt.np, CORR ? 256 : kGeomThreads, 0, h->stream>>>(h->L, fcur, fprev, (T *)h->f, h->flag, h->owner, parity,
-                                                         h->ctr, h->status, h->pt, mark_value((int)(h->steps & 1)));
+    return launch_step(k_refill<T, CORR>, dim3(h->pt.np), dim3(CORR ? 256 : kGeomThreads), 0, h->stream, pdl, h->L, fcur,
+                       fprev, (T *)h->f, h->flag, h->owner, P, h->ctr, h->status, h->pt,
+                       mark_value((int)(h->steps & 1)));
 }
 
-int launch_refill(lbm_s *h, int parity) {
+static int step_rc(cudaError_t e) {
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
+}
+
+int launch_mark(lbm_s *h, int P, bool first, bool pdl) {
+    const bool c = h->pt.corr && !first;
+    switch (h->precision) {
+        case LBM_FP32: return step_rc(c ? mark_launch<float, true>(h, P, 0, pdl) : mark_launch<float, false>(h, P, first, pdl));
+        case LBM_BF16_DEV:
+            return step_rc(c ? mark_launch<__nv_bfloat16, true>(h, P, 0, pdl)
+                             : mark_launch<__nv_bfloat16, false>(h, P, first, pdl));
+        case LBM_FP16_DEV:
+            return step_rc(c ? mark_launch<__half, true>(h, P, 0, pdl) : mark_launch<__half, false>(h, P, first, pdl));
+    }
+    return LBM_ERR_ARG;
+}
+
+int launch_refill(lbm_s *h, int P, bool pdl) {
     const bool c = h->pt.corr != 0;
     switch (h->precision) {
-        case LBM_FP32: c ? refill_launch<float, true>(h, parity) : refill_launch<float, false>(h, parity); break;
+        case LBM_FP32: return step_rc(c ? refill_launch<float, true>(h, P, pdl) : refill_launch<float, false>(h, P, pdl));
         case LBM_BF16_DEV:
-            c ? refill_launch<__nv_bfloat16, true>(h, parity) : refill_launch<__nv_bfloat16, false>(h, parity);
-            break;
+            return step_rc(c ? refill_launch<__nv_bfloat16, true>(h, P, pdl)
+                             : refill_launch<__nv_bfloat16, false>(h, P, pdl));
         case LBM_FP16_DEV:
-            c ? refill_launch<__half, true>(h, parity) : refill_launch<__half, false>(h, parity);
-            break;
-        default: return LBM_ERR_ARG;
+            return step_rc(c ? refill_launch<__half, true>(h, P, pdl) : refill_launch<__half, false>(h, P, pdl));
     }
-    return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
+    return LBM_ERR_ARG;
 }
 
 // Any member with the momentum correction selects the CORR kernels (each

@@ -247,7 +247,7 @@ struct lbm_batch_s;
 // Handle (opaque in the ABI).
 struct lbm_s {
     lbm_batch_s *batch;      // the batch this handle belongs to (steps only through it), or null
-    cudaGraphExec_t graph[2];  // one serial step from parity 0 / 1 (null: not captured)
+    cudaGraphExec_t graph[3];  // one serial step from parity 0 / 1, two from parity 0 (null: not captured)
     bool graph_stale;          // sphere count changed since the capture
     cudaStream_t side;         // branch of the step graph that builds the neighbour lists
     cudaEvent_t ev_fork, ev_nbr;
@@ -378,7 +378,35 @@ struct lbm_batch_s {
 
 // Launchers (one per translation unit).
 namespace lbm {
-int launch_stream_collide(lbm_s *h, int parity, cudaStream_t stream = nullptr);
+// The kernels of a serial step are programmatic dependents of each other in
+// its graph: each may start once every block of the one before has said so
+// (step_next) and touches what that one wrote after step_wait, which returns
+// when it has completed; as every block of every kernel waits, all earlier
+// ones have too.  What a kernel reads before its wait has to be two kernels
+// old, and the kernel between says step_next after its own wait: then all its
+// blocks have seen that older one complete (the refill reads frames behind
+// the marks, the links read marks behind the collide).  In an ordinary launch
+// both return at once.
+__device__ __forceinline__ void step_next() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void step_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Launch of k, with `pdl` as a programmatic dependent of the kernel before it on the stream.
+template <typename... P, typename... A>
+cudaError_t launch_step(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+int launch_stream_collide(lbm_s *h, int parity, bool pdl = false);
+bool collides_by_rows(const lbm_s *h);  // whether that is the row form
 // near tags of one step into `near`, the tagged groups compacted into list / *count and the
 // other groups into far / *far_count
 int launch_near_mark(lbm_s *h, uint8_t *near, uint8_t tag, const SFrame *frames, int *list, int *count, int *far,
@@ -386,16 +414,12 @@ int launch_near_mark(lbm_s *h, uint8_t *near, uint8_t tag, const SFrame *frames,
 int launch_collide_list(lbm_s *h, int parity, const int *list, const int *count, cudaStream_t stream);
 int launch_zieb(lbm_s *h, int P);  // ZIEB face after the step of parity P
 int launch_wait_probe(lbm_s *h);   // a bounded device wait that runs out (self-test)
-int launch_mark(lbm_s *h, int P, bool first = false);  // first: the marks of a new placement
-int launch_refill(lbm_s *h, int parity);
-// after_collide: launched as a programmatic dependent of the collide kernel
-// just before it on the stream (its node codes and link list, which read
-// only the marks, overlap the collide's last blocks; the populations are
-// read after the collide grid has completed).
-int launch_links(lbm_s *h, int parity, bool after_collide = false);
+int launch_mark(lbm_s *h, int P, bool first = false, bool pdl = false);  // first: the marks of a new placement
+int launch_refill(lbm_s *h, int parity, bool pdl = false);
+int launch_links(lbm_s *h, int parity, bool pdl = false);
 int launch_neighbours(lbm_s *h, int force, cudaStream_t stream = nullptr);
 int launch_contact(lbm_s *h);
-int launch_dem(lbm_s *h);
+int launch_dem(lbm_s *h, bool pdl = false);
 int launch_set_populations(lbm_s *h, const double *f_dev, int parity);
 int launch_get_populations(lbm_s *h, double *f_dev, int parity);
 int launch_fields(lbm_s *h, float *rho, float *u, int parity);

@@ -463,13 +463,11 @@ __device__ __forceinline__ void links_body(const Lat &L, const Parts &pt, const 
     LinkAcc acc;
     const int nn = link_nodes(L, Fr.b, flag, owner, p, tl, sh, tl.ncap(cap), status);
     const int total = link_enumerate(sh, tl, nn, cap, acc, status);
-    // Launched as a programmatic dependent of the collide, the CTA may start
-    // while the collide's last blocks run: the codes and the list read only
-    // the marks (a refilled node's flag turns from 2 to 0 in the collide,
-    // fluid either way), the populations only after the collide grid has
-    // completed and its writes are visible.  In an ordinary launch this
-    // wait returns at once.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // the codes and the list read only the marks (a refilled node's flag turns
+    // from 2 to 0 in the collide, fluid either way): they may be made while
+    // the collide's last blocks run, the populations are read after it
+    step_wait();
+    step_next();
     link_apply<T, GI, BATCH>(L, pt, Fr, f, P, tl, sh, dir, total, acc);
     link_reduce_store(pt, p, Fr.b, acc, total, ctr);
 }
