@@ -333,14 +333,15 @@ constexpr int kChanTx = 128;
 // Resident blocks per SM of k_chan_step and k_chan_adj.  With the cut links
 // in kernels of their own both are straight code that waits on its 19 (38)
 // loads, and fewer blocks without spills win: 128x64x64 nodes, 200 spheres,
-// 500 steps, ms per gradient with step / adj at 12 / 10 blocks 71.3, 8 / 10
-// 63.1, 6 / 10 61.1, 12 / 6 62.0, 6 / 6 51.4, 7 / 7 52.0, 5 / 5 50.2 (the
-// links tested per direction inside the node kernels: 110.8; walked per
-// node: 79 at best).  Recorded states are written and read once, dozens of
-// steps apart: streaming stores and loads keep them from evicting G and
+// 500 steps, ms per gradient with step / adj at 6 / 4 blocks 43.4, 6 / 5
+// 43.4, 6 / 6 42.6, 5 / 5 43.4, 7 / 5 44.3; before the inlet and outlet rows
+// moved into the collision's adjoint 12 / 10 took 71.3, 6 / 6 51.4, 5 / 5
+// 50.2 (the links tested per direction inside the node kernels: 110.8; walked
+// per node: 79 at best).  Recorded states are written and read once, dozens
+// of steps apart: streaming stores and loads keep them from evicting G and
 // lambda (2 x 40 MB) from L2 (51.9 -> 51.4 ms).
 #ifndef LBM_CHAN_ADJ_MINB
-#define LBM_CHAN_ADJ_MINB 5
+#define LBM_CHAN_ADJ_MINB 6
 #endif
 #ifndef LBM_CHAN_STEP_MINB
 #define LBM_CHAN_STEP_MINB 6
@@ -472,62 +473,62 @@ __global__ void __launch_bounds__(kChanTx, LBM_CHAN_STEP_MINB) k_chan_step(const
 
 // ---- reverse -----------------------------------------------------------------
 
-// Adjoint of the inlet row of P at step s for the row of fluid node n = (1, y,
-// z), given lambda^s at the row's inlet node: that node's populations are
-// read by the pulls of the five directions c_x = 1 only (li; x = 1 holds
-// interior fluid nodes only).  Adds the adjoint of rho(1, y, z) to lambda^s
-// of every population at n (lam), so that the gathers of step s - 1 find it
-// there; returns the row's part of dJ/du_peak.
-__device__ __forceinline__ double fold_inlet(const ChanGeo &G, const float u_peak, const float (&li)[Q],
-                                             const float *__restrict__ f1, const int z, const int n,
-                                             float *__restrict__ lam) {
-    // inlet: f_i(0) = rho_1 fe_i(1, u_in)
+// The adjoint of the inlet or outlet row of P at step s that ends at fluid
+// node n, given lambda^s at the row's inlet or outlet node (row): that node's
+// populations are read by the pulls of the five directions with c_x = side
+// only (x = 1 and x = nx - 2 hold interior fluid nodes only).  Both depend on
+// the populations at n through rho and j alone, so the row adds a part equal
+// in all directions (all) and one proportional to c_i (dir) to lambda^s at n,
+// where the gathers of step s - 1 find it.
+//
+// Written as additions to what the collision's adjoint had just stored, the
+// row read f^s (19 loads), then lambda^s (19 loads) again and stored it
+// twice, in the blocks that the launch waits for: a reverse step of 48x20x24
+// nodes (with its share of the recomputed forward run) took 26.9 us and takes
+// 17.6 us with the row inside the collision's adjoint, 79.9 and 66.4 us for
+// 128x64x64 nodes.
+constexpr int kRow = 5;  // directions with c_x = 1 (or -1)
+struct RowBar {
+    float all = 0.f, dir[3] = {0.f, 0.f, 0.f};
+    double gup = 0.0, ggx = 0.0;  // the row's parts of dJ/du_peak and dJ/dg_x
+};
+
+// inlet: f_i(0) = rho_1 fe_i(1, u_in)
+__device__ __forceinline__ void fold_inlet(const ChanGeo &G, const float u_peak, const float (&row)[kRow], const int z,
+                                           const float rho1, RowBar &r) {
     const float zh = (z + 0.5f) / G.nz, sh = 4.f * zh * (1.f - zh), ux = u_peak * sh;
-    float e[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) e[i] = f1[(size_t)i * G.N + n];
-    float rho1, jx, jy, jz;
-    moments(e, rho1, jx, jy, jz);
-    float rb = 0.f, ub = 0.f;
+    float ub = 0.f;
+    int k = 0;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         if (cx(i) != 1) continue;
-        const float w = (float)rw36(i) / 36.f, cu = rcx(i) * ux, l = li[i];
-        rb += l * w * (1.f + 3.f * cu + 4.5f * cu * cu - 1.5f * ux * ux);
+        const float w = (float)rw36(i) / 36.f, cu = rcx(i) * ux, l = row[k++];
+        r.all += l * w * (1.f + 3.f * cu + 4.5f * cu * cu - 1.5f * ux * ux);
         ub += l * w * (3.f * rcx(i) + 9.f * cu * rcx(i) - 3.f * ux);
     }
-#pragma unroll
-    for (int i = 0; i < Q; ++i) lam[i * G.Ng] += rb;
-    return (double)ub * rho1 * sh;
+    r.gup = (double)ub * rho1 * sh;
 }
 
-// The same for the outlet row of fluid node n = (nx - 2, y, z): the adjoint
-// of u(nx - 2, y, z), by population; returns the row's part of dJ/dg_x.
-__device__ __forceinline__ double fold_outlet(const ChanGeo &G, const Phys &ph, const float (&lo)[Q],
-                                              const float *__restrict__ f1, const int n, float *__restrict__ lam) {
-    // outlet: f_i(nx-1) = f^eq_i(1, u(nx-2)), u = j / rho + g / 2
-    float e[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) e[i] = f1[(size_t)i * G.N + n];
-    float rho2, jx, jy, jz;
-    moments(e, rho2, jx, jy, jz);
-    const float ir = 1.f / rho2;
-    const float u[3] = {jx * ir + 0.5f * ph.g[0], jy * ir + 0.5f * ph.g[1], jz * ir + 0.5f * ph.g[2]};
+// outlet: f_i(nx-1) = f^eq_i(1, u(nx-2)), u = j / rho + g / 2
+__device__ __forceinline__ void fold_outlet(const float (&row)[kRow], const float (&u)[3], const float (&j)[3],
+                                            const float ir, RowBar &r) {
     float uba[3] = {0.f, 0.f, 0.f};
+    int k = 0;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         if (cx(i) != -1) continue;
-        const float w = (float)rw36(i) / 36.f, l = lo[i];
+        const float w = (float)rw36(i) / 36.f, l = row[k++];
         const float cu = rcx(i) * u[0] + rcy(i) * u[1] + rcz(i) * u[2];
         uba[0] += l * w * (3.f * rcx(i) + 9.f * cu * rcx(i) - 3.f * u[0]);
         uba[1] += l * w * (3.f * rcy(i) + 9.f * cu * rcy(i) - 3.f * u[1]);
         uba[2] += l * w * (3.f * rcz(i) + 9.f * cu * rcz(i) - 3.f * u[2]);
     }
-    const float v[3] = {jx * ir, jy * ir, jz * ir};
 #pragma unroll
-    for (int i = 0; i < Q; ++i)
-        lam[i * G.Ng] += ir * (uba[0] * (rcx(i) - v[0]) + uba[1] * (rcy(i) - v[1]) + uba[2] * (rcz(i) - v[2]));
-    return 0.5 * (double)uba[0];
+    for (int a = 0; a < 3; ++a) {
+        r.dir[a] = ir * uba[a];
+        r.all -= r.dir[a] * (j[a] * ir);
+    }
+    r.ggx = 0.5 * (double)uba[0];
 }
 
 // Vector-Jacobian product of collide_node at deviations d: lam = C'(d)^T gb,
@@ -546,9 +547,13 @@ __device__ __forceinline__ double fold_outlet(const ChanGeo &G, const Phys &ph, 
 // only has to carry the gradient to well within its 1e-3 tolerance.  The deviations are
 // read pair by pair from f (slot stride N; null: the rest state) and the
 // result is written to lam (slot stride Ng), so that only gb is held whole.
-__device__ __forceinline__ void chan_collide_vjp(const Phys &ph, const float *__restrict__ f, const size_t N,
-                                                 const float (&gb)[Q], float *__restrict__ lam, const size_t Ng,
-                                                 float &gx_bar, float &smag_bar) {
+// side 1 (-1): n is the fluid end of the inlet (outlet) row, whose adjoint is
+// added (see RowBar).
+__device__ __forceinline__ void chan_collide_vjp(const ChanGeo &G, const Phys &ph, const float u_peak,
+                                                 const float *__restrict__ f, const float (&gb)[Q],
+                                                 float *__restrict__ lam, const int side, const float (&row)[kRow],
+                                                 const int z, float &gx_bar, float &smag_bar, RowBar &rowb) {
+    const size_t N = (size_t)G.N, Ng = G.Ng;
     // forward intermediates (the moments of d, by opposite pairs)
     const float d0 = f ? __ldcs(f) : 0.f;
     float drho = d0, j[3] = {0.f, 0.f, 0.f}, m[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // m: xx yy zz xy xz yz
@@ -630,11 +635,18 @@ __device__ __forceinline__ void chan_collide_vjp(const Phys &ph, const float *__
         ub[2] -= rho * (2.f * mb[2] * u[2] + mb[4] * u[0] + mb[5] * u[1]);
     }
     // u = j / rho + g / 2
-    const float jb[3] = {ub[0] * ir, ub[1] * ir, ub[2] * ir};
+    float jb[3] = {ub[0] * ir, ub[1] * ir, ub[2] * ir};
     ir_bar += ub[0] * j[0] + ub[1] * j[1] + ub[2] * j[2];
     gx_bar += 0.5f * ub[0];
     rho_bar -= ir_bar * ir * ir;
-    const float dtot = drho_bar + rho_bar;  // rho = 1 + drho
+    float dtot = drho_bar + rho_bar;  // rho = 1 + drho
+    if (side) {
+        if (side > 0) fold_inlet(G, u_peak, row, z, rho, rowb);
+        else fold_outlet(row, u, j, ir, rowb);
+        dtot += rowb.all;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) jb[a] += rowb.dir[a];
+    }
     const float keep = 1.f - om;
     lam[0] = keep * gb[0] + dtot;
 #pragma unroll
@@ -695,34 +707,40 @@ __global__ void __launch_bounds__(kChanTx, LBM_CHAN_ADJ_MINB) k_chan_adj(
     const bool in = c.in && (c.edge || !(c.x == 1 || c.x == G.nx - 2));
     const int n = c.n;
     float gxb = 0.f, smb = 0.f;
-    double gup = 0.0, ggx = 0.0;
+    RowBar rowb;
     const bool live = in && G.type[n] == CH_FLUID;
     const uint32_t pm = live && wd != 0.f ? G.plate[n] : 0u;
     chan_wait();
     if (live) {
-        float gb[Q];
+        float gb[Q], row[kRow] = {0.f, 0.f, 0.f, 0.f, 0.f};
         const float *l1 = lam1 + (n + G.plane);
 #pragma unroll
         for (int i = 0; i < Q; ++i) gb[i] = l1[(ptrdiff_t)(i * G.Ng) + c.off(G, i, 1)];
+        const int side = !c.edge || !fold ? 0 : (c.x == 1 ? 1 : -1);  // c_x of the pulls that read the row's end
+        if (side) {
+            int k1 = 0, k2 = 0;
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                const float *l = l1 + (ptrdiff_t)(i * G.Ng) + c.off(G, i, 1);
+                if (cx(i) == 1) {
+                    if (side > 0) row[k1] = l[-1];
+                    ++k1;
+                }
+                if (cx(i) == -1) {
+                    if (side < 0) row[k2] = l[1];
+                    ++k2;
+                }
+            }
+        }
         if (pm)
 #pragma unroll
             for (int i = 0; i < Q; ++i)
                 if ((pm >> i) & 1u) gb[i] += wd * 2.f * rcx(i);
-        float *l0 = lam0 + (n + G.plane);
-        chan_collide_vjp(ph, fs ? fs + n : nullptr, (size_t)G.N, gb, l0, G.Ng, gxb, smb);
-        if (c.edge && fold) {
-            const int side = c.x == 1 ? 1 : -1;  // c_x of the pulls that read the row's inlet or outlet node
-#pragma unroll
-            for (int i = 0; i < Q; ++i)
-                if (cx(i) == 1 && side == 1) gb[i] = l1[(ptrdiff_t)(i * G.Ng) + c.off(G, i, 1) - 1];
-                else if (cx(i) == -1 && side == -1) gb[i] = l1[(ptrdiff_t)(i * G.Ng) + c.off(G, i, 1) + 1];
-            if (side == 1) gup = fold_inlet(G, u_peak, gb, fs, c.z, n, l0);
-            else ggx = fold_outlet(G, ph, gb, fs, n, l0);
-        }
+        chan_collide_vjp(G, ph, u_peak, fs ? fs + n : nullptr, gb, lam0 + (n + G.plane), side, row, c.z, gxb, smb, rowb);
     }
     const int warp = (blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)) * (kChanTx / 32) + (threadIdx.x >> 5);
     if (c.edge) {
-        warp_part(gup, ggx + (double)gxb, (double)smb, gedge + 3 * warp);
+        warp_part(rowb.gup, rowb.ggx + (double)gxb, (double)smb, gedge + 3 * warp);
     } else {
         const FF a = ff_warp_sum(gxb), b = ff_warp_sum(smb);
         if ((threadIdx.x & 31) == 0) {
