@@ -63,7 +63,7 @@ def collide_source_sha():
     import hashlib
 
     h = hashlib.sha256()
-    for name in ("lbm_collide.cu", "lbm_collide_node.cuh", "lbm_stream.cuh"):
+    for name in ("lbm_collide.cu", "lbm_collide_node.cuh", "lbm_rows.cuh", "lbm_stream.cuh"):
         with open(os.path.join(ROOT, "paper_1703_05158_gb300", "csrc", name), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -405,7 +405,7 @@ def run_ours(args, rank, world, local_rank):
                    "zieb": zieb_params(args).get("zieb"), "mea": args.mea,
                    "parallelism": "replicas" if world > 1 else "single",
                    "l2": "inputs larger than L2 (populations %.2f GB)" % (19 * N * s / 1e9)},
-        "roofline": {"bound": "hbm", "kernel": "k_stream_collide" + (" (near + far launches)" if args.schedule == "overlap" else ""),
+        "roofline": {"bound": "hbm", "kernel": "collide" + (" (near + far launches)" if args.schedule == "overlap" else ""),
                      "achieved": achieved,
                      "peak": peak,
                      "peak_kind": "%s hbm_gbs" % peak_kind, "unit": "GB/s", "frac": achieved / peak,
@@ -421,8 +421,10 @@ def run_ours(args, rank, world, local_rank):
                 "h2d_bytes_per_step": int(hF.numel() * 8 + hT.numel() * 8),
                 "d2h_bytes_per_step": int((oF.numel() + oT.numel() + oX.numel()) * 8)},
         # per step with spheres: overlapped = far collide, near marks, near list, marks, refill,
-        # near collide, links, neighbours, DEM; serial = marks, refill, collide, links, neighbours, DEM
-        "gpu_launches": args.steps * (((9 if args.schedule == "overlap" else 6) if nsph else 1) + int(args.zieb)),
+        # near collide, links, neighbours, islands, DEM; serial = marks, refill, collide, links, neighbours,
+        # islands, DEM; beyond 4096 spheres the DEM is two launches
+        "gpu_launches": args.steps * (((10 if args.schedule == "overlap" else 7) + int(nsph > 4096) if nsph else 1)
+                                      + int(args.zieb)),
     }
     if world == 1 and not args.no_cpu_baseline and not dense:
         line["cpu_baseline"] = cpu_baseline()
@@ -571,15 +573,15 @@ def run_adjoint(args, rank, world, local_rank):
 
 def chan_launches(S, K):
     """Kernel launches of one gradient evaluation of the differentiation form:
-    the forward run (one launch for the initial collision, one per step; the
-    boundary planes ride in the same launches), then per checkpoint segment
-    the recompute (as the forward) and one adjoint launch per step, and the
-    final sum of the gradient parts."""
-    n = S + 1
+    the forward run (one launch for the initial collision, two per step: cut
+    links and step), then per checkpoint segment the recompute (as the
+    forward) and two launches per reverse step (cut links, but for the last
+    step, and adjoint), and the final sum of the gradient parts."""
+    n = 2 * S + 1
     for seg in range(S // K, -1, -1):
         s0, s1 = seg * K, min(seg * K + K - 1, S)
-        n += (s1 - s0 + 1 if s1 > s0 else 0) + (s1 - s0 + 1)
-    return n + 1
+        n += (2 * (s1 - s0) + 1 if s1 > s0 else 0) + 2 * (s1 - s0 + 1)
+    return n  # the last reverse step has no cut-link launch, the sum is one more
 
 
 def ctypes_stream(stream):

@@ -131,10 +131,12 @@ typedef struct {
     int32_t mea;               /* momentum exchange: LBM_MEA_PAPER (Eqs. 25, 26) or LBM_MEA_GALILEAN
                                   (populations carry c - u_b, Wen, Zhang & Fang 2014; not in the
                                   paper); other values: LBM_ERR_ARG */
-    int32_t dem_mode;          /* how the DEM sub-steps run: LBM_DEM_AUTO (one thread-block
-                                  cluster up to 4096 spheres, else a cooperative grid),
-                                  LBM_DEM_CLUSTER or LBM_DEM_GRID; the same arithmetic either way;
-                                  other values: LBM_ERR_ARG */
+    int32_t dem_mode;          /* how the DEM sub-steps of touching groups of more than 32 spheres
+                                  run (smaller groups and single spheres need no barrier between
+                                  thread blocks): LBM_DEM_AUTO (one thread-block cluster up to 4096
+                                  spheres, else a cooperative grid), LBM_DEM_CLUSTER or
+                                  LBM_DEM_GRID; the same arithmetic either way; other values:
+                                  LBM_ERR_ARG */
 } lbm_params;
 
 typedef struct {

@@ -37,16 +37,14 @@
 // that pull; before it, one thread per cut link (k_chan_rlinks) applies the
 // transpose of the bounce-back to lambda^{s+1} in place (see k_chan_lists),
 // so the gather is as plain.  The geometry is fixed, so both lists are made
-// once.
-// C^T is the analytic vector-Jacobian
-// product of collide_node (chan_collide_vjp).  The forward run keeps f^s
-// every K steps; the reverse sweep recomputes each K-step segment from its
-// checkpoint, keeping its f^s, and runs the segment backwards.  The planes
-// next to the inlet and outlet ride in edge blocks of the same launches,
-// which also do the inlet / outlet equilibria of a forward step and fold
-// their adjoint into lambda^s of a reverse step.  Parameter gradients are
-// summed per warp into the warp's own slots and added up once at the end of
-// the sweep.
+// once.  C^T is the analytic vector-Jacobian product of collide_node
+// (chan_collide_vjp).  The forward run keeps f^s every K steps; the reverse
+// sweep recomputes each K-step segment from its checkpoint, keeping its f^s,
+// and runs the segment backwards.  The planes next to the inlet and outlet
+// ride in edge blocks of the same launches, which also do the inlet / outlet
+// equilibria of a forward step and add their adjoint to lambda^s of a reverse
+// step.  Parameter gradients are summed per warp into the warp's own slots
+// and added up once at the end of the sweep.
 #include <cmath>
 #include <vector>
 

@@ -31,7 +31,7 @@
 // arithmetic of a sphere is the same code in each of them.
 //
 // Tangential contact law (Eqs. 2, 3; on when k_t > 0 and mu > 0, the
-// template argument FRIC of the cluster kernel): the readings of the oracle
+// template argument FRIC of the kernels): the readings of the oracle
 // (contact point at the middle of the overlap, v^r = v_a - v_b - ((R_a -
 // delta/2) Om_a + (R_b - delta/2) Om_b) x n, f_t = -k_t delta_t - gamma_t v_t
 // capped at mu max(f^n, 0) along -v_t with delta_t reset to -f_t / k_t,
@@ -1021,7 +1021,7 @@ static bool cluster_attrs(K kernel, bool fric, int cl) {
     return true;
 }
 
-// Largest cluster (16, else 8) that can run k_dem_cluster; 0 if none, or if
+// Largest cluster (16, else 8) that can run k_dem_local; 0 if none, or if
 // max_particles does not fit its registers.
 int dem_cluster_setup(int max_particles, bool small, bool fric) {
     // one simulation: the widest cluster (16 or 8 CTAs: measured equal at
