@@ -59,7 +59,7 @@ int link_capacity(double max_radius) {
 
 size_t link_smem(int ext, int cap) {
     const LinkTile tl(ext);
-    return 8 * (size_t)tl.B * tl.B + 4 * ((size_t)cap + tl.ncap(cap));
+    return 8 * (size_t)tl.B * tl.B + 4 * (size_t)cap + 2 * (size_t)tl.ncap(cap);
 }
 
 // Raise (never lower: other handles may need more) a kernel's dynamic

@@ -46,9 +46,26 @@ __device__ __forceinline__ int wrap1(int x, int n) { return x < 0 ? x + n : (x >
 // The cube of a sphere with e = ceil(R): B nodes per edge at offsets lo ..
 // lo + B - 1 from floor(X).  Its solid nodes have offsets -e + 1 .. e, the
 // links' fluid nodes x = s - c_j and x - c_j lie within two more.
+// A node index t = x + B (y + B z) is split by multiplying with mB = 2^32 / B
+// + 1 and mB2 = 2^32 / B^2 + 1 and taking the high word: exact for t < B^3 <
+// 2^16 (B <= 36), where a division by a run-time B costs some twenty
+// instructions.
 struct LinkTile {
     int lo, B;
-    __host__ __device__ __forceinline__ explicit LinkTile(int e) : lo(-e - 1), B(2 * e + 4) {}
+    unsigned mB, mB2;
+    __host__ __device__ __forceinline__ explicit LinkTile(int e, unsigned mb = 0u, unsigned mb2 = 0u)
+        : lo(-e - 1), B(2 * e + 4), mB(mb), mB2(mb2) {}
+    // row r = y + B z
+    __device__ __forceinline__ void row_yz(int r, int &y, int &z) const {
+        z = (int)__umulhi((unsigned)r, mB);
+        y = r - z * B;
+    }
+    __device__ __forceinline__ void xyz(int t, int &x, int &y, int &z) const {
+        z = (int)__umulhi((unsigned)t, mB2);
+        const int r = t - z * B * B;
+        y = (int)__umulhi((unsigned)r, mB);
+        x = r - y * B;
+    }
     // at most every node of the core, and every listed node has a link
     __host__ __device__ __forceinline__ int ncap(int cap) const {
         const int c = B - 4, c3 = c * c * c;
@@ -57,14 +74,15 @@ struct LinkTile {
 };
 
 // Shared memory of a link CTA: row masks of the fluid nodes (bit i of row
-// y + B z: the node at offsets lo + (i, y, z)), the links (cap entries) and
-// the owned nodes that have links, in (z, y, x) order, packed as
-// i | y << 6 | z << 12 (| j << 18 for a link).
+// y + B z: the node at offsets lo + (i, y, z)), the links (cap entries, packed
+// as i | y << 6 | z << 12 | j << 18) and the node indexes of the owned nodes
+// that have links, in (z, y, x) order.
 struct LinkShared {
     unsigned long long *row;
-    uint32_t *list, *nodes;
+    uint32_t *list;
+    uint16_t *nodes;
     __device__ __forceinline__ LinkShared(unsigned char *smem, int cap, const LinkTile &tl)
-        : row((unsigned long long *)smem), list((uint32_t *)(row + tl.B * tl.B)), nodes(list + cap) {}
+        : row((unsigned long long *)smem), list((uint32_t *)(row + tl.B * tl.B)), nodes((uint16_t *)(list + cap)) {}
 };
 
 // Constants of direction j for the link loop.
@@ -103,33 +121,40 @@ __device__ __forceinline__ int link_nodes(const Lat &L, const int b[3], const ui
     const int B = tl.B, BB = B * B, core = B - 4;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int x0 = b[0] + tl.lo;
-    const bool straight = x0 >= 0 && x0 + B <= L.nx;
+    const int xs = wrap1(x0, L.nx);
     const unsigned long long full = (1ull << B) - 1ull;  // B <= 36
+    // the solid bits of len nodes from n on, from aligned words (the flags are padded to a whole word)
+    auto solid_bits = [&](const int n, const int len) {
+        unsigned long long solid = 0ull;
+        const int sh0 = n & 3;
+        const unsigned *w = (const unsigned *)(flag + (n - sh0));
+        constexpr int kW = 4;
+        for (int k0 = 0; 4 * k0 < len + sh0; k0 += kW) {
+            unsigned v[kW];
+#pragma unroll
+            for (int k = 0; k < kW; ++k) v[k] = 4 * (k0 + k) < len + sh0 ? __ldcg(w + k0 + k) : 0u;
+#pragma unroll
+            for (int k = 0; k < kW; ++k) {
+                const unsigned long long m = solid4(v[k]);
+                const int at = 4 * (k0 + k) - sh0;
+                solid |= at >= 0 ? m << at : m >> -at;
+            }
+        }
+        return solid & ((1ull << len) - 1ull);
+    };
     for (int r = threadIdx.x; r < BB; r += blockDim.x) {
-        const int z = b[2] + tl.lo + r / B;
+        int ty, tz;
+        tl.row_yz(r, ty, tz);
+        const int z = b[2] + tl.lo + tz;
         unsigned long long solid = full;
         if (z >= 0 && z < L.nz) {
-            const int n0 = L.nx * (wrap1(b[1] + tl.lo + r % B, L.ny) + L.ny * z);
+            const int n0 = L.nx * (wrap1(b[1] + tl.lo + ty, L.ny) + L.ny * z);
+            int n = n0 + xs, len = min(B, L.nx - xs);
             solid = 0ull;
-            if (straight) {  // aligned words (the flags are padded to a whole word)
-                const int n = n0 + x0, sh0 = n & 3;
-                const unsigned *w = (const unsigned *)(flag + (n - sh0));
-                constexpr int kW = 4;
-                for (int k0 = 0; 4 * k0 < B + sh0; k0 += kW) {
-                    unsigned v[kW];
-#pragma unroll
-                    for (int k = 0; k < kW; ++k) v[k] = 4 * (k0 + k) < B + sh0 ? __ldcg(w + k0 + k) : 0u;
-#pragma unroll
-                    for (int k = 0; k < kW; ++k) {
-                        const unsigned long long m = solid4(v[k]);
-                        const int at = 4 * (k0 + k) - sh0;
-                        solid |= at >= 0 ? m << at : m >> -at;
-                    }
-                }
-                solid &= full;
-            } else {
-                for (int i = 0; i < B; ++i)
-                    if (__ldcg(flag + n0 + wrap1(x0 + i, L.nx)) & 1) solid |= 1ull << i;
+#pragma unroll 1
+            for (int at = 0; at < B; n = n0, len = B - at) {  // past a periodic face, the rest from the row's start
+                solid |= solid_bits(n, len) << at;
+                at += len;
             }
         }
         sh.row[r] = ~solid & full;
@@ -137,7 +162,9 @@ __device__ __forceinline__ int link_nodes(const Lat &L, const int b[3], const ui
     __syncthreads();
     int total = 0;
     for (int r0 = 0; r0 < BB; r0 += blockDim.x) {
-        const int r = r0 + threadIdx.x, y = r % B, z = r / B;
+        const int r = r0 + threadIdx.x;
+        int y, z;
+        tl.row_yz(r, y, z);
         unsigned long long s = 0ull;
         if (r < BB && y >= 2 && y < B - 2 && z >= 2 && z < B - 2) {
             const unsigned long long *f = sh.row + r;
@@ -178,11 +205,10 @@ __device__ __forceinline__ int link_nodes(const Lat &L, const int b[3], const ui
             if (w < wid) pos += wsum[w];
             round += wsum[w];
         }
-        const uint32_t yz = (uint32_t)(y << 6 | z << 12);
         while (s) {
             const int i = __ffsll((long long)s) - 1;
             s &= s - 1ull;
-            if (pos < ncap) sh.nodes[pos] = yz | (uint32_t)i;
+            if (pos < ncap) sh.nodes[pos] = (uint16_t)(i + B * r);
             ++pos;
         }
         total += round;
@@ -223,8 +249,9 @@ __device__ __forceinline__ int link_enumerate(const LinkShared &sh, const LinkTi
         const int k = k0 + threadIdx.x;
         uint32_t mask = 0u, t = 0u;
         if (k < nn) {
-            t = sh.nodes[k];
-            const int i = t & 63, y = (t >> 6) & 63, z = t >> 12;
+            int i, y, z;
+            tl.xyz(sh.nodes[k], i, y, z);
+            t = (uint32_t)(i | y << 6 | z << 12);
             const unsigned long long *f = sh.row + y + B * z;
             uint32_t win[3][3];  // bits 0, 1, 2: the nodes at x - 1, x, x + 1 of row (y + dy, z + dz)
 #pragma unroll
@@ -457,7 +484,9 @@ __device__ __forceinline__ void links_body(const Lat &L, const Parts &pt, const 
     // small sphere among large ones scans only its own.  Nodes are listed in
     // (z, y, x) order whatever the extent, so the link list, and every sum
     // over it, is the same for any extent that holds the sphere.
-    const LinkTile tl(min(ext, (int)ceilf(Fr.R)));
+    const int e = min(ext, (int)ceilf(Fr.R));
+    const unsigned B = 2u * (unsigned)e + 4u;
+    const LinkTile tl(e, 0xFFFFFFFFu / B + 1u, 0xFFFFFFFFu / (B * B) + 1u);
     const LinkShared sh(smem, cap, tl);
     link_dirs(L, tl, dir);
     LinkAcc acc;
