@@ -357,12 +357,15 @@ __device__ __forceinline__ void chan_wait() {
 // The node of a thread of the per-node kernels.  Blocks of the first
 // gridDim.z - nz slabs (`edge`, dispatched first) take the nodes next to the
 // inlet (x = 1) and to the outlet (x = nx - 2), one thread per (side, y, z);
-// the others one node each of the lattice.
+// the others one node each of the lattice, from the top plane down where down
+// is set: steps alternate, so that one begins with the planes the step before
+// ended with, which are still in L2 (a gradient of 500 steps at 128x64x64, whose
+// states of 40 MB do not all fit, 42.6 -> 41.7 ms; 48x20x24 the same).
 struct ChanNode {
     int x, y, z, n;
     int ym, yp;  // element offsets of y - 1 and y + 1 (periodic)
     bool edge, in;
-    __device__ __forceinline__ explicit ChanNode(const ChanGeo &G) {
+    __device__ __forceinline__ ChanNode(const ChanGeo &G, const int down) {
         const int ex = (int)gridDim.z - G.nz;
         edge = (int)blockIdx.z < ex;
         if (edge) {
@@ -377,6 +380,7 @@ struct ChanNode {
             x = blockIdx.x * kChanTx + threadIdx.x;
             y = blockIdx.y;
             z = (int)blockIdx.z - ex;
+            if (down) z = G.nz - 1 - z;
             in = x < G.nx;
         }
         n = x + G.nx * (y + G.ny * z);
@@ -416,8 +420,8 @@ template <bool PULL>
 __global__ void __launch_bounds__(kChanTx, LBM_CHAN_STEP_MINB) k_chan_step(const ChanGeo G, const Phys ph, const float u_peak,
                                                        const float *__restrict__ Gin, const float *__restrict__ fin,
                                                        float *__restrict__ frec, float *__restrict__ Gout,
-                                                       double *__restrict__ drag, int *__restrict__ status) {
-    const ChanNode c(G);
+                                                       double *__restrict__ drag, int *__restrict__ status, const int down) {
+    const ChanNode c(G, down);
     const int n = c.n;
     const uint8_t t = c.in ? G.type[n] : (uint8_t)CH_SOLID;
     const bool live = PULL ? t == CH_FLUID : is_fluid_type(t);
@@ -699,8 +703,8 @@ __global__ void __launch_bounds__(kLinkTx) k_chan_rlinks(const uint4 *__restrict
 // pairs (g_x, smag) of the others in gpart.
 __global__ void __launch_bounds__(kChanTx, LBM_CHAN_ADJ_MINB) k_chan_adj(
     const ChanGeo G, const Phys ph, const float u_peak, const float *__restrict__ lam1, const float *__restrict__ fs,
-    const float wd, float *__restrict__ lam0, const int fold, float4 *__restrict__ gpart, double *__restrict__ gedge) {
-    const ChanNode c(G);
+    const float wd, float *__restrict__ lam0, const int fold, float4 *__restrict__ gpart, double *__restrict__ gedge, const int down) {
+    const ChanNode c(G, down);
     // the planes x = 1 and x = nx - 2 belong to the edge blocks
     const bool in = c.in && (c.edge || !(c.x == 1 || c.x == G.nx - 2));
     const int n = c.n;
@@ -910,13 +914,13 @@ int chan_run(lbm_channel_s *c, const float *fin, int s0, int s1, Rec rec, bool w
     const dim3 grid = chan_grid(c->p, 0), grid_edge = chan_grid(c->p, chan_slabs(c->p));
     const float up = (float)c->theta[0];
     int rc = chan_launch(c, k_chan_step<false>, grid, kChanTx, g, c->ph, up, nullptr, fin, nullptr, c->G[s0 & 1],
-                         with_drag && s0 >= 1 ? c->drag + (s0 - 1) : nullptr, c->status);
+                         with_drag && s0 >= 1 ? c->drag + (s0 - 1) : nullptr, c->status, s0 & 1);
     for (int s = s0 + 1; s <= s1 && !rc; ++s) {
         if (c->nlinks)
             rc = chan_launch(c, k_chan_flinks, dim3((c->nlinks + kLinkTx - 1) / kLinkTx), kLinkTx, c->flist, c->nlinks,
                              c->G[(s - 1) & 1]);
         if (!rc) rc = chan_launch(c, k_chan_step<true>, grid_edge, kChanTx, g, c->ph, up, c->G[(s - 1) & 1], nullptr, rec(s),
-                         c->G[s & 1], with_drag ? c->drag + (s - 1) : nullptr, c->status);
+                         c->G[s & 1], with_drag ? c->drag + (s - 1) : nullptr, c->status, s & 1);
     }
     return rc;
 }
@@ -1129,7 +1133,7 @@ int lbm_channel_backward(lbm_channel c, double *grad) {
                                  c->rlist, c->nlinks, c->special, c->nspecial, c->lam[(s + 1) & 1]);
             if (!rc)
                 rc = chan_launch(c, k_chan_adj, grid_edge, kChanTx, g, c->ph, up, c->lam[(s + 1) & 1], s == 0 ? nullptr : fs,
-                             w, c->lam[s & 1], s > 0 ? 1 : 0, c->gpart, c->gedge);
+                             w, c->lam[s & 1], s > 0 ? 1 : 0, c->gpart, c->gedge, s & 1);
         }
     }
     if (!rc) rc = chan_launch(c, k_chan_gsum, dim3(1), 256, c->gedge, nedge, c->gpart, nwarps, c->grad);
