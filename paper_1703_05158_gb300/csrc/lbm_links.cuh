@@ -166,14 +166,15 @@ __device__ __forceinline__ int link_nodes(const Lat &L, const int b[3], const ui
         int y, z;
         tl.row_yz(r, y, z);
         unsigned long long s = 0ull;
-        if (r < BB && y >= 2 && y < B - 2 && z >= 2 && z < B - 2) {
+        const int zb = b[2] + tl.lo + z;  // rows outside the box are solid, but nobody owns their nodes
+        if (r < BB && y >= 2 && y < B - 2 && z >= 2 && z < B - 2 && zb >= 0 && zb < L.nz) {
             const unsigned long long *f = sh.row + r;
             const unsigned long long lines = f[-1] | f[1] | f[-B] | f[B], mid = f[0];
             const unsigned long long any = (mid | lines) << 1 | (mid | lines) >> 1 | lines |
                                            f[-1 - B] | f[1 - B] | f[-1 + B] | f[1 + B];
             s = any & ~mid & (((1ull << core) - 1ull) << 2);  // solid, next to a fluid node, in the core
             if (s) {
-                const int n0 = L.nx * (wrap1(b[1] + tl.lo + y, L.ny) + L.ny * (b[2] + tl.lo + z));
+                const int n0 = L.nx * (wrap1(b[1] + tl.lo + y, L.ny) + L.ny * zb);
                 unsigned long long own = 0ull, c = s;
                 constexpr int kOwn = 8;
                 while (c) {
