@@ -348,7 +348,8 @@ constexpr int kChanTx = 128;
 // A kernel of a channel run is a programmatic dependent of the one before
 // it on the stream: it may start once every block of that one has started,
 // reads the static geometry of its nodes, and touches populations, adjoints
-// and sums only after chan_wait (the completion of the kernel before).
+// and sums only after chan_wait (the completion of the kernel before), through
+// pointers without __restrict__ (see step_wait).
 __device__ __forceinline__ void chan_wait() {
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -399,7 +400,7 @@ struct ChanNode {
 // else G_j(x)/(2q) + (2q-1)/(2q) G_i(x), i = opp(j).
 constexpr int kLinkTx = 128;
 __global__ void __launch_bounds__(kLinkTx) k_chan_flinks(const uint4 *__restrict__ list, const int count,
-                                                         float *__restrict__ G) {
+                                                         float *G) {
     const int t = blockIdx.x * kLinkTx + threadIdx.x;
     const uint4 r = t < count ? list[t] : make_uint4(0u, 0u, 0u, 0u);
     chan_wait();
@@ -418,9 +419,8 @@ __global__ void __launch_bounds__(kLinkTx) k_chan_flinks(const uint4 *__restrict
 // outlet (x = nx - 1) nodes; G = f there.
 template <bool PULL>
 __global__ void __launch_bounds__(kChanTx, LBM_CHAN_STEP_MINB) k_chan_step(const ChanGeo G, const Phys ph, const float u_peak,
-                                                       const float *__restrict__ Gin, const float *__restrict__ fin,
-                                                       float *__restrict__ frec, float *__restrict__ Gout,
-                                                       double *__restrict__ drag, int *__restrict__ status, const int down) {
+                                                       const float *Gin, const float *fin, float *frec, float *Gout,
+                                                       double *drag, int *status, const int down) {
     const ChanNode c(G, down);
     const int n = c.n;
     const uint8_t t = c.in ? G.type[n] : (uint8_t)CH_SOLID;
@@ -670,7 +670,7 @@ __device__ __forceinline__ void chan_collide_vjp(const ChanGeo &G, const Phys &p
 // the list's links, then its special records.
 __global__ void __launch_bounds__(kLinkTx) k_chan_rlinks(const uint4 *__restrict__ list, const int count,
                                                          const ChanSpecial *__restrict__ sp, const int nsp,
-                                                         float *__restrict__ lam) {
+                                                         float *lam) {
     const int t = blockIdx.x * kLinkTx + threadIdx.x;
     const uint4 r = t < count ? list[t] : make_uint4(0u, kNoSlot, kNoSlot, 0u);
     chan_wait();
@@ -702,8 +702,8 @@ __global__ void __launch_bounds__(kLinkTx) k_chan_rlinks(const uint4 *__restrict
 // steps (no atomics): FP64 triples of the edge warps in gedge, float-float
 // pairs (g_x, smag) of the others in gpart.
 __global__ void __launch_bounds__(kChanTx, LBM_CHAN_ADJ_MINB) k_chan_adj(
-    const ChanGeo G, const Phys ph, const float u_peak, const float *__restrict__ lam1, const float *__restrict__ fs,
-    const float wd, float *__restrict__ lam0, const int fold, float4 *__restrict__ gpart, double *__restrict__ gedge, const int down) {
+    const ChanGeo G, const Phys ph, const float u_peak, const float *lam1, const float *fs, const float wd,
+    float *lam0, const int fold, float4 *gpart, double *gedge, const int down) {
     const ChanNode c(G, down);
     // the planes x = 1 and x = nx - 2 belong to the edge blocks
     const bool in = c.in && (c.edge || !(c.x == 1 || c.x == G.nx - 2));
@@ -755,8 +755,8 @@ __global__ void __launch_bounds__(kChanTx, LBM_CHAN_ADJ_MINB) k_chan_adj(
 
 // grad[0..2] += the sums of the warps' parts: ne FP64 triples of the edge
 // warps, nb float-float pairs (g_x, smag) from warp ne on.
-__global__ void __launch_bounds__(256) k_chan_gsum(const double *__restrict__ gedge, int ne,
-                                                   const float4 *__restrict__ gpart, int nb, double *__restrict__ grad) {
+__global__ void __launch_bounds__(256) k_chan_gsum(const double *gedge, int ne, const float4 *gpart, int nb,
+                                                   double *grad) {
     chan_wait();
     double a[3] = {0.0, 0.0, 0.0};
     for (int k = threadIdx.x; k < ne; k += blockDim.x)

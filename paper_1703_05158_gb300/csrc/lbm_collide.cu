@@ -40,8 +40,8 @@ namespace lbm {
 #define LBM_SC_MINB_ODD 4
 #endif
 template <int ODD, typename T>
-__global__ void __launch_bounds__(256, ODD ? LBM_SC_MINB_ODD : LBM_SC_MINB_EVEN) k_stream_collide(const Lat L, const Phys ph, T *__restrict__ f,
-                                                        uint8_t *__restrict__ flag, int *__restrict__ status, const int down) {
+__global__ void __launch_bounds__(256, ODD ? LBM_SC_MINB_ODD : LBM_SC_MINB_EVEN) k_stream_collide(const Lat L, const Phys ph, T *f, uint8_t *flag,
+                                                        int *status, const int down) {
     // the link kernel reads the marks before its wait: it may start once every
     // block here has seen the refill (and so the marks) complete
     step_wait();
@@ -118,8 +118,7 @@ constexpr int kRowThreads = 256;  // consumers at most
 
 template <int ODD, typename T, int PITCH>
 __global__ void __launch_bounds__(kRowThreads + 32, rows_minb(PITCH))
-    k_collide_rows(const Lat L, const Phys ph, T *__restrict__ f, uint8_t *__restrict__ flag, int *__restrict__ status,
-                   const RowPlan pl, const int down) {
+    k_collide_rows(const Lat L, const Phys ph, T *f, uint8_t *flag, int *status, const RowPlan pl, const int down) {
     step_wait();  // as in k_stream_collide
     step_next();
     rows_body<ODD, T, PITCH>(
@@ -206,9 +205,8 @@ __global__ void __launch_bounds__(TPB, MINB) k_collide_batch_tab(const __grid_co
 
 // 16-bit storage: two nodes per thread (sc_pair).  Requires even nx.
 template <int ODD, typename T>
-__global__ void __launch_bounds__(128, 8) k_stream_collide2(const Lat L, const Phys ph, T *__restrict__ f,
-                                                            uint8_t *__restrict__ flag, int *__restrict__ status,
-                                                            const int down) {
+__global__ void __launch_bounds__(128, 8) k_stream_collide2(const Lat L, const Phys ph, T *f, uint8_t *flag,
+                                                            int *status, const int down) {
     step_wait();  // as in k_stream_collide
     step_next();
     const int xp = blockIdx.x * blockDim.x + threadIdx.x;

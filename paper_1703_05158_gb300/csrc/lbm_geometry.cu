@@ -137,9 +137,8 @@ __device__ __forceinline__ int mark_node(const Lat &L, const SFrame &F, const SF
 // The plain marks: flag cur and owner p on the nodes sphere p wins; without
 // contact candidates and not `full` (the first marks of a placement) only on
 // those it did not contain at the previous step's centre (fprev).
-__device__ __forceinline__ void mark_body(const Lat &L, const Parts &pt, const SFrame *__restrict__ fcur,
-                                          const SFrame *__restrict__ fprev, uint8_t *__restrict__ flag,
-                                          int32_t *__restrict__ owner, const uint8_t cur, const int full) {
+__device__ __forceinline__ void mark_body(const Lat &L, const Parts &pt, const SFrame *fcur, const SFrame *fprev,
+                                          uint8_t *flag, int32_t *owner, const uint8_t cur, const int full) {
     const int p = blockIdx.x;
     __shared__ SFrame nf[MAX_NBR_SMEM];
     __shared__ int nid[MAX_NBR_SMEM];
@@ -184,9 +183,8 @@ __device__ __forceinline__ void mark_body(const Lat &L, const Parts &pt, const S
 // node (lane i loads f_i); the CTA writes the total to Fcorr / Tcorr (zero
 // when it covers nothing).  blockDim.x = 256.
 template <typename T>
-__device__ __forceinline__ void mark_corr_body(const Lat &L, const Parts &pt, const SFrame *__restrict__ fcur,
-                                               uint8_t *__restrict__ flag, int32_t *__restrict__ owner,
-                                               const T *__restrict__ f, const int P, const uint8_t cur) {
+__device__ __forceinline__ void mark_corr_body(const Lat &L, const Parts &pt, const SFrame *fcur, uint8_t *flag,
+                                               int32_t *owner, const T *f, const int P, const uint8_t cur) {
     constexpr int kCovRound = 1024;
     const int p = blockIdx.x;
     __shared__ SFrame nf[MAX_NBR_SMEM];
@@ -289,9 +287,8 @@ constexpr int kGeomThreads = LBM_GEOM_THREADS;
 // refill.
 template <typename T, bool CORR>
 __global__ void __launch_bounds__(CORR ? 256 : kGeomThreads, CORR ? 4 : 2048 / kGeomThreads)
-    k_mark(const Lat L, const Parts pt, const SFrame *__restrict__ fcur, const SFrame *__restrict__ fprev,
-           uint8_t *__restrict__ flag, int32_t *__restrict__ owner, const T *__restrict__ f, const int P,
-           const uint8_t cur, const int full, unsigned long long *__restrict__ ctr) {
+    k_mark(const Lat L, const Parts pt, const SFrame *fcur, const SFrame *fprev, uint8_t *flag, int32_t *owner, const T *f,
+           const int P, const uint8_t cur, const int full, unsigned long long *ctr) {
     step_wait();  // first: the refill reads the frames before its own wait
     step_next();
     if (blockIdx.x == 0 && threadIdx.x < 2) ctr[threadIdx.x] = 0ull;  // links and refilled nodes of this step
@@ -319,10 +316,9 @@ constexpr int kRefillCap = 512;
 
 template <typename T, bool CORR>
 __device__ __forceinline__ void refill_body(const Lat &L, const SFrame *__restrict__ fcur,
-                                            const SFrame *__restrict__ fprev, T *__restrict__ f,
-                                            uint8_t *__restrict__ flag, const int32_t *__restrict__ owner,
-                                            const int P, unsigned long long *__restrict__ ctr,
-                                            int *__restrict__ status, const Parts &pt, const uint8_t cur) {
+                                            const SFrame *__restrict__ fprev, T *f, uint8_t *flag,
+                                            const int32_t *owner, const int P, unsigned long long *ctr, int *status,
+                                            const Parts &pt, const uint8_t cur) {
     __shared__ int list[kRefillCap], cand[CORR ? 1 : kRefillCap];
     __shared__ int count, ncand;
     const int p = blockIdx.x;
@@ -491,10 +487,9 @@ __device__ __forceinline__ void refill_body(const Lat &L, const SFrame *__restri
 
 template <typename T, bool CORR>
 __global__ void __launch_bounds__(CORR ? 256 : kGeomThreads, CORR ? 4 : 1280 / kGeomThreads) k_refill(const Lat L, const SFrame *__restrict__ fcur,
-                                                const SFrame *__restrict__ fprev, T *__restrict__ f,
-                                                uint8_t *__restrict__ flag, const int32_t *__restrict__ owner,
-                                                const int P, unsigned long long *__restrict__ ctr,
-                                                int *__restrict__ status, const Parts pt, const uint8_t cur) {
+                                                const SFrame *__restrict__ fprev, T *f, uint8_t *flag,
+                                                const int32_t *owner, const int P, unsigned long long *ctr,
+                                                int *status, const Parts pt, const uint8_t cur) {
     step_next();
     refill_body<T, CORR>(L, fcur, fprev, f, flag, owner, P, ctr, status, pt, cur);
 }

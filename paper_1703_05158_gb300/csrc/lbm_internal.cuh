@@ -385,8 +385,11 @@ namespace lbm {
 // ones have too.  What a kernel reads before its wait has to be two kernels
 // old, and the kernel between says step_next after its own wait: then all its
 // blocks have seen that older one complete (the refill reads frames behind
-// the marks, the links read marks behind the collide).  In an ordinary launch
-// both return at once.
+// the marks, the links read marks behind the collide).  A pointer that is
+// loaded from after the wait carries no __restrict__: that would state that
+// nobody else writes there while the kernel runs, which lets the compiler take
+// the read-only path or move the load ahead of the wait, and the kernel before
+// may still be writing.  In an ordinary launch both return at once.
 __device__ __forceinline__ void step_next() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void step_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -27,10 +27,9 @@ namespace lbm {
 
 template <typename T, bool GI>
 __global__ void __launch_bounds__(256, LBM_LINK_MINB) k_links(const Lat L, const Parts pt, const SFrame *__restrict__ fcur,
-                                               T *__restrict__ f,
-                                               uint8_t *__restrict__ flag, const int32_t *__restrict__ owner,
-                                               const int P, const int ext, const int cap, int *__restrict__ status,
-                                               unsigned long long *__restrict__ ctr) {
+                                               T *f, const uint8_t *__restrict__ flag,
+                                               const int32_t *__restrict__ owner, const int P, const int ext,
+                                               const int cap, int *status, unsigned long long *ctr) {
     links_body<T, GI, LBM_LINK_BATCH>(L, pt, fcur, f, flag, owner, P, ext, cap, status, ctr, pt.order[blockIdx.x]);
 }
 

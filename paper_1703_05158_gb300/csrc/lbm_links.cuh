@@ -474,10 +474,9 @@ __device__ __forceinline__ void link_reduce_store(const Parts &pt, const int p, 
 // after the step's collide and refill.
 template <typename T, bool GI, int BATCH = 6>
 __device__ __forceinline__ void links_body(const Lat &L, const Parts &pt, const SFrame *__restrict__ fcur,
-                                           T *__restrict__ f, const uint8_t *__restrict__ flag,
+                                           T *f, const uint8_t *__restrict__ flag,
                                            const int32_t *__restrict__ owner, const int P, const int ext,
-                                           const int cap, int *__restrict__ status,
-                                           unsigned long long *__restrict__ ctr, const int p) {
+                                           const int cap, int *status, unsigned long long *ctr, const int p) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ LinkDir dir[Q];
     const SFrame Fr = fcur[p];
