@@ -97,31 +97,37 @@ __global__ void __launch_bounds__(256, 4) k_collide_list2(const Lat L, const Phy
 }
 
 // Rows through shared memory (lbm_rows.cuh), three CTAs per SM of 256
-// consumers (two for buffers of 2 KB).  HBM-bound in FP32: 256^3 with 2000
-// spheres, us per launch at even / odd parity 394 / 394 (6.4 TB/s, 94% of a
-// copy) where a thread per node with global loads took 385 / 452; collide
-// phase 422 -> 396 us at 256^3, two CTAs 464, four (56 registers) 477.
+// consumers.  HBM-bound in FP32: 256^3 with 2000 spheres, us per launch at
+// even / odd parity 394 / 394 (6.4 TB/s, 94% of a copy) where a thread per
+// node with global loads took 385 / 452; collide phase 422 -> 396 us at 256^3,
+// two CTAs 464, four (56 registers) 477.
 //
-// Where: the lattice has to exceed L2 (256x256x16, 80 MB: 26.6 us per step
-// node-wise, 28.7 by rows; x 24: 45.4 and 43.6; 128^3: 57.7 both) and whole
-// rows of 112 nodes or more fill 7/8 of a buffer (128x256x256: 213 -> 208,
-// 240x200x200 260 -> 253; four rows of 64: 106.6 -> 109.0, 160 of 256
-// nodes filled: 110.5 -> 130; one row of 512 in 2 KB buffers: 112.6 -> 159).
+// Where: the lattice has to exceed L2 (FP32 256x256x16, 80 MB: 26.6 us per
+// step node-wise, 28.7 by rows; x 24: 45.4 and 43.6; 128^3: 57.7 both; FP16 /
+// BF16 512x96x80, 150 MB: 78.4 / 77.0 by the pair kernel, 80.8 / 81.4 by
+// rows) and whole rows fill 7/8 of a 1 KB buffer (FP32 128x256x256: 213 ->
+// 208, 240x200x200 260 -> 253; four rows of 64: 106.6 -> 109.0, 160 of 256
+// nodes filled: 110.5 -> 130).  Rows of more than a buffer in buffers of 2 KB,
+// two CTAs per SM, lose (one FP32 row of 512: 112.6 -> 159; FP16 without
+// spheres 640x256x128 428 -> 639, 1024x128x80 209 -> 271).
 // 16-bit storage is bound by instruction issue, and the pair kernel does the
-// conversions of two nodes from one word: at rows of 512 bytes it stays ahead
-// (297 us against 320 at four CTAs, 325 at three), at rows of 1 KB or more the
-// copies win (512x256x256 FP16: 613 against 700 us).
-constexpr long long kRowsFrom = 1ll << 21;
-constexpr int rows_minb(int pitch) { return pitch > 1024 ? 2 : 3; }
-constexpr int rows_smem(int pitch) { return 226 * 1024 / rows_minb(pitch) - 1536; }
+// conversions of two nodes from one word: two rows of 512 bytes in a buffer
+// lose to it (297 us against 320 at four CTAs, 325 at three), one row of 896
+// to 1024 bytes wins among spheres, whose solid halves the pair kernel stores
+// element by element (us per step, pair / rows: 512x256x256 with 4000 spheres
+// FP16 880 / 783, BF16 845 / 785; 448x256x256 823 / 747, 794 / 746;
+// 480x256x256 870 / 787, 837 / 786; 512x256x128 without 318 / 313, 311 / 315).
+constexpr long long kRowsFrom = 1ll << 23;  // bytes of a slot array
+constexpr int kRowCtas = 3;
+constexpr int kRowSmem = 226 * 1024 / kRowCtas - 1536;
 constexpr int kRowThreads = 256;  // consumers at most
 
-template <int ODD, typename T, int PITCH>
-__global__ void __launch_bounds__(kRowThreads + 32, rows_minb(PITCH))
+template <int ODD, typename T>
+__global__ void __launch_bounds__(kRowThreads + 32, kRowCtas)
     k_collide_rows(const Lat L, const Phys ph, T *f, uint8_t *flag, int *status, const RowPlan pl, const int down) {
     step_wait();  // as in k_stream_collide
     step_next();
-    rows_body<ODD, T, PITCH>(
+    rows_body<ODD, T>(
         [&](int u) {
             return RowUnit<T>(L, ph, f, flag, status, pl.dnx, pl.dpp, pl.per_plane, pl.rows,
                               down ? pl.units - 1 - u : u);
@@ -133,14 +139,13 @@ __global__ void __launch_bounds__(kRowThreads + 32, rows_minb(PITCH))
 // and fill a buffer (see above), else stages = 0.
 static RowPlan rows_plan(const Lat &L, size_t esize) {
     RowPlan p{};
-    const int bytes = L.nx * (int)esize, rows = std::max(1, kRowThreads / L.nx);
-    if (bytes % 16 != 0 || L.N < kRowsFrom) return p;
-    if (esize == 4 ? L.nx < 112 || rows * L.nx < 224 || L.nx > kRowThreads : bytes < 1024 || bytes > 2048) return p;
+    const int fit = kRowPitch / (int)esize, rows = std::max(1, fit / L.nx);  // nodes and rows of a buffer
+    if (L.nx * esize % 16 != 0 || L.N * (long long)esize < kRowsFrom) return p;
+    if (rows * L.nx > fit || 8 * rows * L.nx < 7 * fit || L.nx < (esize == 4 ? 112 : fit / 2 + 1)) return p;
     p.rows = std::min(rows, L.ny);
     const int U = p.rows * L.nx, passes = (U + kRowThreads - 1) / kRowThreads;
     p.consumers = ((U + passes - 1) / passes + 31) / 32 * 32;
-    p.pitch = U * (int)esize <= 1024 ? 1024 : 2048;
-    p.stages = std::min(kRowStages, rows_smem(p.pitch) / (Q * p.pitch));
+    p.stages = std::min(kRowStages, kRowSmem / (Q * kRowPitch));
     p.per_plane = (L.ny + p.rows - 1) / p.rows;
     p.units = p.per_plane * L.nz;
     p.dpp = FastDiv((unsigned)p.per_plane);
@@ -226,23 +231,15 @@ static int sweep_down(const lbm_s *h, int parity) {
     return parity && link_bytes < 120e6;
 }
 
-template <int ODD, typename T, int PITCH>
-static int launch_rows_p(lbm_s *h, const RowPlan &p, bool pdl) {
-    constexpr int kSmem = rows_smem(PITCH);
-    const auto k = k_collide_rows<ODD, T, PITCH>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess) return LBM_ERR_CUDA;
-    const int grid = std::min(p.units, h->sms * rows_minb(PITCH));
-    return launch_step(k, dim3(grid), dim3(p.consumers + 32), p.stages * Q * PITCH, h->stream, pdl, h->L, h->ph, (T *)h->f,
-                       h->flag, h->status, p, sweep_down(h, ODD)) == cudaSuccess
-               ? LBM_OK
-               : LBM_ERR_CUDA;
-}
-
 template <int ODD, typename T>
 static int launch_rows(lbm_s *h, const RowPlan &p, bool pdl) {
-    if constexpr (sizeof(T) == 2)
-        if (p.pitch == 2048) return launch_rows_p<ODD, T, 2048>(h, p, pdl);
-    return launch_rows_p<ODD, T, 1024>(h, p, pdl);
+    const auto k = k_collide_rows<ODD, T>;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmem) != cudaSuccess) return LBM_ERR_CUDA;
+    const int grid = std::min(p.units, h->sms * kRowCtas);
+    return launch_step(k, dim3(grid), dim3(p.consumers + 32), p.stages * Q * kRowPitch, h->stream, pdl, h->L, h->ph,
+                       (T *)h->f, h->flag, h->status, p, sweep_down(h, ODD)) == cudaSuccess
+               ? LBM_OK
+               : LBM_ERR_CUDA;
 }
 
 template <int ODD, typename T>

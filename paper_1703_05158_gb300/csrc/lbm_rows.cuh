@@ -58,13 +58,13 @@ __device__ __forceinline__ void bulk_store(void *dst, uint32_t src, int bytes) {
                  : "memory");
 }
 
-constexpr int kRowStages = 4;  // most stages of a CTA
+constexpr int kRowStages = 4;    // most stages of a CTA
+constexpr int kRowPitch = 1024;  // bytes of one slot buffer of a stage
 
 // Units of a lattice: `rows` consecutive rows of one plane (fewer at its
 // end), and the launch that works through them.
 struct RowPlan {
     int rows, per_plane, units, stages;
-    int pitch;      // bytes of a slot buffer
     int consumers;  // threads, a multiple of 32
     FastDiv dpp, dnx;
 };
@@ -88,14 +88,14 @@ struct RowUnit {
     }
 };
 
-// The units 0 .. units - 1 that get(u) describes (a RowUnit).  PITCH: bytes of
-// one slot buffer of a stage (a compile-time constant, so that a node's 19
-// elements are one base and immediate offsets).
-template <int ODD, typename T, int PITCH, typename Get>
+// The units 0 .. units - 1 that get(u) describes (a RowUnit).  A stage's slot
+// buffers lie a fixed pitch apart, so that a node's 19 elements are one base
+// and immediate offsets.
+template <int ODD, typename T, typename Get>
 __device__ __forceinline__ void rows_body(Get get, const int units, const int nst, const int consumers) {
     extern __shared__ __align__(128) unsigned char rows_buf[];
     __shared__ __align__(8) unsigned long long bars[2 * kRowStages];
-    constexpr int kStage = Q * PITCH, kP = PITCH / (int)sizeof(T);
+    constexpr int kStage = Q * kRowPitch, kP = kRowPitch / (int)sizeof(T);
     const uint32_t full0 = smem_addr(bars), done0 = full0 + 8 * kRowStages;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, cwarps = consumers >> 5;
     if (threadIdx.x == 0) {
@@ -108,7 +108,7 @@ __device__ __forceinline__ void rows_body(Get get, const int units, const int ns
     __syncthreads();
     const int mine = ((int)blockIdx.x < units) ? (units - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     if (warp == cwarps) {  // producer
-        const uint32_t buf = smem_addr(rows_buf) + lane * PITCH;
+        const uint32_t buf = smem_addr(rows_buf) + lane * kRowPitch;
         const int k = lane < Q ? lane : 0, oy = ODD ? rcy(k) : 0, oz = ODD ? rcz(k) : 0;
         // calls fn(global, shared, bytes) for the runs of rows of unit `it` in this lane's slot array
         auto rows = [&](int it, auto fn) {
