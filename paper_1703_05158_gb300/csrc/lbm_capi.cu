@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "lbm_internal.cuh"
+#include "lbm_route.cuh"
 
 using namespace lbm;
 
@@ -196,32 +197,45 @@ double *state_stage(lbm_s *h) {
     return h->state_host;
 }
 
+// What a caller's pointer points to.  The query takes 0.2 us.
+ArrayAt array_at(const lbm_s *h, const void *p) {
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        a.type = cudaMemoryTypeUnregistered;
+    }
+    const Mem mem = a.type == cudaMemoryTypeDevice    ? Mem::device
+                    : a.type == cudaMemoryTypeManaged ? Mem::managed
+                    : a.type == cudaMemoryTypeHost    ? Mem::pinned
+                                                      : Mem::pageable;
+    return {mem, a.device == h->device, (uintptr_t)p};
+}
+
 // F, T, X, V, Omega of the spheres to the caller's five arrays (any may be
-// null), then the stream settled.  Device arrays are written by one kernel
-// (a place that is not a whole double's needs the byte copies), host arrays
-// through pinned memory (without it, by pageable copies).
+// null), then the stream settled.  One kernel writes the device arrays (see
+// route_device) and, for host arrays, pinned memory that the host copies from;
+// the others by a copy each.
 int state_out(lbm_s *h, double *const *out, int where) {
     const size_t n3 = 3 * (size_t)h->pt.np, v3 = n3 * sizeof(double);
-    bool any = false, whole = true;
-    for (int k = 0; k < 5; ++k) {
-        any = any || out[k];
-        whole = whole && ((uintptr_t)out[k] & 7) == 0;
-    }
-    if (!any || n3 == 0) return settle(h);
+    if (n3 == 0) return settle(h);
+    const double *src[5] = {h->pt.Fh, h->pt.Th, h->pt.X, h->pt.V, h->pt.W};
+    double *to[5] = {}, *stage = where == LBM_HOST ? state_stage(h) : nullptr;
+    bool staged[5] = {}, any = false;
     int rc = LBM_OK;
-    if (where == LBM_DEVICE ? !whole : !state_stage(h)) {
-        const double *src[5] = {h->pt.Fh, h->pt.Th, h->pt.X, h->pt.V, h->pt.W};
-        for (int k = 0; k < 5 && !rc; ++k) rc = copy_out(h, out[k], src[k], v3, where);
-        const int s = settle(h);
-        return rc ? rc : s;
+    for (int k = 0; k < 5 && !rc; ++k) {
+        if (!out[k]) continue;
+        const ArrayAt at = array_at(h, out[k]);
+        switch (where == LBM_DEVICE ? route_device(at) : route_host(at, stage != nullptr)) {
+            case Route::kernel: to[k] = out[k]; break;
+            case Route::staged: to[k] = stage + n3 * k, staged[k] = true; break;
+            case Route::copy: rc = copy_out(h, out[k], src[k], v3, where); break;
+        }
+        any = any || to[k];
     }
-    double *to[5];
-    for (int k = 0; k < 5; ++k) to[k] = where == LBM_DEVICE ? out[k] : (out[k] ? h->state_host + n3 * k : nullptr);
-    rc = launch_state(h, to);
-    const int s = rc ? settle(h) : settle_posted(h);
-    if (!rc && where == LBM_HOST)
-        for (int k = 0; k < 5; ++k)
-            if (out[k]) std::memcpy(out[k], to[k], v3);
+    if (!rc && any) rc = launch_state(h, to);
+    const int s = rc || !any ? settle(h) : settle_posted(h);
+    for (int k = 0; k < 5 && !rc; ++k)
+        if (staged[k]) std::memcpy(out[k], to[k], v3);
     return rc ? rc : s;
 }
 
@@ -658,9 +672,10 @@ int lbm_set_particle_load(lbm_handle h, const double *force, const double *torqu
     }
     const double *F = stage && force ? stage : force;
     const double *T = stage && torque ? stage + 3 * (size_t)h->pt.np : torque;
-    if (v3 && ((uintptr_t)F & 7) == 0 && ((uintptr_t)T & 7) == 0) {
+    const auto direct = [&](const double *p) { return !p || stage || route_device(array_at(h, p)) == Route::kernel; };
+    if (v3 && direct(F) && direct(T)) {
         rc = launch_load(h, F, T);
-    } else if (v3) {  // device arrays that do not start at a whole double
+    } else if (v3) {  // arrays that a kernel does not read (see route_device)
         rc = F ? copy_in(h, h->pt.Fx, F, v3, where)
                : (cudaMemsetAsync(h->pt.Fx, 0, v3, h->stream) == cudaSuccess ? LBM_OK : LBM_ERR_CUDA);
         if (!rc)
