@@ -185,19 +185,15 @@ int copy_out(lbm_s *h, void *dst, const void *src, size_t n, int where) {
     return cudaMemcpyAsync(dst, src, n, k, h->stream) == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
 }
 
-// Pinned memory for the loads and state of all spheres: made with the handle
-// up to this many spheres, with the first host read beyond it.
-constexpr int kStateHostNow = 1 << 15;
-double *state_stage(lbm_s *h) {
-    if (!h->state_host &&
-        cudaMallocHost((void **)&h->state_host, 15 * sizeof(double) * (size_t)h->p.max_particles) != cudaSuccess) {
-        cudaGetLastError();
-        h->state_host = nullptr;
-    }
-    return h->state_host;
-}
+// Spheres whose loads and state go to pageable host arrays through the
+// handle's pinned memory, which is made with the handle.  A read of all five
+// arrays takes 15 us and 2 ns per sphere and array that way (the kernel's
+// write and the host's copy), a copy of its own 11 us per array and next to
+// nothing per sphere: us by kernel / by copies at 31 spheres 20 / 58, 4000
+// 46 / 63, 6000 60 / 61, 33000 274 / 80.
+constexpr int kStateStage = 4096;
 
-// What a caller's pointer points to.  The query takes 0.2 us.
+// What a caller's pointer points to.  The query takes 0.15 us.
 ArrayAt array_at(const lbm_s *h, const void *p) {
     cudaPointerAttributes a{};
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -208,25 +204,25 @@ ArrayAt array_at(const lbm_s *h, const void *p) {
                     : a.type == cudaMemoryTypeManaged ? Mem::managed
                     : a.type == cudaMemoryTypeHost    ? Mem::pinned
                                                       : Mem::pageable;
-    return {mem, a.device == h->device, (uintptr_t)p};
+    return {mem, a.device == h->device, (uintptr_t)(mem == Mem::pinned ? a.devicePointer : p)};
 }
 
 // F, T, X, V, Omega of the spheres to the caller's five arrays (any may be
-// null), then the stream settled.  One kernel writes the device arrays (see
-// route_device) and, for host arrays, pinned memory that the host copies from;
-// the others by a copy each.
+// null), then the stream settled.  One kernel writes device and pinned arrays
+// in place (see route_device, route_host) and, for a few spheres, pinned memory
+// that the host copies from; the others are a copy each.
 int state_out(lbm_s *h, double *const *out, int where) {
     const size_t n3 = 3 * (size_t)h->pt.np, v3 = n3 * sizeof(double);
     if (n3 == 0) return settle(h);
     const double *src[5] = {h->pt.Fh, h->pt.Th, h->pt.X, h->pt.V, h->pt.W};
-    double *to[5] = {}, *stage = where == LBM_HOST ? state_stage(h) : nullptr;
+    double *to[5] = {}, *stage = h->pt.np <= kStateStage ? h->state_host : nullptr;
     bool staged[5] = {}, any = false;
     int rc = LBM_OK;
     for (int k = 0; k < 5 && !rc; ++k) {
         if (!out[k]) continue;
         const ArrayAt at = array_at(h, out[k]);
         switch (where == LBM_DEVICE ? route_device(at) : route_host(at, stage != nullptr)) {
-            case Route::kernel: to[k] = out[k]; break;
+            case Route::kernel: to[k] = (double *)at.at; break;
             case Route::staged: to[k] = stage + n3 * k, staged[k] = true; break;
             case Route::copy: rc = copy_out(h, out[k], src[k], v3, where); break;
         }
@@ -461,7 +457,11 @@ int lbm_create(const lbm_params *prm, lbm_handle *out) {
         cudaGetLastError();
         rc = LBM_ERR_NOMEM;
     }
-    if (!rc && M > 0 && M <= kStateHostNow) state_stage(h);
+    if (!rc && M > 0 &&
+        cudaMallocHost((void **)&h->state_host, 15 * sizeof(double) * (size_t)std::min(M, kStateStage)) != cudaSuccess) {
+        cudaGetLastError();
+        h->state_host = nullptr;  // reads then take a copy per array
+    }
     if (!rc && M > 0 && links_setup(h->tile_ext, h->link_cap) != LBM_OK) rc = LBM_ERR_CUDA;
     // overlapped schedule (spheres only): near tags, second stream, events
     h->overlap = M > 0 && p.schedule == LBM_SCHEDULE_OVERLAP;

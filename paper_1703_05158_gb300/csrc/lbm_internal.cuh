@@ -266,7 +266,7 @@ struct lbm_s {
     int32_t *owner;
     int *status;             // device status word
     int *status_host;        // pinned mirror
-    double *state_host;      // pinned [5][max_particles][3]: loads and state on their way to the caller
+    double *state_host;      // pinned: loads and state of a few spheres on their way to the caller (or null)
     unsigned *bar;           // DEM grid-barrier counter
     unsigned long long *ctr; // [0] links, [1] refilled, [2] fluid-count scratch
     int parity;              // parity of the next step

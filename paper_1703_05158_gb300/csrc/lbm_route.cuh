@@ -8,8 +8,9 @@ namespace lbm {
 
 enum class Mem { pageable, pinned, device, managed };
 
-// An array of a call: what kind of memory it lies in, and whether that is of
-// the handle's device (pinned memory: allocated beside it).
+// An array of a call: what kind of memory it lies in, whether that is of the
+// handle's device (pinned memory: allocated beside it), and its address for
+// kernels.
 struct ArrayAt {
     Mem mem;
     bool here;
@@ -27,9 +28,11 @@ inline Route route_device(const ArrayAt &a) {
     return a.mem == Mem::device && a.here && a.at % 8 == 0 ? Route::kernel : Route::copy;
 }
 
-// Outputs of a call that says host memory: device memory among them cannot be
-// filled by the host.
+// Outputs of a call that says host memory, `have_stage`: its values fit the
+// handle's pinned memory.  Pinned arrays are written in place; device memory
+// among them cannot be filled by the host.
 inline Route route_host(const ArrayAt &a, bool have_stage) {
+    if (a.mem == Mem::pinned && a.here && a.at && a.at % 8 == 0) return Route::kernel;
     return a.mem != Mem::device && have_stage ? Route::staged : Route::copy;
 }
 

@@ -1,8 +1,10 @@
 """Which arrays of a call a kernel may touch: memory of the handle's own device
-that starts at a whole double, and nothing else (no other device's memory, no
-host memory in a call that says device memory); nor does the host write to
-device memory in a call that says host memory.  The rule is compiled by itself,
-so that it is tried for every kind of memory without a GPU."""
+that starts at a whole double, pinned arrays of a call that says host memory,
+and nothing else (no other device's memory, no host memory in a call that says
+device memory); nor does the host write to device memory in a call that says
+host memory.  The rule is compiled by itself, so that it is tried for every
+kind of memory without a GPU.  Many spheres are read by copies, a few through
+pinned memory: the values are the same."""
 import ctypes
 import itertools
 import os
@@ -36,9 +38,11 @@ def test_device_calls(rule):
 
 
 def test_host_calls(rule):
-    for mem, here, stage in itertools.product(range(4), (0, 1), (0, 1)):
+    for mem, here, stage, at in itertools.product(range(4), (0, 1), (0, 1), (0, 4096, 4100, 4104)):
         want = COPY if mem == DEVICE or not stage else STAGED
-        assert rule.host(mem, here, ctypes.c_ulong(4096), stage) == want, (mem, here, stage)
+        if mem == PINNED and here and at in (4096, 4104):
+            want = KERNEL
+        assert rule.host(mem, here, ctypes.c_ulong(at), stage) == want, (mem, here, stage, at)
 
 
 @pytest.mark.gpu
@@ -73,3 +77,31 @@ def test_a_device_load_in_a_capture():
         lat.close()
     for a, b in zip(*runs):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [1, 4096, 4097, 9000])
+def test_host_arrays_of_every_kind(n):
+    torch = pytest.importorskip("torch")
+    from paper_1703_05158_gb300 import lbm
+
+    X = np.array([(3.0 + 5 * (a % 32), 3.0 + 5 * (a // 32 % 32), 3.0 + 5 * (a // 1024)) for a in range(n)])
+    lat = lbm.Lattice(160, 160, 48, tau0=0.7, max_particles=n + 3, max_radius=2.0)
+    lat.set_particles(X, V=np.full((n, 3), 0.01), R=np.full(n, 1.8))
+    lat.set_load(F=1e-3 * X, T=2e-3 * X)
+    lat.step(3)
+    dev = [torch.empty((n, 3), dtype=torch.float64, device="cuda") for _ in range(5)]
+    lbm.lbm_particle_state(lat.h, *dev)
+    want = [d.cpu().numpy() for d in dev]
+    assert all(np.abs(w).max() > 0 for w in want)
+    pageable = [np.empty((n, 3)) for _ in range(5)]
+    pinned = [torch.empty((n, 3), dtype=torch.float64, pin_memory=True).numpy() for _ in range(5)]
+    odd = torch.empty(5 * n * 24 + 8, dtype=torch.uint8, pin_memory=True).numpy()
+    shifted = [np.frombuffer(odd[4 + k * n * 24:4 + (k + 1) * n * 24].data, dtype=np.float64).reshape(n, 3)
+               for k in range(5)]
+    for arrays in (pageable, pinned, shifted, [pageable[0] * 0, pinned[1] * 0] + shifted[2:]):
+        at = [ctypes.c_void_p(a.ctypes.data) for a in arrays]
+        assert lbm.load().lbm_particle_state(lat.h, *at, lbm.LBM_HOST) == 0
+        for a, w in zip(arrays, want):
+            assert np.array_equal(a, w)
+    lat.close()
