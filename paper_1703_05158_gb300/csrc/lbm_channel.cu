@@ -511,9 +511,12 @@ __device__ __forceinline__ void fold_inlet(const ChanGeo &G, const float u_peak,
     r.gup = (double)ub * rho1 * sh;
 }
 
-// outlet: f_i(nx-1) = f^eq_i(1, u(nx-2)), u = j / rho + g / 2
-__device__ __forceinline__ void fold_outlet(const float (&row)[kRow], const float (&u)[3], const float (&j)[3],
-                                            const float ir, RowBar &r) {
+// outlet: f_i(nx-1) = f^eq_i(1, u(nx-2)), u = j / rho + g / 2 (1 / rho rounded,
+// not the approximate one of the collision's adjoint)
+__device__ __forceinline__ void fold_outlet(const Phys &ph, const float (&row)[kRow], const float (&j)[3],
+                                            const float rho, RowBar &r) {
+    const float ir = __fdiv_rn(1.f, rho);
+    const float u[3] = {j[0] * ir + 0.5f * ph.g[0], j[1] * ir + 0.5f * ph.g[1], j[2] * ir + 0.5f * ph.g[2]};
     float uba[3] = {0.f, 0.f, 0.f};
     int k = 0;
 #pragma unroll
@@ -644,7 +647,7 @@ __device__ __forceinline__ void chan_collide_vjp(const ChanGeo &G, const Phys &p
     float dtot = drho_bar + rho_bar;  // rho = 1 + drho
     if (side) {
         if (side > 0) fold_inlet(G, u_peak, row, z, rho, rowb);
-        else fold_outlet(row, u, j, ir, rowb);
+        else fold_outlet(ph, row, j, rho, rowb);
         dtot += rowb.all;
 #pragma unroll
         for (int a = 0; a < 3; ++a) jb[a] += rowb.dir[a];
