@@ -49,6 +49,7 @@
 #include <vector>
 
 #include "lbm_collide_node.cuh"
+#include "lbm_sum.cuh"
 
 namespace lbm {
 namespace {
@@ -275,28 +276,6 @@ __device__ __forceinline__ void moments(const float *d, float &rho, float &jx, f
         jy += rcy(i) * d[i];
         jz += rcz(i) * d[i];
     }
-}
-
-// Unevaluated FP32 sum h + l of a running total: about 46 bits where the
-// FP64 pipe (1/64 of the FP32 rate) would cost the reverse step more than
-// its arithmetic.  ff_add: two-sum (Knuth) of the high parts, the errors
-// and low parts added, renormalised.
-struct FF {
-    float h, l;
-};
-__device__ __forceinline__ FF ff_add(const FF a, const FF b) {
-    const float s = __fadd_rn(a.h, b.h), bb = __fsub_rn(s, a.h);
-    const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, bb)), __fsub_rn(b.h, bb));
-    const float l = __fadd_rn(__fadd_rn(a.l, b.l), e);
-    const float h = __fadd_rn(s, l);
-    return {h, __fsub_rn(l, __fsub_rn(h, s))};
-}
-__device__ __forceinline__ FF ff_warp_sum(float v) {
-    FF a = {v, 0.f};
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        a = ff_add(a, FF{__shfl_xor_sync(0xffffffffu, a.h, o), __shfl_xor_sync(0xffffffffu, a.l, o)});
-    return a;
 }
 
 // Warp sums of three values added to the warp's own slots dst[0..2] (the
@@ -702,11 +681,11 @@ __global__ void __launch_bounds__(kLinkTx) k_chan_rlinks(const uint4 *__restrict
 // ChanNode), which with `fold` also gather lambda^s at the row's inlet or
 // outlet node and fold its adjoint in for the next reverse step.  The parts
 // of dJ/d(u_peak, g_x, smag) of each warp are added to its own slots over the
-// steps (no atomics): FP64 triples of the edge warps in gedge, float-float
-// pairs (g_x, smag) of the others in gpart.
+// steps in FP64 (no atomics): triples of the edge warps in gedge, pairs
+// (g_x, smag) of the others in gpart.
 __global__ void __launch_bounds__(kChanTx, LBM_CHAN_ADJ_MINB) k_chan_adj(
     const ChanGeo G, const Phys ph, const float u_peak, const float *lam1, const float *fs, const float wd,
-    float *lam0, const int fold, float4 *gpart, double *gedge, const int down) {
+    float *lam0, const int fold, double *gpart, double *gedge, const int down) {
     const ChanNode c(G, down);
     // the planes x = 1 and x = nx - 2 belong to the edge blocks
     const bool in = c.in && (c.edge || !(c.x == 1 || c.x == G.nx - 2));
@@ -715,7 +694,10 @@ __global__ void __launch_bounds__(kChanTx, LBM_CHAN_ADJ_MINB) k_chan_adj(
     RowBar rowb;
     const bool live = in && G.type[n] == CH_FLUID;
     const uint32_t pm = live && wd != 0.f ? G.plate[n] : 0u;
+    const int warp = (blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)) * (kChanTx / 32) + (threadIdx.x >> 5);
+    const int part = 2 * warp + (threadIdx.x & 1);
     chan_wait();
+    const double sum0 = c.edge ? 0.0 : gpart[part];  // early: nothing hides its latency at the end
     if (live) {
         float gb[Q], row[kRow] = {0.f, 0.f, 0.f, 0.f, 0.f};
         const float *l1 = lam1 + (n + G.plane);
@@ -743,22 +725,17 @@ __global__ void __launch_bounds__(kChanTx, LBM_CHAN_ADJ_MINB) k_chan_adj(
                 if ((pm >> i) & 1u) gb[i] += wd * 2.f * rcx(i);
         chan_collide_vjp(G, ph, u_peak, fs ? fs + n : nullptr, gb, lam0 + (n + G.plane), side, row, c.z, gxb, smb, rowb);
     }
-    const int warp = (blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)) * (kChanTx / 32) + (threadIdx.x >> 5);
     if (c.edge) {
         warp_part(rowb.gup, rowb.ggx + (double)gxb, (double)smb, gedge + 3 * warp);
     } else {
-        const FF a = ff_warp_sum(gxb), b = ff_warp_sum(smb);
-        if ((threadIdx.x & 31) == 0) {
-            const float4 v = gpart[warp];
-            const FF x = ff_add(a, FF{v.x, v.y}), y = ff_add(b, FF{v.z, v.w});
-            gpart[warp] = make_float4(x.h, x.l, y.h, y.l);
-        }
+        const double s = warp_sum2(gxb, smb);
+        if ((threadIdx.x & 31) < 2) gpart[part] = sum0 + s;
     }
 }
 
 // grad[0..2] += the sums of the warps' parts: ne FP64 triples of the edge
-// warps, nb float-float pairs (g_x, smag) from warp ne on.
-__global__ void __launch_bounds__(256) k_chan_gsum(const double *gedge, int ne, const float4 *gpart, int nb,
+// warps, nb pairs (g_x, smag) from warp ne on.
+__global__ void __launch_bounds__(256) k_chan_gsum(const double *gedge, int ne, const double *gpart, int nb,
                                                    double *grad) {
     chan_wait();
     double a[3] = {0.0, 0.0, 0.0};
@@ -766,9 +743,8 @@ __global__ void __launch_bounds__(256) k_chan_gsum(const double *gedge, int ne, 
 #pragma unroll
         for (int c = 0; c < 3; ++c) a[c] += gedge[3 * k + c];
     for (int k = ne + threadIdx.x; k < ne + nb; k += blockDim.x) {
-        const float4 v = gpart[k];
-        a[1] += (double)v.x + (double)v.y;
-        a[2] += (double)v.z + (double)v.w;
+        a[1] += gpart[2 * k];
+        a[2] += gpart[2 * k + 1];
     }
     __shared__ double sh[3][8];
 #pragma unroll
@@ -798,8 +774,8 @@ struct lbm_channel_s {
     uint4 *flist = nullptr, *rlist = nullptr;  // cut links of a forward / reverse step
     ChanSpecial *special = nullptr;
     int nlinks = 0, nspecial = 0;
-    float4 *gpart = nullptr;  // per-warp parts of dJ/d(g_x, smag), of the edge warps of dJ/d(u_peak, g_x, smag)
-    double *gedge = nullptr;  // (k_chan_adj)
+    // per-warp parts of dJ/d(g_x, smag), of the edge warps of dJ/d(u_peak, g_x, smag) (k_chan_adj)
+    double *gpart = nullptr, *gedge = nullptr;
     double *X = nullptr, *R = nullptr;
     float *G[2] = {nullptr, nullptr}, *lam[2] = {nullptr, nullptr};
     float *seg = nullptr;   // K states f^s of a segment
@@ -979,7 +955,7 @@ int lbm_channel_create(const lbm_channel_params *prm, int32_t n, const double *p
     const size_t NQs = (size_t)c->N * Q, NQg = NQs + 2 * (size_t)Q * p.nx * p.ny;
     if (!rc) rc = calloc_dev(c, &c->type, (size_t)c->N);
     if (!rc) rc = calloc_dev(c, &c->plate, (size_t)c->N);
-    if (!rc) rc = calloc_dev(c, &c->gpart, (size_t)chan_warps(p, chan_slabs(p) + p.nz));
+    if (!rc) rc = calloc_dev(c, &c->gpart, 2 * (size_t)chan_warps(p, chan_slabs(p) + p.nz));
     if (!rc) rc = calloc_dev(c, &c->gedge, 3 * (size_t)chan_warps(p, chan_slabs(p)));
     if (!rc) rc = calloc_dev(c, &c->X, 3 * (size_t)n);
     if (!rc) rc = calloc_dev(c, &c->R, (size_t)n);
@@ -1115,7 +1091,7 @@ int lbm_channel_backward(lbm_channel c, double *grad) {
     const float up = (float)c->theta[0];
     const float wd = (float)(1.0 / (S - c->p.avg_from + 1));
     int rc = cudaMemsetAsync(c->grad, 0, 3 * sizeof(double), c->stream) == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
-    if (!rc && (cudaMemsetAsync(c->gpart, 0, sizeof(float4) * (size_t)(nedge + nwarps), c->stream) != cudaSuccess ||
+    if (!rc && (cudaMemsetAsync(c->gpart, 0, 2 * sizeof(double) * (size_t)(nedge + nwarps), c->stream) != cudaSuccess ||
                 cudaMemsetAsync(c->gedge, 0, 3 * sizeof(double) * (size_t)nedge, c->stream) != cudaSuccess))
         rc = LBM_ERR_CUDA;
     // lambda^{S+1} = 0, with no inlet / outlet adjoint
