@@ -17,7 +17,10 @@
 // warp works through the units u = blockIdx.x, + gridDim.x, ...: lane k of
 // the producer owns buffer k of every stage, issues its loads, and when the
 // consumers have finished a stage its stores; a stage is loaded again when
-// its stores have read it.  Every wait is bounded.
+// its stores have read it.  Every wait is bounded; a producer that gives one up
+// waits (bounded again) for the loads it has in flight before it leaves the
+// shared memory they write to (a lane that gives up leaves the kernel, so no
+// __syncwarp of the others waits for it for longer).
 #pragma once
 
 #include "lbm_collide_node.cuh"
@@ -88,6 +91,14 @@ struct RowUnit {
     }
 };
 
+// A producer lane that gave up a wait at unit `it`: the status, and a wait for
+// the loads of the units up to `loaded`.  Out of line: inlined, it cost the
+// FP16 form half a percent.
+static __device__ __noinline__ void rows_give_up(int *status, uint32_t full0, int it, int loaded, int nst, int lane) {
+    if (lane == 0) atomicOr(status, ST_TIMEOUT);
+    for (; it < loaded; ++it) mbar_wait(full0 + 8 * (it % nst), (it / nst) & 1);
+}
+
 // The units 0 .. units - 1 that get(u) describes (a RowUnit).  A stage's slot
 // buffers lie a fixed pitch apart, so that a node's 19 elements are one base
 // and immediate offsets.
@@ -137,8 +148,9 @@ __device__ __forceinline__ void rows_body(Get get, const int units, const int ns
             if (lane < Q) rows(it, [&](T *g, uint32_t s, int bytes) { bulk_load(s, g, bytes, bar); });
         };
         bool ok = true;
-        for (int it = 0; it < nst && it < mine; ++it) load(it);
-        for (int it = 0; it < mine; ++it) {
+        int loaded = min(nst, mine), it = 0;  // units whose loads have been issued; the unit at work
+        for (int i = 0; i < loaded; ++i) load(i);
+        for (; it < mine; ++it) {
             ok = mbar_wait(done0 + 8 * (it % nst), (it / nst) & 1);
             if (!ok) break;
             if (lane < Q) rows(it, [&](T *g, uint32_t s, int bytes) { bulk_store(g, s, bytes); });
@@ -148,9 +160,10 @@ __device__ __forceinline__ void rows_body(Get get, const int units, const int ns
                 asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
                 __syncwarp();
                 load(it - 1 + nst);
+                loaded = it + nst;
             }
         }
-        if (!ok && lane == 0) atomicOr(get(blockIdx.x).status, ST_TIMEOUT);
+        if (!ok) rows_give_up(get(blockIdx.x).status, full0, it, loaded, nst, lane);
         asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     } else {
         for (int it = 0; it < mine; ++it) {

@@ -13,7 +13,9 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 # channel's link lists)
 COMPLETE = {"k_refill": {"fcur", "fprev"}, "refill_body": {"fcur", "fprev"},
             "k_links": {"fcur", "flag", "owner"}, "links_body": {"fcur", "flag", "owner"},
-            "k_chan_flinks": {"list"}, "k_chan_rlinks": {"list", "sp"}}
+            "k_chan_flinks": {"list"}, "k_chan_rlinks": {"list", "sp"},
+            # not loaded from at all: read by bulk copies in assembly, or only added to
+            "k_collide_rows": {"f", "status"}}
 BODIES = {"mark_body", "mark_corr_body", "refill_body", "links_body", "rows_body"}
 
 
