@@ -1250,10 +1250,10 @@ int lbm_batch_create(const lbm_params *params, int32_t count, lbm_batch *out) {
         if (params[i].device != params[0].device || params[i].precision != params[0].precision ||
             params[i].cuda_stream != params[0].cuda_stream)
             return LBM_ERR_ARG;
-    // Each link CTA scans its own sphere's tile (extent ceil(R) + 2, within
-    // that of its member's max_radius), which the member's own box rule in
-    // lbm_create keeps from wrapping onto itself; only the link kernel's
-    // shared memory is sized for the batch's largest tile.
+    // Each link CTA scans its own sphere's cube (2 ceil(R) + 4 nodes per edge,
+    // see LinkTile), which the member's own box rule in lbm_create keeps from
+    // wrapping onto itself; only the link kernel's shared memory is sized for
+    // the batch's largest sphere.
     lbm_batch_s *b = new (std::nothrow) lbm_batch_s();
     if (!b) return LBM_ERR_NOMEM;
     b->device = params[0].device;

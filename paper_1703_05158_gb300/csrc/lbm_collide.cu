@@ -225,9 +225,12 @@ __global__ void __launch_bounds__(128, 8) k_stream_collide2(const Lat L, const P
 // down: the planes the step before ended with are still in L2.  Us per step
 // one way / alternating: 201x150x101 91.8 / 81.1, 160^3 110.5 / 101.2, 256^3
 // 404 / 401, 256^3 BF16 312 / 308; lattices that fit L2 the same.  The link
-// kernel in between takes L2 for its own scattered blocks (158 bytes per
-// link): 160^3 with 400 spheres 158.7 / 155.7, 256^3 with 2000 533.6 / 534.8,
-// so the sweep alternates while that is less than L2.
+// kernel in between takes L2 for its own scattered blocks: 160^3 with 400
+// spheres of radius 4 158.7 / 155.7, 256^3 with 2000 533.6 / 534.8.  The line
+// between the two, 760,000 links of spheres of the handle's largest radius
+// (120 MB at the 158 bytes per link measured in FP32), is a measured one for
+// this GPU's 129 MB of L2; smaller spheres than the handle allows, and 16-bit
+// storage, reach it early and keep the one-way sweep.
 static int sweep_down(const lbm_s *h, int parity) {
     const double r = h->p.max_radius, link_bytes = h->pt.np * 72.0 * r * r * 158.0;
     return parity && link_bytes < 120e6;

@@ -81,25 +81,18 @@ struct Store;
 template <>
 struct Store<float> {
     static __device__ __forceinline__ float ld(const float *p) { return *p; }
-    static __device__ __forceinline__ float ldcg(const float *p) { return __ldcg(p); }  // through L2 only
     static __device__ __forceinline__ void st(float *p, float v) { *p = v; }
     static __device__ __forceinline__ float rt(float v) { return v; }  // v as stored and read back
 };
 template <>
 struct Store<__nv_bfloat16> {
     static __device__ __forceinline__ float ld(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
-    static __device__ __forceinline__ float ldcg(const __nv_bfloat16 *p) {
-        return __uint_as_float((unsigned)__ldcg((const unsigned short *)p) << 16);
-    }
     static __device__ __forceinline__ void st(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
     static __device__ __forceinline__ float rt(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
 };
 template <>
 struct Store<__half> {
     static __device__ __forceinline__ float ld(const __half *p) { return __half2float(*p); }
-    static __device__ __forceinline__ float ldcg(const __half *p) {
-        return __half2float(__ushort_as_half(__ldcg((const unsigned short *)p)));
-    }
     static __device__ __forceinline__ void st(__half *p, float v) { *p = __float2half_rn(v); }
     static __device__ __forceinline__ float rt(float v) { return __half2float(__float2half_rn(v)); }
 };

@@ -492,7 +492,7 @@ __device__ __forceinline__ void links_body(const Lat &L, const Parts &pt, const 
     LinkAcc acc;
     const int nn = link_nodes(L, Fr.b, flag, owner, p, tl, sh, tl.ncap(cap), status);
     const int total = link_enumerate(sh, tl, nn, cap, acc, status);
-    // the codes and the list read only the marks (a refilled node's flag turns
+    // the rows and the list read only the marks (a refilled node's flag turns
     // from 2 to 0 in the collide, fluid either way): they may be made while
     // the collide's last blocks run, the populations are read after it
     step_wait();
