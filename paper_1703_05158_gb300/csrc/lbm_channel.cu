@@ -465,9 +465,9 @@ __global__ void __launch_bounds__(kChanTx, LBM_CHAN_STEP_MINB) k_chan_step(const
 // Written as additions to what the collision's adjoint had just stored, the
 // row read f^s (19 loads), then lambda^s (19 loads) again and stored it
 // twice, in the blocks that the launch waits for: a reverse step of 48x20x24
-// nodes (with its share of the recomputed forward run) took 26.9 us and takes
-// 17.6 us with the row inside the collision's adjoint, 79.9 and 66.4 us for
-// 128x64x64 nodes.
+// nodes (with its share of the recomputed forward run) took 26.9 us and then,
+// with the row inside the collision's adjoint, 17.2 us, 79.9 and 64.6 us for
+// 128x64x64 nodes (17.7 and 62.2 now).
 constexpr int kRow = 5;  // directions with c_x = 1 (or -1)
 struct RowBar {
     float all = 0.f, dir[3] = {0.f, 0.f, 0.f};

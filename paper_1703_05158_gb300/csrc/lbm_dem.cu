@@ -838,8 +838,8 @@ __global__ void __launch_bounds__(256) k_neighbours(const Lat L, const Parts pt,
 // rebuild[sp], so it is cleared here; the commits may set rebuild[sp ^ 1].
 // Latency-bound: with every sphere in one cluster or grid and a barrier per
 // sub-step it took 15 us for 1 or 31 spheres and 17 us for 2000 (cluster),
-// 42 us for 8136 with friction (grid); now 9, 9, 11 and 13 us (ncu, cold),
-// the step 48.4 -> 42.1 us at 64^3 with 31 spheres and 941 -> 911 us at 256^3
+// 42 us for 8136 with friction (grid); now 10, 10, 11.5 and 13 us (ncu, cold,
+// the last with 3 us of k_dem_grid behind it), the step 48.4 -> 42.1 us at 64^3 with 31 spheres and 941 -> 911 us at 256^3
 // with 8136.
 template <bool FRIC, bool CL>
 __global__ void __launch_bounds__(kDemThreads) k_dem_local(const Lat L, const Parts pt, SFrame *fnext, const int sp,
